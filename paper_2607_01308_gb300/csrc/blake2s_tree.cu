@@ -31,24 +31,55 @@ __device__ __forceinline__ uint32_t rotr8(uint32_t x) { return __byte_perm(x, 0,
 __device__ __forceinline__ uint32_t rotr12(uint32_t x) { return __funnelshift_r(x, x, 12); }
 __device__ __forceinline__ uint32_t rotr7(uint32_t x) { return __funnelshift_r(x, x, 7); }
 
-// a + b + x on the FMA pipe. An SM sub-partition's integer ALU pipe accepts one warp
-// instruction every two cycles and must take G's four xors and four rotations; a
-// three-input add left to it (one IADD3) would make that ten instructions per G. As
-// two multiply-adds by a 1 the compiler cannot see through (a __constant__ it must
-// load, so it cannot fold the product into an add), the sum goes to the FMA pipe,
-// which the compiler already gives the two-input adds: per G, 8 ALU and 6 FMA
-// instructions instead of 10 and 2. Measured on a q4b-shaped fragment: 0.326 instead
-// of 0.397 ms per 604 MB; rotations moved to the FMA pipe as well (a multiply and a
-// high multiply by 2^25) made it slower.
-__constant__ uint32_t g_one = 1;
-__device__ __forceinline__ uint32_t add3(uint32_t a, uint32_t b, uint32_t x) {
-    return (a + b * g_one) + x * g_one;
+// Where G's operations run. An SM sub-partition issues one warp instruction per cycle; its
+// integer ALU pipe and the half of its FMA pipe that multiplies integers each accept one
+// every two cycles. G's four xors and four rotations belong to the ALU pipe (16 cycles a
+// warp), which bounds the leaf kernel; the additions are moved to the FMA pipe as
+// multiply-adds by a 1 the compiler cannot see through (a __constant__ it must load, so it
+// cannot fold the product into an add; inline, so that it keeps the shape below).
+//
+// a + b + x: x is added first. b is the last word that the previous half of G produced, so
+// this leaves one addition instead of two on G's chain of dependent operations: one warp
+// alone took 0.89 instead of 1.08 us per compression (the tree levels run few warps).
+//
+// The rotation by 16 can move as well: x * 2^16 is its upper half, and a two-way 16-bit dot
+// product with (0, 1) adds its lower half: two multiply-type instructions for one byte
+// permutation. Moving it in t of the 8 G's of a round leaves (8 - t/8) x 2 ALU cycles,
+// (6 + t/4) x 2 FMA cycles and 14 + t/8 issue cycles per G, balanced at t = 5. Measured over
+// 45 choices of the G's (2.4 GB of leaves, 1.356 ms with the earlier order of additions and
+// no rotation moved): 1.364 ms with t = 0, 1.305 with 3, 1.273 to 1.300 with 5 or 6, 1.330
+// with 8; the choice below is the fastest. ALU 92 %, FMA 89 % and issue 91 % busy.
+__constant__ uint32_t g_one = 1, g_64k = 65536, g_upper_half = 0x0100;
+__device__ __forceinline__ uint32_t mad1(uint32_t x, uint32_t y) {
+    uint32_t r;
+    asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(r) : "r"(x), "r"(g_one), "r"(y));
+    return r;
+}
+__device__ __forceinline__ uint32_t add3(uint32_t a, uint32_t b, uint32_t x) { return mad1(b, mad1(x, a)); }
+
+__device__ __forceinline__ uint32_t rotr16_fma(uint32_t x) {
+    uint32_t r;
+    asm("dp2a.lo.u32.u32 %0, %1, %2, %3;" : "=r"(r) : "r"(x), "r"(g_upper_half), "r"(x * g_64k));
+    return r;
 }
 
-// The G mixing function of RFC 7693, Section 3.1 (rotation distances 16, 12, 8, 7).
-#define CM_G(a, b, c, d, x, y)      \
+// Which G's rotate by 16 on the FMA pipe (bit g of kMask: the round's G number g): five of
+// the eight in the leaf kernel, none in kernels that run few warps (bound by the chain of
+// dependent operations, which the dot product lengthens).
+// Beside a render (kBesideRender), whose own instructions take issue slots and the FMA pipe,
+// three: the Qwen3-4B-shaped merge of 4 x 4096 tokens took 1.71 ms with 3, 1.71 with 2, 1.72
+// with none or one and 1.77 with 5; the arity merge 0.77, 0.79, 0.80 and 0.78.
+constexpr uint32_t kIssueBound = 0xD6u, kBesideRender = 0x52u, kLatencyBound = 0u;
+template <uint32_t kMask, int kG>
+__device__ __forceinline__ uint32_t rotate16(uint32_t x) {
+    return (kMask >> kG) & 1u ? rotr16_fma(x) : rotr16(x);
+}
+
+// The G mixing function of RFC 7693, Section 3.1 (rotation distances 16, 12, 8, 7); g is
+// G's place in its round.
+#define CM_G(g, a, b, c, d, x, y)   \
     a = add3(a, b, (x));            \
-    d = rotr16(d ^ a);              \
+    d = rotate16<kFmaMask, g>(d ^ a);     \
     c = c + d;                      \
     b = rotr12(b ^ c);              \
     a = add3(a, b, (y));            \
@@ -59,18 +90,19 @@ __device__ __forceinline__ uint32_t add3(uint32_t a, uint32_t b, uint32_t x) {
 // One round: four column mixes, then four diagonal mixes, message words taken in
 // the order of that round's SIGMA row (RFC 7693, Section 2.7).
 #define CM_ROUND(s0, s1, s2, s3, s4, s5, s6, s7, s8, s9, s10, s11, s12, s13, s14, s15) \
-    CM_G(v0, v4, v8, v12, m[s0], m[s1])                                                \
-    CM_G(v1, v5, v9, v13, m[s2], m[s3])                                                \
-    CM_G(v2, v6, v10, v14, m[s4], m[s5])                                               \
-    CM_G(v3, v7, v11, v15, m[s6], m[s7])                                               \
-    CM_G(v0, v5, v10, v15, m[s8], m[s9])                                               \
-    CM_G(v1, v6, v11, v12, m[s10], m[s11])                                             \
-    CM_G(v2, v7, v8, v13, m[s12], m[s13])                                              \
-    CM_G(v3, v4, v9, v14, m[s14], m[s15])
+    CM_G(0, v0, v4, v8, v12, m[s0], m[s1])                                             \
+    CM_G(1, v1, v5, v9, v13, m[s2], m[s3])                                             \
+    CM_G(2, v2, v6, v10, v14, m[s4], m[s5])                                            \
+    CM_G(3, v3, v7, v11, v15, m[s6], m[s7])                                            \
+    CM_G(4, v0, v5, v10, v15, m[s8], m[s9])                                            \
+    CM_G(5, v1, v6, v11, v12, m[s10], m[s11])                                          \
+    CM_G(6, v2, v7, v8, v13, m[s12], m[s13])                                           \
+    CM_G(7, v3, v4, v9, v14, m[s14], m[s15])
 
 // Compression function F (RFC 7693, Section 3.2), 10 rounds. t = bytes hashed
 // so far including this block; the last-node flag is applied together with the
 // last-block flag, on the node's final compression.
+template <uint32_t kFmaMask>
 __device__ __forceinline__ void compress(uint32_t h[8], const uint32_t m[16], uint64_t t,
                                          bool last_block, bool last_node) {
     uint32_t v0 = h[0], v1 = h[1], v2 = h[2], v3 = h[3];
@@ -239,6 +271,7 @@ __device__ __forceinline__ const uint8_t *cursor_next(const LeafLaunch &a, Strea
 
 constexpr int kLeafThreads = kLeafBlockThreads;
 
+template <uint32_t kFmaMask>
 __global__ void __launch_bounds__(kLeafThreads)
 leaf_hash_kernel(const __grid_constant__ LeafGroup grp) {
     // the blocks after the leaf blocks compute norm keys, one thread per row of K[l*]:
@@ -279,7 +312,7 @@ leaf_hash_kernel(const __grid_constant__ LeafGroup grp) {
                         w2 = load_nc(p + 64 * b + 32), w3 = load_nc(p + 64 * b + 48);
             const uint32_t m[16] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w,
                                     w2.x, w2.y, w2.z, w2.w, w3.x, w3.y, w3.z, w3.w};
-            compress(h, m, (b + 1) * 64, b == 15, last_node);
+            compress<kFmaMask>(h, m, (b + 1) * 64, b == 15, last_node);
         }
         if (CM_IN_BOUNDS(a.digests + leaf * kDigestBytes, kDigestBytes, a.digests,
                          a.num_leaves * kDigestBytes))
@@ -300,7 +333,7 @@ leaf_hash_kernel(const __grid_constant__ LeafGroup grp) {
         const uint32_t m[16] = {w[0].x, w[0].y, w[0].z, w[0].w, w[1].x, w[1].y, w[1].z, w[1].w,
                                 w[2].x, w[2].y, w[2].z, w[2].w, w[3].x, w[3].y, w[3].z, w[3].w};
         const uint32_t end = (b + 1) * 64 < len ? (b + 1) * 64 : len;
-        compress(h, m, end, b + 1 == nblocks, last_node);
+        compress<kFmaMask>(h, m, end, b + 1 == nblocks, last_node);
     }
     if (CM_IN_BOUNDS(a.digests + leaf * kDigestBytes, kDigestBytes, a.digests,
                      a.num_leaves * kDigestBytes))
@@ -349,7 +382,7 @@ inner_hash_kernel(const uint8_t *__restrict__ children, uint64_t num_children,
         const uint32_t m[16] = {w[0].x, w[0].y, w[0].z, w[0].w, w[1].x, w[1].y, w[1].z, w[1].w,
                                 w[2].x, w[2].y, w[2].z, w[2].w, w[3].x, w[3].y, w[3].z, w[3].w};
         const uint32_t end = (b + 1) * 64 < len ? (b + 1) * 64 : len;
-        compress(h, m, end, b + 1 == nblocks, last_node);
+        compress<kLatencyBound>(h, m, end, b + 1 == nblocks, last_node);
     }
     if (CM_IN_BOUNDS(out + j * kDigestBytes, kDigestBytes, out, num_nodes * kDigestBytes))
         store_digest(out + j * kDigestBytes, h);
@@ -374,7 +407,7 @@ __device__ __forceinline__ void hash_node_from(uint4 *stage, uint32_t len, uint8
         const uint32_t m[16] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w,
                                 w2.x, w2.y, w2.z, w2.w, w3.x, w3.y, w3.z, w3.w};
         const uint32_t end = (b + 1) * 64 < len ? (b + 1) * 64 : len;
-        compress(h, m, end, b + 1 == nblocks, last_node);
+        compress<kLatencyBound>(h, m, end, b + 1 == nblocks, last_node);
     }
     if (CM_IN_BOUNDS(out + j * kDigestBytes, kDigestBytes, out, num_nodes * kDigestBytes))
         store_digest(out + j * kDigestBytes, h);
@@ -445,7 +478,7 @@ level1_kernel(const __grid_constant__ TreeTop t) {
         const uint32_t m[16] = {w[0].x, w[0].y, w[0].z, w[0].w, w[1].x, w[1].y, w[1].z, w[1].w,
                                 w[2].x, w[2].y, w[2].z, w[2].w, w[3].x, w[3].y, w[3].z, w[3].w};
         const uint32_t end = (b + 1) * 64 < len ? (b + 1) * 64 : len;
-        compress(h, m, end, b + 1 == nblocks, last_node);
+        compress<kIssueBound>(h, m, end, b + 1 == nblocks, last_node);
     }
     if (CM_IN_BOUNDS(f.level[1] + j * kDigestBytes, kDigestBytes, f.level[1], f.size[1] * kDigestBytes))
         store_digest(f.level[1] + j * kDigestBytes, h);
@@ -503,7 +536,7 @@ CM_DEFINE_BOUNDS_READER(take_hash_bounds_violations)
 
 int leaf_hash_blocks_per_sm() {
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, leaf_hash_kernel, kLeafThreads, 0) != cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, leaf_hash_kernel<kIssueBound>, kLeafThreads, 0) != cudaSuccess)
         return 0;
     return n;
 }
@@ -531,7 +564,10 @@ cudaError_t launch_leaf_hash_group(const LeafGroup &in, cudaStream_t stream, Lea
     }
     const uint64_t blocks = phases == LeafPhases::kBoth ? leaf_blocks + norm_blocks : leaf_blocks;
     if (blocks == 0) return cudaSuccess;
-    leaf_hash_kernel<<<(unsigned)blocks, kLeafThreads, 0, stream>>>(g);
+    if (phases == LeafPhases::kLeaves)   // the norm keys run ahead, to start a render beside
+        leaf_hash_kernel<kBesideRender><<<(unsigned)blocks, kLeafThreads, 0, stream>>>(g);
+    else
+        leaf_hash_kernel<kIssueBound><<<(unsigned)blocks, kLeafThreads, 0, stream>>>(g);
     return cudaGetLastError();
 }
 
@@ -701,8 +737,8 @@ extern "C" cm_status cm_fragment_id_static(const cm_fragment *frag, int32_t rout
 // Register-only kernels that measure the ceiling of the content-address kernels on the
 // current GPU (a profiling aid for their roofline): chains of three-input xors, one
 // integer-ALU instruction each, and the compression function above applied to register
-// data with no memory traffic, counted as the 648 operations per 64-byte block that
-// issue on the integer ALU pipe (10 rounds x 8 G x (4 xors + 4 rotations) + 8 xors).
+// data with no memory traffic, counted as the 648 xors and rotations of a 64-byte block
+// (10 rounds x 8 G x (4 xors + 4 rotations) + 8 xors).
 
 namespace cm {
 namespace {
@@ -732,7 +768,7 @@ compress_probe_kernel(uint32_t *out, int blocks) {
 #pragma unroll
     for (int i = 0; i < 16; ++i) m[i] = tid ^ ((uint32_t)i * 0x9E3779B9u);
     for (int b = 0; b < blocks; ++b) {
-        compress(h, m, (uint64_t)(b + 1) * 64, false, false);
+        compress<kIssueBound>(h, m, (uint64_t)(b + 1) * 64, false, false);
         m[0] ^= h[0];
         m[7] ^= h[3];
         m[11] ^= h[6];
