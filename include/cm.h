@@ -128,8 +128,7 @@ cm_status cm_fragment_id(cm_context *ctx, const cm_fragment *frag, cm_stream_t s
  * exits.
  *   routing_layer  l* (0-indexed); < 0 selects floor(num_layers / 2)
  *   id_out         DEVICE, 16-byte aligned, 16 bytes: receives the id
- *   norm_key_out   DEVICE, 8-byte aligned, seq_len uint64: receives Q[t] (it is zeroed
- *                  on `stream` first, then accumulated)
+ *   norm_key_out   DEVICE, 8-byte aligned, seq_len uint64: receives Q[t]
  * Limit: the fragment's K and V bytes (2 * L * H * T * d * 2) must not exceed 1 GiB;
  * larger fragments return CM_ERR_UNSUPPORTED (use cm_fragment_id).
  * Every call looks the array's device address up (cudaGetSymbolAddress, on the calling
@@ -155,8 +154,8 @@ cm_status cm_ingest(cm_set *set, const cm_fragment *frag, cm_stream_t stream, cm
 
 /* Ingest of n deliveries in order (Algorithm 2, Ingest, applied n times): the same
  * result as n calls of cm_ingest, with one pass of GPU work for all of them (per 32
- * fragments one leaf-hash launch, which also computes the norm keys, and one or two
- * launches for the tree levels above the leaves) and a single synchronisation of
+ * fragments one leaf-hash launch, one for the norm keys, and one or two for the tree levels
+ * above the leaves) and a single synchronisation of
  * `stream`. A delivery whose id is
  * already in the set, or equal to an earlier delivery of the same batch, is
  * absorbed. All fragments must have the set's shape (or one common shape if the
@@ -394,7 +393,8 @@ cm_status cm_context_set_render_warps(cm_context *ctx, int32_t warps);
 
 /* Device time per kernel, accumulated while timing is on (a profiling aid). */
 typedef struct cm_kernel_times {
-    double leaf_hash_ms;          /* content address, level 0 (one launch per up to 32 fragments) */
+    double leaf_hash_ms;          /* content address, level 0 (one launch per up to 32 fragments),
+                                     the norm keys beside it included */
     int64_t leaf_hash_launches;
     double inner_hash_ms;         /* content address, tree levels above the leaves (one
                                      kernel per call, or two when the call has 32,768 or
@@ -403,8 +403,8 @@ typedef struct cm_kernel_times {
     double render_ms;             /* render / BagMerge */
     int64_t render_launches;
     int64_t leaf_hash_fragments;  /* fragments hashed by those leaf-hash launches */
-    int64_t aux_launches;         /* launches of the small kernels (result readback, byte
-                                     comparison), counted, not timed */
+    int64_t aux_launches;         /* launches of the small kernels (norm keys, byte
+                                     comparison, readback), counted, not timed */
 } cm_kernel_times;
 
 /* Turn kernel timing on or off for ctx. While on, every launch the context makes

@@ -1,5 +1,5 @@
 // Content address Id(C) (Section 4.3; Algorithm 2, Id) and the routing-layer
-// norm key (Eq. rho), computed in one pass over the fragment's bytes.
+// norm key (Eq. rho).
 //
 // Id is a BLAKE2s tree hash (RFC 7693 compression function; tree parameters of
 // the BLAKE2 paper, Section 2.10) of the byte stream K[0] V[0] ... K[L-1] V[L-1]:
@@ -7,11 +7,10 @@
 // digests, shapes and dtype in the salt, seq_len in the personalisation.
 //
 // Level 0 runs one thread per leaf: 16 compressions of 64-byte blocks, loaded as
-// 128-bit vectors straight from the fragment buffers. The same launch computes the
-// norm key with one thread per row of K[l*]: the squared norm of the key in fp64 in
-// ascending element order, then the quantised norm (round-half-even of 2^20 * sqrt,
-// saturated at 2^44 - 1) added into Q[t] with a 64-bit integer atomic: integer
-// addition is associative, so Q does not depend on the order the atomics land in.
+// 128-bit vectors straight from the fragment buffers. A launch beside it computes the norm key from K[l*]: a row's squared norm in fp64 in ascending element
+// order by one thread, then the quantised norm (round-half-even of 2^20 * sqrt,
+// saturated at 2^44 - 1) summed over heads into Q[t] as 64-bit integers: integer
+// addition is associative, so Q does not depend on the order of the heads.
 #include "cm_bounds.h"
 #include "cm_hash_kernels.h"
 
@@ -204,30 +203,45 @@ __device__ __forceinline__ double accumulate_squares(uint4 w, double ss) {
     return ss;
 }
 
-// Norm key of row r of K[l*] (Eq. rho; the plane is [H][T][d], so r = h*T + t): one
-// thread reads the row's d/8 vectors and accumulates its squared norm, then adds the
-// quantised norm into Q[t].
-__device__ __forceinline__ void norm_row(const LeafLaunch &a, uint64_t r) {
+// Quantised norm of row r of K[l*] (Eq. rho; the plane is [H][T][d], so r = h*T + t).
+__device__ __forceinline__ unsigned long long row_norm(const LeafLaunch &a, uint64_t r) {
     const uint8_t *row = a.k + a.norm_begin / 2 + r * a.row_bytes;   // K[l*] at stream offset 2 l* plane
     const uint32_t nvec = a.row_bytes >> 4;
     double ss = 0.0;
-    for (uint32_t v = 0; v < nvec; v += 4) {
-        uint4 w[4];
+    for (uint32_t v = 0; v < nvec; v += 8) {   // a 128-byte line's loads in flight together
+        uint4 w[8];
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
+        for (int q = 0; q < 8; ++q)
             if (v + q < nvec)
                 w[q] = CM_IN_BOUNDS(row + 16 * (v + q), 16, a.k + a.norm_begin / 2, a.plane_bytes)
                            ? load_nc(row + 16 * (v + q))
                            : make_uint4(0, 0, 0, 0);
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
+        for (int q = 0; q < 8; ++q)
             if (v + q < nvec) ss = accumulate_squares(w[q], ss);
     }
     const double scaled = __dsqrt_rn(ss) * 1048576.0;     // exact scaling by 2^20
-    const unsigned long long q =
-        (scaled < (double)kQMax) ? __double2ull_rn(scaled) : kQMax;   // NaN saturates too
-    const uint64_t t = r % a.seq_len;
-    if (CM_IN_BOUNDS(a.norm_key + t, 8, a.norm_key, (uint64_t)a.seq_len * 8)) atomicAdd(a.norm_key + t, q);
+    return (scaled < (double)kQMax) ? __double2ull_rn(scaled) : kQMax;   // NaN saturates too
+}
+
+// Norm keys of the tokens of norm block `block` of one fragment: norm_lanes(H) threads share a
+// token's heads, each summing its rows' quantised norms; the integer sums are then added in
+// shared memory. Every Q[t] is written once, by a plain store, so Q needs no zeroing and may
+// lie in host memory that the device maps.
+__device__ __forceinline__ void norm_block(const LeafLaunch &a, uint32_t block) {
+    __shared__ unsigned long long part[kLeafBlockThreads];
+    const uint32_t lanes = norm_lanes(a.heads), tokens = kLeafBlockThreads / lanes;
+    const uint32_t tl = threadIdx.x % tokens, hl = threadIdx.x / tokens;
+    const uint64_t t = (uint64_t)block * tokens + tl;
+    unsigned long long q = 0;
+    if (hl < lanes && t < a.seq_len)
+        for (uint32_t h = hl; h < a.heads; h += lanes) q += row_norm(a, (uint64_t)h * a.seq_len + t);
+    part[threadIdx.x] = q;
+    __syncthreads();
+    if (hl == 0 && t < a.seq_len) {
+        for (uint32_t k = 1; k < lanes; ++k) q += part[tl + k * tokens];
+        if (CM_IN_BOUNDS(a.norm_key + t, 8, a.norm_key, (uint64_t)a.seq_len * 8)) a.norm_key[t] = q;
+    }
 }
 
 // Cursor over the fragment's byte stream K[0] V[0] K[1] V[1] ...: every segment
@@ -269,22 +283,32 @@ __device__ __forceinline__ const uint8_t *cursor_next(const LeafLaunch &a, Strea
     return p;
 }
 
+// A launch with programmatic stream serialisation may start while the launch before it on the
+// stream drains: its blocks wait here until that launch has completed and its writes are
+// visible.
+__device__ __forceinline__ void wait_for_previous_launch() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+// Lets the launch after this one start once every block has come this far (or ended).
+__device__ __forceinline__ void allow_next_launch() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 constexpr int kLeafThreads = kLeafBlockThreads;
 
 template <uint32_t kFmaMask>
 __global__ void __launch_bounds__(kLeafThreads)
 leaf_hash_kernel(const __grid_constant__ LeafGroup grp) {
-    // the blocks after the leaf blocks compute norm keys, one thread per row of K[l*]:
-    // they fill SMs that the last wave of leaf blocks leaves idle
+    // the blocks after the leaf blocks, one per fragment, zero its tree levels' arrival counters
+    // for the tree launch (done by the leaf threads it cost them 8 registers), and end after
+    // the launch before this one, so that the tree launch comes after both
     const uint32_t x = blockIdx.x;
     const uint32_t leaf_blocks = (uint32_t)grp.block_begin[grp.count];
     if (x >= leaf_blocks) {
-        const uint32_t k = x - leaf_blocks;
-        uint32_t fi = 0;
-        while (fi + 1 < grp.count && k >= grp.norm_block_begin[fi + 1]) ++fi;
-        const LeafLaunch &a = grp.frag[fi];
-        const uint64_t r = (uint64_t)(k - grp.norm_block_begin[fi]) * kLeafThreads + threadIdx.x;
-        if (r < (a.plane_bytes >> (__ffs(a.row_bytes) - 1))) norm_row(a, r);
+        const LeafLaunch &a = grp.frag[x - leaf_blocks];
+        for (uint32_t i = threadIdx.x; i < a.num_arrivals; i += kLeafThreads)
+            if (CM_IN_BOUNDS(a.arrivals + i, 4, a.arrivals, (uint64_t)a.num_arrivals * 4)) a.arrivals[i] = 0;
+        wait_for_previous_launch();
         return;
     }
     uint32_t fi = 0;                                   // the block's fragment (uniform)
@@ -340,62 +364,31 @@ leaf_hash_kernel(const __grid_constant__ LeafGroup grp) {
         store_digest(a.digests + leaf * kDigestBytes, h);
 }
 
-// The norm-key rows of a group alone (the blocks that follow the leaf blocks in
-// leaf_hash_kernel, as their own launch): one thread per row of K[l*].
+// The norm keys of a group: the blocks walk over the group's norm blocks. Ahead of a leaf
+// launch they are at most one to an SM (the FP64 pipe bounds them, the ALU and FMA pipes the
+// leaves), and the leaves start as soon as they run.
 __global__ void __launch_bounds__(kLeafThreads)
 norm_key_kernel(const __grid_constant__ LeafGroup grp) {
-    const uint32_t k = blockIdx.x;
+    allow_next_launch();
+    const uint32_t total = (uint32_t)grp.norm_block_begin[grp.count];
     uint32_t fi = 0;
-    while (fi + 1 < grp.count && k >= grp.norm_block_begin[fi + 1]) ++fi;
-    const LeafLaunch &a = grp.frag[fi];
-    const uint64_t r = (uint64_t)(k - grp.norm_block_begin[fi]) * kLeafThreads + threadIdx.x;
-    if (r < (a.plane_bytes >> (__ffs(a.row_bytes) - 1))) norm_row(a, r);
+    for (uint64_t k = blockIdx.x; k < total; k += gridDim.x) {
+        while (fi + 1 < grp.count && k >= grp.norm_block_begin[fi + 1]) ++fi;
+        norm_block(grp.frag[fi], (uint32_t)(k - grp.norm_block_begin[fi]));
+        __syncthreads();   // the sums in shared memory have been read
+    }
 }
 
 constexpr int kInnerThreads = 32;
 
-__global__ void __launch_bounds__(kInnerThreads)
-inner_hash_kernel(const uint8_t *__restrict__ children, uint64_t num_children,
-                  uint8_t *__restrict__ out, uint64_t num_nodes, uint32_t depth,
-                  const __grid_constant__ TreeParams tp) {
-    const uint64_t j = (uint64_t)blockIdx.x * kInnerThreads + threadIdx.x;
-    if (j >= num_nodes) return;
-    const uint64_t first = j * kFanout;
-    const uint64_t nc64 = num_children - first;
-    const uint32_t nc = nc64 < (uint64_t)kFanout ? (uint32_t)nc64 : (uint32_t)kFanout;
-    const uint32_t len = nc * kDigestBytes;
-    const uint32_t nblocks = (len + 63) / 64;
-    const bool last_node = j + 1 == num_nodes;
-    const uint8_t *src = children + first * kDigestBytes;
-
-    uint32_t h[8];
-    node_init(h, tp, j, depth);
-    for (uint32_t b = 0; b < nblocks; ++b) {
-        uint4 w[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const uint32_t off = b * 64 + q * 16;
-            w[q] = off < len && CM_IN_BOUNDS(src + off, 16, children, num_children * kDigestBytes)
-                       ? load_nc(src + off)
-                       : make_uint4(0, 0, 0, 0);
-        }
-        const uint32_t m[16] = {w[0].x, w[0].y, w[0].z, w[0].w, w[1].x, w[1].y, w[1].z, w[1].w,
-                                w[2].x, w[2].y, w[2].z, w[2].w, w[3].x, w[3].y, w[3].z, w[3].w};
-        const uint32_t end = (b + 1) * 64 < len ? (b + 1) * 64 : len;
-        compress<kLatencyBound>(h, m, end, b + 1 == nblocks, last_node);
-    }
-    if (CM_IN_BOUNDS(out + j * kDigestBytes, kDigestBytes, out, num_nodes * kDigestBytes))
-        store_digest(out + j * kDigestBytes, h);
-}
-
-// Node j of a tree level over the digests at `children` (num_children of them): its
-// 16 * min(16, num_children - 16 j) bytes, at most four 64-byte blocks, staged in the
-// thread's 256-byte slice of shared memory so that one copy of the compression loop
-// serves every level (the tree top runs few warps per SM; unrolled copies of the
-// compression would not fit the instruction cache).
-__device__ __forceinline__ void hash_node_from(uint4 *stage, uint32_t len, uint8_t *out,
-                                               uint64_t j, uint64_t num_nodes, uint32_t depth,
-                                               const TreeParams &tp) {
+// Digest of node j of a tree level from its 16 * min(16, num_children - 16 j) bytes of
+// children's digests, at most four 64-byte blocks, staged in the thread's 256-byte slice of
+// shared memory so that one copy of the compression loop serves every level (the tree top
+// runs few warps per SM; unrolled copies of the compression would not fit the instruction
+// cache).
+__device__ __forceinline__ uint4 node_digest(const uint4 *stage, uint32_t len, uint64_t j,
+                                             uint64_t num_nodes, uint32_t depth,
+                                             const TreeParams &tp) {
     const uint32_t nblocks = (len + 63) / 64;
     const bool last_node = j + 1 == num_nodes;
     uint32_t h[8];
@@ -409,28 +402,29 @@ __device__ __forceinline__ void hash_node_from(uint4 *stage, uint32_t len, uint8
         const uint32_t end = (b + 1) * 64 < len ? (b + 1) * 64 : len;
         compress<kLatencyBound>(h, m, end, b + 1 == nblocks, last_node);
     }
-    if (CM_IN_BOUNDS(out + j * kDigestBytes, kDigestBytes, out, num_nodes * kDigestBytes))
-        store_digest(out + j * kDigestBytes, h);
+    return make_uint4(h[0], h[1], h[2], h[3]);
 }
 
-// Loads node j's children (zero-padded to 256 bytes) into `stage`; returns their length.
-// kCoherent: the children were written by other threads of the same launch, so they
-// are read through L2 (ld.global.cg) instead of the non-coherent path.
-template <bool kCoherent>
+// Bytes of children under node j of a level above one of num_children nodes.
+__device__ __forceinline__ uint32_t child_bytes(uint64_t num_children, uint64_t j) {
+    const uint64_t left = num_children - j * kFanout;
+    return (left < (uint64_t)kFanout ? (uint32_t)left : (uint32_t)kFanout) * kDigestBytes;
+}
+
+// Loads node j's children (zero-padded to 256 bytes) into `stage`; returns their length. Read
+// through L2 (ld.global.cg): other threads of this launch, or of the launch that this one
+// overlaps, wrote them.
 __device__ __forceinline__ uint32_t stage_children(uint4 *stage, const uint8_t *children,
                                                    uint64_t num_children, uint64_t j) {
     static_assert(kFanout * kDigestBytes <= 256, "an inner node must fit four blocks");
-    const uint64_t first = j * kFanout;
-    const uint64_t nc64 = num_children - first;
-    const uint32_t nc = nc64 < (uint64_t)kFanout ? (uint32_t)nc64 : (uint32_t)kFanout;
-    const uint32_t len = nc * kDigestBytes;
-    const uint4 *src = reinterpret_cast<const uint4 *>(children + first * kDigestBytes);
+    const uint32_t len = child_bytes(num_children, j);
+    const uint4 *src = reinterpret_cast<const uint4 *>(children + j * kFanout * kDigestBytes);
     uint4 w[16];
 #pragma unroll
     for (int q = 0; q < 16; ++q) {
         const bool in = (uint32_t)(q * 16) < len &&
                         CM_IN_BOUNDS(src + q, 16, children, num_children * kDigestBytes);
-        w[q] = in ? (kCoherent ? __ldcg(src + q) : __ldg(src + q)) : make_uint4(0, 0, 0, 0);
+        w[q] = in ? __ldcg(src + q) : make_uint4(0, 0, 0, 0);
     }
 #pragma unroll
     for (int q = 0; q < 16; ++q) stage[q] = w[q];
@@ -450,19 +444,18 @@ constexpr int kLevel1Threads = 128;
 // hashes a node, and with no shared memory many warps fit on an SM.
 __global__ void __launch_bounds__(kLevel1Threads)
 level1_kernel(const __grid_constant__ TreeTop t) {
+    wait_for_previous_launch();
     const uint64_t g = (uint64_t)blockIdx.x * kLevel1Threads + threadIdx.x;
     if (g >= t.node_begin[t.count]) return;
     uint32_t fi = 0;
     while (fi + 1 < t.count && g >= t.node_begin[fi + 1]) ++fi;
     const TreeTopFragment &f = t.frag[fi];
     const uint64_t j = g - t.node_begin[fi];
-    const uint64_t first = j * kFanout;
-    const uint64_t nc64 = f.size[0] - first;
-    const uint32_t nc = nc64 < (uint64_t)kFanout ? (uint32_t)nc64 : (uint32_t)kFanout;
-    const uint32_t len = nc * kDigestBytes;
+    if (j >= f.size[1]) return;
+    const uint32_t len = child_bytes(f.size[0], j);
     const uint32_t nblocks = (len + 63) / 64;
     const bool last_node = j + 1 == f.size[1];
-    const uint8_t *src = f.level[0] + first * kDigestBytes;
+    const uint8_t *src = f.level[0] + j * kFanout * kDigestBytes;
     uint32_t h[8];
     node_init(h, f.tree, j, 1);
 #pragma unroll 1
@@ -472,7 +465,7 @@ level1_kernel(const __grid_constant__ TreeTop t) {
         for (int q = 0; q < 4; ++q) {
             const uint32_t off = b * 64 + q * 16;
             w[q] = off < len && CM_IN_BOUNDS(src + off, 16, f.level[0], f.size[0] * kDigestBytes)
-                       ? load_nc(src + off)
+                       ? __ldcg(reinterpret_cast<const uint4 *>(src + off))
                        : make_uint4(0, 0, 0, 0);
         }
         const uint32_t m[16] = {w[0].x, w[0].y, w[0].z, w[0].w, w[1].x, w[1].y, w[1].z, w[1].w,
@@ -484,38 +477,64 @@ level1_kernel(const __grid_constant__ TreeTop t) {
         store_digest(f.level[1] + j * kDigestBytes, h);
 }
 
-// Levels kStart and up (node_begin: prefix sums of the level-kStart sizes, 0 for a
-// fragment without that level): one thread per level-kStart node hashes it; then,
-// level by level, the thread that completes a parent's last child hashes the parent.
+// Levels kStart and up (node_begin: prefix sums of the level-kStart sizes, each rounded up to
+// a warp, 0 for a fragment without that level): one thread per level-kStart node hashes it,
+// and lanes 0 and 16 then hash the two parents whose children the warp just hashed (a warp's
+// 32 nodes are those of two parents), handed over in shared memory; from there, level by
+// level, the thread that completes a parent's last child hashes the parent. The chain of
+// levels bounds it: about 0.9 us per compression, four to a node, and between levels a
+// store, an arrival and the loads of 16 digests, which the hand-over saves once.
 template <int kStart>
 __global__ void __launch_bounds__(kInnerThreads)
 tree_top_kernel(const __grid_constant__ TreeTop t) {
+    static_assert(kInnerThreads == 32, "a block is one warp: its lanes hand digests over");
     __shared__ uint4 stage_all[kInnerThreads][16];
-    uint4 *stage = stage_all[threadIdx.x];
-    const uint64_t g = (uint64_t)blockIdx.x * kInnerThreads + threadIdx.x;
-    if (g >= t.node_begin[t.count]) return;
-    uint32_t fi = 0;
+    wait_for_previous_launch();
+    const uint32_t lane = threadIdx.x;
+    const uint64_t g = (uint64_t)blockIdx.x * kInnerThreads + lane;
+    uint32_t fi = 0;                                   // the warp's fragment (uniform)
     while (fi + 1 < t.count && g >= t.node_begin[fi + 1]) ++fi;
     const TreeTopFragment &f = t.frag[fi];
     uint64_t j = g - t.node_begin[fi];
-    uint32_t len = stage_children<false>(stage, f.level[kStart - 1], f.size[kStart - 1], j);
-    for (uint32_t k = kStart;; ++k) {
-        hash_node_from(stage, len, f.level[k], j, f.size[k], k, f.tree);
+    uint32_t k = kStart;
+    const bool mine = j < f.size[k];
+    uint4 digest = make_uint4(0, 0, 0, 0);
+    if (mine) {
+        const uint32_t len = stage_children(stage_all[lane], f.level[k - 1], f.size[k - 1], j);
+        digest = node_digest(stage_all[lane], len, j, f.size[k], k, f.tree);
+    }
+    if (k + 1 < f.levels) {
+        // lane l's digest is child l % 16 of the parent that lane 16 (l / 16) hashes
+        __syncwarp();
+        stage_all[lane & 16u][lane & 15u] = digest;
+        __syncwarp();
+        if (!mine || (lane & 15u) != 0) return;
+        const uint32_t len = child_bytes(f.size[k], j / kFanout);
+        j /= kFanout;
+        ++k;
+        digest = node_digest(stage_all[lane], len, j, f.size[k], k, f.tree);
+    } else if (!mine) {
+        return;
+    }
+    for (;;) {
+        uint8_t *out = f.level[k] + j * kDigestBytes;
+        if (CM_IN_BOUNDS(out, kDigestBytes, f.level[k], f.size[k] * kDigestBytes))
+            *reinterpret_cast<uint4 *>(out) = digest;
         if (k + 1 >= f.levels) break;
         // this thread finished node j of level k; the one that finishes the last child of
         // parent j / 16 hashes the parent
         const uint64_t parent = j / kFanout;
-        const uint64_t first = parent * kFanout;
-        const uint64_t left = f.size[k] - first;
-        const uint32_t siblings = left < (uint64_t)kFanout ? (uint32_t)left : (uint32_t)kFanout;
+        const uint32_t len = child_bytes(f.size[k], parent);
         // one acquire-release add: it publishes this node's digest and, for the thread
         // that counts the last sibling, makes every sibling's digest visible
         if (!CM_IN_BOUNDS(f.arrivals[k + 1] + parent, 4, f.arrivals[k + 1], f.size[k + 1] * 4))
             return;
         const uint32_t done = arrive_acq_rel(f.arrivals[k + 1] + parent) + 1;
-        if (done != siblings) return;
+        if (done * kDigestBytes != len) return;
         j = parent;
-        len = stage_children<true>(stage, f.level[k], f.size[k], j);
+        stage_children(stage_all[lane], f.level[k], f.size[k], j);
+        ++k;
+        digest = node_digest(stage_all[lane], len, j, f.size[k], k, f.tree);
     }
 }
 
@@ -541,87 +560,101 @@ int leaf_hash_blocks_per_sm() {
     return n;
 }
 
-cudaError_t launch_leaf_hash_group(const LeafGroup &in, cudaStream_t stream, LeafPhases phases) {
+namespace {
+
+// Launches a kernel that may start once every block of the launch before it on `stream` has
+// ended or called allow_next_launch; it waits for that launch where it has to
+// (wait_for_previous_launch). The kernels that a tree launch follows do not call it: its
+// one-warp blocks, placed while the leaves still hold most SMs, would crowd on the free ones
+// (one 1021-token ingest 200 us with the call, 160 us without, 167 us launched plainly).
+template <class P>
+cudaError_t launch_after(void (*kernel)(P), uint64_t blocks, int threads, cudaStream_t stream, const P &p) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, p);
+}
+
+}  // namespace
+
+cudaError_t launch_leaf_hash_group(const LeafGroup &g, bool with_norms, int num_sms, cudaStream_t stream) {
+    if (g.count > (uint32_t)kMaxLeafGroup) return cudaErrorInvalidValue;
+    if (g.count == 0) return cudaSuccess;
+    const uint64_t blocks = g.block_begin[g.count] + g.count;   // leaves, then arrival counters
+    if (blocks > 0x7FFFFFFFull) return cudaErrorInvalidValue;
+    if (!with_norms) {   // the norm keys run elsewhere, to start a render beside the leaves
+        leaf_hash_kernel<kBesideRender><<<(unsigned)blocks, kLeafThreads, 0, stream>>>(g);
+        return cudaGetLastError();
+    }
+    const cudaError_t e = launch_norm_keys(g, (uint64_t)num_sms, stream);
+    if (e != cudaSuccess) return e;
+    return launch_after(leaf_hash_kernel<kIssueBound>, blocks, kLeafThreads, stream, g);
+}
+
+cudaError_t launch_norm_keys(const LeafGroup &in, uint64_t max_blocks, cudaStream_t stream) {
     if (in.count > (uint32_t)kMaxLeafGroup) return cudaErrorInvalidValue;
     if (in.count == 0) return cudaSuccess;
     LeafGroup g = in;
-    uint64_t norm_blocks = 0;
     for (uint32_t i = 0; i < g.count; ++i) {
-        const LeafLaunch &a = g.frag[i];
-        const uint64_t rows = a.row_bytes ? a.plane_bytes / a.row_bytes : 0;
-        g.norm_block_begin[i] = norm_blocks;
-        norm_blocks += (rows + kLeafThreads - 1) / kLeafThreads;
+        const uint64_t tokens = kLeafBlockThreads / norm_lanes(g.frag[i].heads);   // per block
+        g.norm_block_begin[i + 1] = g.norm_block_begin[i] + (g.frag[i].seq_len + tokens - 1) / tokens;
     }
-    g.norm_block_begin[g.count] = norm_blocks;
-    const uint64_t leaf_blocks = g.block_begin[g.count];
-    if (leaf_blocks + norm_blocks > 0x7FFFFFFFull) return cudaErrorInvalidValue;
-    // leaf blocks first, then norm-key blocks; a grid of the leaf blocks alone has no
-    // norm-key block, and the norm keys alone run in their own kernel
-    if (phases == LeafPhases::kNormKeys) {
-        if (norm_blocks == 0) return cudaSuccess;
-        norm_key_kernel<<<(unsigned)norm_blocks, kLeafThreads, 0, stream>>>(g);
-        return cudaGetLastError();
-    }
-    const uint64_t blocks = phases == LeafPhases::kBoth ? leaf_blocks + norm_blocks : leaf_blocks;
-    if (blocks == 0) return cudaSuccess;
-    if (phases == LeafPhases::kLeaves)   // the norm keys run ahead, to start a render beside
-        leaf_hash_kernel<kBesideRender><<<(unsigned)blocks, kLeafThreads, 0, stream>>>(g);
-    else
-        leaf_hash_kernel<kIssueBound><<<(unsigned)blocks, kLeafThreads, 0, stream>>>(g);
+    const uint64_t total = g.norm_block_begin[g.count];
+    if (total > 0x7FFFFFFFull) return cudaErrorInvalidValue;
+    const uint64_t blocks = total < max_blocks ? total : max_blocks;
+    norm_key_kernel<<<(unsigned)blocks, kLeafThreads, 0, stream>>>(g);
     return cudaGetLastError();
 }
 
-cudaError_t launch_leaf_hash(const LeafLaunch &a, cudaStream_t stream) {
-    LeafGroup g;
-    std::memset(&g, 0, sizeof g);
-    g.count = 1;
-    g.block_begin[1] = (a.num_leaves + kLeafThreads - 1) / kLeafThreads;   // as the host does
-    g.frag[0] = a;
-    return launch_leaf_hash_group(g, stream, LeafPhases::kBoth);
-}
-
-cudaError_t launch_inner_hash(const uint8_t *children, uint64_t num_children, uint8_t *out,
-                              uint64_t num_nodes, uint32_t depth, const TreeParams &tree,
-                              cudaStream_t stream) {
-    if (num_nodes == 0) return cudaSuccess;
-    const uint64_t blocks = (num_nodes + kInnerThreads - 1) / kInnerThreads;
-    inner_hash_kernel<<<(unsigned)blocks, kInnerThreads, 0, stream>>>(children, num_children, out,
-                                                                    num_nodes, depth, tree);
-    return cudaGetLastError();
+static uint64_t level1_nodes(const TreeTop &t) {
+    uint64_t n = 0;
+    for (uint32_t i = 0; i < t.count; ++i) n += t.frag[i].size[1];
+    return n;
 }
 
 int tree_top_kernels(const TreeTop &t) {
-    if (t.count == 0 || t.count > (uint32_t)kMaxGroup || t.node_begin[t.count] == 0) return 0;
-    if (t.node_begin[t.count] < kSplitLevel1Nodes) return 1;
+    const uint64_t nodes = t.count > (uint32_t)kMaxGroup ? 0 : level1_nodes(t);
+    if (nodes < kSplitLevel1Nodes) return nodes == 0 ? 0 : 1;
     for (uint32_t i = 0; i < t.count; ++i)
         if (t.frag[i].levels >= 3) return 2;
     return 1;
 }
 
-cudaError_t launch_tree_top(const TreeTop &t, cudaStream_t stream) {
-    if (t.count > (uint32_t)kMaxGroup) return cudaErrorInvalidValue;
-    if (t.count == 0) return cudaSuccess;
-    const uint64_t total1 = t.node_begin[t.count];
-    if (total1 == 0) return cudaSuccess;
-    if (total1 < kSplitLevel1Nodes) {
-        // one launch from level 1: the level-2 parents are hashed by the threads that
-        // finish their last child, with no second launch
-        tree_top_kernel<1><<<(unsigned)((total1 + kInnerThreads - 1) / kInnerThreads),
-                             kInnerThreads, 0, stream>>>(t);
-        return cudaGetLastError();
+namespace {
+
+// node_begin for one thread per node of level `k`: each fragment's nodes rounded up to whole
+// warps, so that no warp holds nodes of two fragments.
+void count_level(TreeTop &t, uint32_t k) {
+    for (uint32_t i = 0; i < t.count; ++i) {
+        const uint64_t nodes = k < t.frag[i].levels ? t.frag[i].size[k] : 0;
+        t.node_begin[i + 1] = t.node_begin[i] + (nodes + kInnerThreads - 1) / kInnerThreads * kInnerThreads;
     }
-    level1_kernel<<<(unsigned)((total1 + kLevel1Threads - 1) / kLevel1Threads), kLevel1Threads, 0,
-                    stream>>>(t);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    TreeTop u = t;   // the same fragments, counted by their level-2 nodes
-    for (uint32_t i = 0; i < u.count; ++i)
-        u.node_begin[i + 1] = u.node_begin[i] + (u.frag[i].levels >= 3 ? u.frag[i].size[2] : 0);
-    const uint64_t total2 = u.node_begin[u.count];
-    if (total2 == 0) return cudaSuccess;
-    tree_top_kernel<2><<<(unsigned)((total2 + kInnerThreads - 1) / kInnerThreads), kInnerThreads,
-                         0, stream>>>(u);
-    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_tree_top(const TreeTop &in, cudaStream_t stream) {
+    if (in.count > (uint32_t)kMaxGroup) return cudaErrorInvalidValue;
+    const int kernels = tree_top_kernels(in);
+    if (kernels == 0) return cudaSuccess;
+    TreeTop t = in;
+    count_level(t, 1);
+    const uint64_t total1 = t.node_begin[t.count];
+    if (level1_nodes(in) < kSplitLevel1Nodes)
+        // one launch from level 1: the level-2 parents are hashed by the warps that hash their
+        // children, with no second launch
+        return launch_after(tree_top_kernel<1>, total1 / kInnerThreads, kInnerThreads, stream, t);
+    const cudaError_t e = launch_after(level1_kernel, (total1 + kLevel1Threads - 1) / kLevel1Threads,
+                                       kLevel1Threads, stream, t);
+    if (e != cudaSuccess || kernels == 1) return e;
+    count_level(t, 2);
+    return launch_after(tree_top_kernel<2>, t.node_begin[t.count] / kInnerThreads, kInnerThreads, stream, t);
 }
 
 cudaError_t launch_compare(const void *a, const void *b, uint64_t bytes, unsigned int *flag,
@@ -641,7 +674,7 @@ cudaError_t launch_compare(const void *a, const void *b, uint64_t bytes, unsigne
 //
 // cm_fragment_id_static computes what cm_fragment_id computes, for callers that
 // cannot allocate device memory: its scratch (the digests of every tree level
-// below the root) lives in the file-scope array below, which every GPU that loads
+// below the root and the arrival counters) lives in the file-scope array below, which every GPU that loads
 // this library holds for the life of the process. Host code never uses the
 // array's name as an address: every call looks the array's device address up with
 // cudaGetSymbolAddress, with the calling thread's device current, and keeps no copy
@@ -685,14 +718,19 @@ extern "C" cm_status cm_fragment_id_static(const cm_fragment *frag, int32_t rout
                                 "1 GiB that its static scratch covers; use cm_fragment_id");
         while (sizes.size() == 1 || sizes.back() > 1)
             sizes.push_back((sizes.back() + kFanout - 1) / kFanout);
-        // levels below the root in the static array, each 256-byte aligned; the root
-        // (the last level, one node) is written straight to id_out
+        // levels below the root in the static array, each 256-byte aligned, then the arrival
+        // counters of the levels >= 2; the root (the last level, one node) is written straight
+        // to id_out
         std::vector<size_t> off;
         size_t used = 0;
         for (size_t k = 0; k + 1 < sizes.size(); ++k) {
             off.push_back(used);
             used += ((size_t)sizes[k] * kDigestBytes + 255) & ~(size_t)255;
         }
+        const size_t arrivals_off = used;
+        uint32_t num_arrivals = 0;
+        for (size_t k = 2; k < sizes.size(); ++k) num_arrivals += (uint32_t)sizes[k];
+        used += (size_t)num_arrivals * 4;
         if (used > kStaticScratchBytes)
             return report_error(CM_ERR_UNSUPPORTED, "static scratch layout overflow");
         cudaError_t e = cudaSuccess;
@@ -704,8 +742,6 @@ extern "C" cm_status cm_fragment_id_static(const cm_fragment *frag, int32_t rout
             return report_error(CM_ERR_CUDA, cudaGetErrorString(e));
         }
         uint8_t *scratch = static_cast<uint8_t *>(addr);
-        e = cudaMemsetAsync(norm_key_out, 0, (size_t)T * sizeof(uint64_t), cs);
-        if (e != cudaSuccess) return report_error(CM_ERR_CUDA, cudaGetErrorString(e));
         LeafLaunch a;
         a.k = static_cast<const uint8_t *>(frag->k);
         a.v = static_cast<const uint8_t *>(frag->v);
@@ -716,16 +752,38 @@ extern "C" cm_status cm_fragment_id_static(const cm_fragment *frag, int32_t rout
         a.row_bytes = (uint32_t)d * 2;
         a.seq_len = (uint32_t)T;
         a.norm_key = reinterpret_cast<unsigned long long *>(norm_key_out);
+        a.heads = (uint32_t)H;
+        a.num_arrivals = num_arrivals;
+        a.arrivals = reinterpret_cast<uint32_t *>(scratch + arrivals_off);
         a.digests = scratch + off[0];
         a.tree = make_tree_params(L, H, d, T);
-        e = launch_leaf_hash(a, cs);
+        LeafGroup g;
+        std::memset(&g, 0, sizeof g);
+        g.count = 1;
+        g.block_begin[1] = (a.num_leaves + kLeafThreads - 1) / kLeafThreads;
+        g.frag[0] = a;
+        int device = 0, num_sms = 0;
+        e = cudaGetDevice(&device);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, device);
+        if (e == cudaSuccess) e = launch_leaf_hash_group(g, true, num_sms, cs);
         if (e != cudaSuccess) return report_error(CM_ERR_CUDA, cudaGetErrorString(e));
-        for (size_t k = 1; k < sizes.size(); ++k) {
-            uint8_t *out = (k + 1 == sizes.size()) ? static_cast<uint8_t *>(id_out) : scratch + off[k];
-            e = launch_inner_hash(scratch + off[k - 1], sizes[k - 1], out, sizes[k], (uint32_t)k,
-                                  a.tree, cs);
-            if (e != cudaSuccess) return report_error(CM_ERR_CUDA, cudaGetErrorString(e));
+        TreeTop top;
+        std::memset(&top, 0, sizeof top);
+        top.count = 1;
+        TreeTopFragment &tf = top.frag[0];
+        tf.levels = (uint32_t)sizes.size();
+        uint32_t *arrivals = a.arrivals;
+        for (size_t k = 0; k < sizes.size(); ++k) {
+            tf.size[k] = sizes[k];
+            tf.level[k] = k + 1 == sizes.size() ? static_cast<uint8_t *>(id_out) : scratch + off[k];
+            if (k >= 2) {
+                tf.arrivals[k] = arrivals;
+                arrivals += sizes[k];
+            }
         }
+        tf.tree = a.tree;
+        e = launch_tree_top(top, cs);
+        if (e != cudaSuccess) return report_error(CM_ERR_CUDA, cudaGetErrorString(e));
         return CM_OK;
     } catch (...) {
         return report_error(CM_ERR_OOM, "host allocation failed");

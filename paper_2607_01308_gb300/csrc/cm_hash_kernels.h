@@ -33,18 +33,21 @@ struct LeafLaunch {
     uint64_t norm_begin;           // stream offset of K[l*]; its length is plane_bytes
     uint32_t row_bytes;            // d*2; a power of two in [32, 1024]
     uint32_t seq_len;              // T
-    unsigned long long *norm_key;  // Q[T] accumulators, zeroed before the launch
+    uint32_t heads;                // H
+    uint32_t num_arrivals;         // arrival counters of the tree levels >= 2
+    uint32_t *arrivals;            // zeroed by the leaf launch
+    unsigned long long *norm_key;  // Q[T] out: every entry is written, once
     uint8_t *digests;              // num_leaves * 16 bytes out
     TreeParams tree;
 };
 
 // Level 0 of up to kMaxLeafGroup fragments in one launch: one thread per leaf, the
 // leaf blocks of fragment i being [block_begin[i], block_begin[i + 1]) (set by the
-// caller); after the last leaf block, one thread per row of K[l*] for the routing-layer
-// norm key, the norm blocks of fragment i being block_begin[count] +
-// [norm_block_begin[i], norm_block_begin[i + 1]) (set by the launcher).
+// caller); then one block per fragment that zeroes its arrival counters.
 constexpr int kMaxLeafGroup = 32;
-constexpr int kLeafBlockThreads = 128;   // threads (= leaves or rows) per block of the leaf launch
+constexpr int kLeafBlockThreads = 128;   // threads (= leaves) per block of the leaf launch
+// Threads of a norm block that share one token's heads (the block's other tokens side by side).
+__host__ __device__ constexpr uint32_t norm_lanes(uint32_t heads) { return heads < 32u ? (heads ? heads : 1u) : 32u; }
 struct LeafGroup {
     uint32_t count;
     uint32_t pad_;
@@ -52,43 +55,38 @@ struct LeafGroup {
     uint64_t norm_block_begin[kMaxLeafGroup + 1];
     LeafLaunch frag[kMaxLeafGroup];
 };
-// kBoth: leaves and norm keys in one launch; kLeaves / kNormKeys: one of the two (the
-// norm keys alone read only K[l*], 1/(2L) of the bytes).
-enum class LeafPhases { kBoth, kLeaves, kNormKeys };
-cudaError_t launch_leaf_hash_group(const LeafGroup &g, cudaStream_t stream, LeafPhases phases);
+// with_norms: the group's norm keys too, in a launch of their own beside the leaves; without,
+// they have been launched elsewhere (launch_norm_keys) to start a render beside the leaves.
+cudaError_t launch_leaf_hash_group(const LeafGroup &g, bool with_norms, int num_sms, cudaStream_t stream);
+// The routing-layer norm keys of the group, norm_lanes(H) threads to a token, by at most
+// max_blocks blocks. They read only K[l*], 1/(2L) of the bytes. (Norm block i of fragment f is
+// norm_block_begin[f] + i, set by the launcher.)
+cudaError_t launch_norm_keys(const LeafGroup &g, uint64_t max_blocks, cudaStream_t stream);
 // Leaf-hash blocks that fit on one SM at once (occupancy of leaf_hash_kernel), or 0 on error.
 int leaf_hash_blocks_per_sm();
-
-// Level 0 of one fragment (a group of one).
-cudaError_t launch_leaf_hash(const LeafLaunch &a, cudaStream_t stream);
-
-// Level `depth` >= 1: node j hashes the digests of children [16 j, 16 j + 16).
-cudaError_t launch_inner_hash(const uint8_t *children, uint64_t num_children, uint8_t *out,
-                              uint64_t num_nodes, uint32_t depth, const TreeParams &tree,
-                              cudaStream_t stream);
 
 constexpr int kMaxGroup = 32;
 
 // Every tree level above the leaves, for up to kMaxGroup fragments. One thread per
-// level-s node hashes it; then, level by level, the thread that completes a parent's
-// last child (a per-node arrival counter, zeroed before the launch) hashes that parent,
-// up to the root. No thread ever waits for another. With fewer than kSplitLevel1Nodes
-// level-1 nodes in all, one launch with s = 1. With more, a first launch hashes level 1
-// with every lane of a warp busy and many warps per SM, and a second runs the scheme
-// above with s = 2 (in one launch, each warp would hash 32 level-1 nodes and then two
-// level-2 parents with two of its lanes). The caller sets node_begin from the level-1
-// sizes.
+// level-s node hashes it, and the warp hashes the parents of its nodes; then, level by
+// level, the thread that completes a parent's last child (a per-node arrival counter, zeroed
+// by the leaf launch) hashes that parent, up to the root. No thread ever waits for another
+// block's. With fewer than kSplitLevel1Nodes level-1 nodes in all, one launch with s = 1.
+// With more, a first launch hashes level 1 with every lane of a warp busy and many warps per
+// SM, and a second runs the scheme above with s = 2 (in one launch, each warp would hash 32
+// level-1 nodes and then two level-2 parents with two of its lanes).
 constexpr int kMaxLevels = 12;
 struct TreeTopFragment {
     uint8_t *level[kMaxLevels];       // digests of level k; level[levels - 1] is the root
     uint64_t size[kMaxLevels];        // nodes of level k
-    uint32_t *arrivals[kMaxLevels];   // per node of level k >= 2: children finished so far
+    uint32_t *arrivals[kMaxLevels];   // per node of level k >= 2: children finished so far (0 before)
     uint32_t levels;                  // >= 2
     TreeParams tree;
 };
 struct TreeTop {
     uint32_t count;
-    uint64_t node_begin[kMaxGroup + 1];   // prefix sum of the fragments' level-1 sizes (level 2 in the second launch)
+    // prefix sums of the nodes of the level that a launch starts from (set by launch_tree_top)
+    uint64_t node_begin[kMaxGroup + 1];
     TreeTopFragment frag[kMaxGroup];
 };
 constexpr uint64_t kSplitLevel1Nodes = 32768;

@@ -216,23 +216,16 @@ cm_status ensure_scratch(cm_context *ctx, size_t dev_bytes, size_t host_bytes) {
     return CM_OK;
 }
 
-// Reads a small device result (`bytes` at `src`) into ctx->h_pinned + host_off, enqueued
-// on `stream`: stored by the SMs through the buffer's mapped address when everything is
-// 4-byte granular (so the read does not wait behind bulk device-to-host copies of other
-// streams on the copy engine), else by a copy.
-cudaError_t read_small_at(cm_context *ctx, size_t host_off, const void *src, size_t bytes,
-                          cudaStream_t stream) {
-    if (ctx->h_pinned_dev && bytes % 4 == 0 && host_off % 4 == 0 &&
-        (reinterpret_cast<uintptr_t>(src) & 3u) == 0) {
-        if (ctx->timing) ++ctx->aux_launches;
-        return cm::launch_readback(static_cast<uint8_t *>(ctx->h_pinned_dev) + host_off, src, bytes,
-                                   stream);
-    }
-    return cudaMemcpyAsync(ctx->h_pinned + host_off, src, bytes, cudaMemcpyDeviceToHost, stream);
-}
-
+// Reads a small device result (`bytes` at `src`) into ctx->h_pinned, enqueued on `stream`:
+// stored by the SMs through the buffer's mapped address when everything is 4-byte granular
+// (so the read does not wait behind bulk device-to-host copies of other streams on the copy
+// engine), else by a copy.
 cudaError_t read_small(cm_context *ctx, const void *src, size_t bytes, cudaStream_t stream) {
-    return read_small_at(ctx, 0, src, bytes, stream);
+    if (ctx->h_pinned_dev && bytes % 4 == 0 && (reinterpret_cast<uintptr_t>(src) & 3u) == 0) {
+        if (ctx->timing) ++ctx->aux_launches;
+        return cm::launch_readback(ctx->h_pinned_dev, src, bytes, stream);
+    }
+    return cudaMemcpyAsync(ctx->h_pinned, src, bytes, cudaMemcpyDeviceToHost, stream);
 }
 
 // BLAKE2s parameter block (32 bytes) of the tree, node offset and depth zero,
@@ -302,19 +295,19 @@ cudaError_t timed_launch(cm_context *ctx, int kind, cudaStream_t stream, F &&lau
 
 // The scratch of one content-address pass over n fragments (Section 4.3; Algorithm 2,
 // Id): device [roots n x 16][Q of fragment 0]...[Q of fragment n-1][arrival counters of
-// the nodes at levels >= 2][the levels below each root]; the pinned host buffer receives
-// [roots][Q ...] at the same offsets.
+// the nodes at levels >= 2][the levels below each root]; the pinned host buffer holds
+// [roots][Q ...] at the same offsets, and the kernels write them there when it is mapped
+// (the device areas of the same name are then unused).
 struct DigestPlan {
     struct Frag {
         std::vector<uint64_t> sizes;     // nodes per level, leaves first; the last is the root
         std::vector<size_t> level_off;   // device offsets of the levels below the root
         size_t q_off = 0, arr_off = 0;
-        uint64_t plane = 0, stream_bytes = 0;
-        int32_t rl = 0;
+        uint32_t num_arrivals = 0;
         cm::TreeParams tp;
     };
     std::vector<Frag> f;
-    size_t roots_bytes = 0, host_bytes = 0, zero_end = 0, dev_bytes = 0;
+    size_t roots_bytes = 0, host_bytes = 0, dev_bytes = 0;
 };
 
 cm_status plan_digest(cm_context *ctx, const cm_fragment *const *frags, size_t n, DigestPlan &plan) {
@@ -324,11 +317,10 @@ cm_status plan_digest(cm_context *ctx, const cm_fragment *const *frags, size_t n
     for (size_t i = 0; i < n; ++i) {
         const cm_fragment *f = frags[i];
         DigestPlan::Frag &l = plan.f[i];
-        l.rl = routing_layer_for(ctx, f->num_layers);
-        if (l.rl >= f->num_layers) return fail(CM_ERR_INVALID_ARG, "routing layer >= num_layers");
-        l.plane = (uint64_t)f->num_kv_heads * f->seq_len * f->head_dim * 2;
-        l.stream_bytes = 2ull * f->num_layers * l.plane;
-        l.sizes.assign(1, ceil_div(l.stream_bytes, cm::kLeafBytes));
+        if (routing_layer_for(ctx, f->num_layers) >= f->num_layers)
+            return fail(CM_ERR_INVALID_ARG, "routing layer >= num_layers");
+        const uint64_t stream_bytes = 4ull * f->num_layers * f->num_kv_heads * f->seq_len * f->head_dim;
+        l.sizes.assign(1, ceil_div(stream_bytes, cm::kLeafBytes));
         while (l.sizes.size() == 1 || l.sizes.back() > 1)
             l.sizes.push_back(ceil_div(l.sizes.back(), cm::kFanout));
         if (l.sizes.size() > (size_t)cm::kMaxLevels)
@@ -338,12 +330,12 @@ cm_status plan_digest(cm_context *ctx, const cm_fragment *const *frags, size_t n
         l.tp = tree_params(f->num_layers, f->num_kv_heads, f->head_dim, f->seq_len);
     }
     plan.host_bytes = off;   // roots and norm keys
-    // the arrival counters follow the norm keys, so that one memset zeroes both
     for (size_t i = 0; i < n; ++i) {
-        plan.f[i].arr_off = off;
-        for (size_t k = 2; k < plan.f[i].sizes.size(); ++k) off += (size_t)plan.f[i].sizes[k] * 4;
+        DigestPlan::Frag &l = plan.f[i];
+        l.arr_off = off;
+        for (size_t k = 2; k < l.sizes.size(); ++k) l.num_arrivals += (uint32_t)l.sizes[k];
+        off += (size_t)l.num_arrivals * 4;
     }
-    plan.zero_end = off;
     off = (off + 255) & ~(size_t)255;
     for (size_t i = 0; i < n; ++i) {
         DigestPlan::Frag &l = plan.f[i];
@@ -356,18 +348,33 @@ cm_status plan_digest(cm_context *ctx, const cm_fragment *const *frags, size_t n
     return CM_OK;
 }
 
+// The leaf-launch descriptor of a fragment, its outputs left to the caller.
+cm::LeafLaunch leaf_launch(const cm_context *ctx, const cm_fragment *f, const cm::TreeParams &tp) {
+    cm::LeafLaunch a;
+    std::memset(&a, 0, sizeof a);
+    a.k = static_cast<const uint8_t *>(f->k);
+    a.v = static_cast<const uint8_t *>(f->v);
+    a.plane_bytes = (uint64_t)f->num_kv_heads * f->seq_len * f->head_dim * 2;
+    a.stream_bytes = 2ull * f->num_layers * a.plane_bytes;
+    a.num_leaves = ceil_div(a.stream_bytes, cm::kLeafBytes);
+    a.norm_begin = 2ull * (uint64_t)routing_layer_for(ctx, f->num_layers) * a.plane_bytes;
+    a.row_bytes = (uint32_t)f->head_dim * 2;
+    a.seq_len = (uint32_t)f->seq_len;
+    a.heads = (uint32_t)f->num_kv_heads;
+    a.tree = tp;
+    return a;
+}
+
 // Enqueues a planned pass on `stream` (the scratch already holds plan.dev_bytes and
-// plan.host_bytes): the leaf launches of up to kMaxLeafGroup fragments each (with the
-// norm keys when with_norms), the tree levels above the leaves (level 1, then the levels
-// above it: two launches per kMaxGroup fragments), and the results' way to the pinned
-// buffer. When the buffer is mapped, the kernels that hash the roots store them there
-// directly and only the norm keys are read back; otherwise roots and keys are copied.
+// plan.host_bytes): the leaf launches of up to kMaxLeafGroup fragments each, beside their norm
+// keys (with_norms; without, those run ahead of a render that starts beside the leaves), then
+// the tree levels above the leaves (level 1, then the levels
+// above it: one or two launches per kMaxGroup fragments). When the pinned buffer is mapped,
+// the kernels store the roots and norm keys there; otherwise they are copied.
 cm_status enqueue_digest(cm_context *ctx, const DigestPlan &plan, const cm_fragment *const *frags,
                          size_t n, cudaStream_t stream, bool with_norms) {
     uint8_t *base = ctx->d_scratch;
-    uint8_t *roots = ctx->h_pinned_dev ? static_cast<uint8_t *>(ctx->h_pinned_dev) : base;
-    CM_CUDA_TRY(cudaMemsetAsync(base + plan.roots_bytes, 0, plan.zero_end - plan.roots_bytes, stream),
-                "zeroing the norm keys and arrival counters");
+    uint8_t *results = ctx->h_pinned_dev ? static_cast<uint8_t *>(ctx->h_pinned_dev) : base;
     std::unique_ptr<cm::LeafGroup> grp(new cm::LeafGroup);
     for (size_t g0 = 0; g0 < n; g0 += (size_t)cm::kMaxLeafGroup) {
         const size_t gn = std::min(n - g0, (size_t)cm::kMaxLeafGroup);
@@ -377,26 +384,20 @@ cm_status enqueue_digest(cm_context *ctx, const DigestPlan &plan, const cm_fragm
             const cm_fragment *f = frags[g0 + q];
             const DigestPlan::Frag &l = plan.f[g0 + q];
             cm::LeafLaunch &a = grp->frag[q];
-            a.k = static_cast<const uint8_t *>(f->k);
-            a.v = static_cast<const uint8_t *>(f->v);
-            a.plane_bytes = l.plane;
-            a.stream_bytes = l.stream_bytes;
-            a.num_leaves = l.sizes[0];
-            a.norm_begin = 2ull * (uint64_t)l.rl * l.plane;
-            a.row_bytes = (uint32_t)f->head_dim * 2;
-            a.seq_len = (uint32_t)f->seq_len;
-            a.norm_key = reinterpret_cast<unsigned long long *>(base + l.q_off);
+            a = leaf_launch(ctx, f, l.tp);
+            a.num_arrivals = l.num_arrivals;
+            a.arrivals = reinterpret_cast<uint32_t *>(base + l.arr_off);
+            a.norm_key = reinterpret_cast<unsigned long long *>(results + l.q_off);
             a.digests = base + l.level_off[0];
-            a.tree = l.tp;
             grp->block_begin[q + 1] = grp->block_begin[q] + ceil_div(a.num_leaves, (uint64_t)cm::kLeafBlockThreads);
         }
         if (grp->block_begin[gn] > 0x7FFFFFFFull)
             return fail(CM_ERR_UNSUPPORTED, "leaf-hash launch exceeds 2^31 - 1 blocks");
-        const cm::LeafPhases phases = with_norms ? cm::LeafPhases::kBoth : cm::LeafPhases::kLeaves;
         CM_CUDA_TRY(timed_launch(ctx, kTimeLeaf, stream,
-                                 [&] { return cm::launch_leaf_hash_group(*grp, stream, phases); }),
+                                 [&] { return cm::launch_leaf_hash_group(*grp, with_norms, ctx->num_sms, stream); }),
                     "leaf hash launch");
         if (ctx->timing) ctx->leaf_fragments += (int64_t)gn;
+        if (ctx->timing && with_norms) ++ctx->aux_launches;
     }
     std::unique_ptr<cm::TreeTop> top(new cm::TreeTop);
     std::memset(top.get(), 0, sizeof(cm::TreeTop));
@@ -416,25 +417,21 @@ cm_status enqueue_digest(cm_context *ctx, const DigestPlan &plan, const cm_fragm
         size_t a_off = l.arr_off;
         for (size_t k = 0; k < l.sizes.size(); ++k) {
             tf.size[k] = l.sizes[k];
-            tf.level[k] = (k + 1 == l.sizes.size()) ? roots + 16 * i : base + l.level_off[k];
+            tf.level[k] = (k + 1 == l.sizes.size()) ? results + 16 * i : base + l.level_off[k];
             if (k >= 2) {
                 tf.arrivals[k] = reinterpret_cast<uint32_t *>(base + a_off);
                 a_off += (size_t)l.sizes[k] * 4;
             }
         }
         tf.tree = l.tp;
-        top->node_begin[c + 1] = top->node_begin[c] + l.sizes[1];
         top->count = c + 1;
         if (top->count == (uint32_t)cm::kMaxGroup) CM_CUDA_TRY(flush(), "tree-top launch");
     }
     CM_CUDA_TRY(flush(), "tree-top launch");
     if (!ctx->h_pinned_dev)
-        CM_CUDA_TRY(read_small_at(ctx, 0, base, with_norms ? plan.host_bytes : plan.roots_bytes, stream),
+        CM_CUDA_TRY(cudaMemcpyAsync(ctx->h_pinned, base, with_norms ? plan.host_bytes : plan.roots_bytes,
+                                    cudaMemcpyDeviceToHost, stream),
                     "digest copy");
-    else if (with_norms)
-        CM_CUDA_TRY(read_small_at(ctx, plan.roots_bytes, base + plan.roots_bytes,
-                                  plan.host_bytes - plan.roots_bytes, stream),
-                    "norm-key copy");
     return CM_OK;
 }
 
@@ -465,14 +462,14 @@ cm_status fragments_digest(cm_context *ctx, const cm_fragment *const *frags, siz
 }
 
 // Enqueues Q[t] of n fragments alone (Eq. rho) on `stream`: one launch of the norm-key
-// row threads per kMaxLeafGroup fragments (they read only K[l*]) into device scratch at
-// dev_off (q_off[i] after it for fragment i; zeroed first), then a copy to the pinned
-// buffer at host_off (same relative offsets).
+// blocks per kMaxLeafGroup fragments (they read only K[l*]) into the pinned buffer at
+// host_off (q_off[i] after it for fragment i), through device scratch at dev_off (same
+// relative offsets) when the buffer is not mapped.
 cm_status enqueue_norm_keys(cm_context *ctx, const cm_fragment *const *frags, size_t n,
                             cudaStream_t stream, size_t dev_off, size_t host_off,
                             const std::vector<size_t> &q_off, size_t bytes) {
-    uint8_t *base = ctx->d_scratch + dev_off;
-    CM_CUDA_TRY(cudaMemsetAsync(base, 0, bytes, stream), "zeroing the norm keys");
+    uint8_t *base = ctx->h_pinned_dev ? static_cast<uint8_t *>(ctx->h_pinned_dev) + host_off
+                                      : ctx->d_scratch + dev_off;
     std::unique_ptr<cm::LeafGroup> grp(new cm::LeafGroup);
     for (size_t g0 = 0; g0 < n; g0 += (size_t)cm::kMaxLeafGroup) {
         const size_t gn = std::min(n - g0, (size_t)cm::kMaxLeafGroup);
@@ -481,26 +478,16 @@ cm_status enqueue_norm_keys(cm_context *ctx, const cm_fragment *const *frags, si
         for (size_t q = 0; q < gn; ++q) {
             const cm_fragment *f = frags[g0 + q];
             cm::LeafLaunch &a = grp->frag[q];
-            a.k = static_cast<const uint8_t *>(f->k);
-            a.v = static_cast<const uint8_t *>(f->v);
-            a.plane_bytes = (uint64_t)f->num_kv_heads * f->seq_len * f->head_dim * 2;
-            a.stream_bytes = 2ull * f->num_layers * a.plane_bytes;
-            a.num_leaves = ceil_div(a.stream_bytes, cm::kLeafBytes);
-            a.norm_begin = 2ull * (uint64_t)routing_layer_for(ctx, f->num_layers) * a.plane_bytes;
-            a.row_bytes = (uint32_t)f->head_dim * 2;
-            a.seq_len = (uint32_t)f->seq_len;
+            a = leaf_launch(ctx, f, tree_params(f->num_layers, f->num_kv_heads, f->head_dim, f->seq_len));
             a.norm_key = reinterpret_cast<unsigned long long *>(base + q_off[g0 + q]);
-            a.tree = tree_params(f->num_layers, f->num_kv_heads, f->head_dim, f->seq_len);
-            grp->block_begin[q + 1] =
-                grp->block_begin[q] + ceil_div(a.num_leaves, (uint64_t)cm::kLeafBlockThreads);
         }
-        if (grp->block_begin[gn] > 0x7FFFFFFFull)
-            return fail(CM_ERR_UNSUPPORTED, "leaf-hash launch exceeds 2^31 - 1 blocks");
-        CM_CUDA_TRY(cm::launch_leaf_hash_group(*grp, stream, cm::LeafPhases::kNormKeys),
+        CM_CUDA_TRY(cm::launch_norm_keys(*grp, UINT64_MAX, stream),
                     "norm-key launch");
         if (ctx->timing) ++ctx->aux_launches;
     }
-    CM_CUDA_TRY(read_small_at(ctx, host_off, base, bytes, stream), "norm-key copy");
+    if (!ctx->h_pinned_dev)
+        CM_CUDA_TRY(cudaMemcpyAsync(ctx->h_pinned + host_off, base, bytes, cudaMemcpyDeviceToHost, stream),
+                    "norm-key copy");
     return CM_OK;
 }
 
