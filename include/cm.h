@@ -246,9 +246,9 @@ cm_status cm_render(const cm_set *set, void *k_out, void *v_out, int64_t capacit
  * fragments, the other sets', every delivery) whose integer tail sums S, lengths and
  * per-token norm keys all agree are taken for one fragment; if the remaining S are
  * pairwise distinct, the canonical order of Algorithm 1 does not depend on the ids: the
- * render starts at once on a stream of the context, with narrow CTAs, while the content
- * address runs on `stream`. When the ids are known the set is checked to hold exactly
- * the fragments rendered, in that order (different fragments taken for one, or sharing
+ * render starts on a stream of the context, with narrow CTAs, while the content address
+ * runs on `stream`: at once, or (middling sizes) as its first level ends. When the ids are
+ * known the set is checked to hold exactly the fragments rendered, in that order (different fragments taken for one, or sharing
  * an address, which the paper's collision assumption excludes, fail the check; then the
  * target is rendered again after the first render, so the result is still exact). With
  * a tie of S between members that differ in length or norm keys, with the re-delivery

@@ -583,13 +583,16 @@ cudaError_t launch_after(void (*kernel)(P), uint64_t blocks, int threads, cudaSt
 
 }  // namespace
 
-cudaError_t launch_leaf_hash_group(const LeafGroup &g, bool with_norms, int num_sms, cudaStream_t stream) {
+cudaError_t launch_leaf_hash_group(const LeafGroup &g, LeafMode mode, int num_sms, cudaStream_t stream) {
     if (g.count > (uint32_t)kMaxLeafGroup) return cudaErrorInvalidValue;
     if (g.count == 0) return cudaSuccess;
     const uint64_t blocks = g.block_begin[g.count] + g.count;   // leaves, then arrival counters
     if (blocks > 0x7FFFFFFFull) return cudaErrorInvalidValue;
-    if (!with_norms) {   // the norm keys run elsewhere, to start a render beside the leaves
-        leaf_hash_kernel<kBesideRender><<<(unsigned)blocks, kLeafThreads, 0, stream>>>(g);
+    if (mode != LeafMode::kWithNorms) {
+        if (mode == LeafMode::kBesideRender)
+            leaf_hash_kernel<kBesideRender><<<(unsigned)blocks, kLeafThreads, 0, stream>>>(g);
+        else
+            leaf_hash_kernel<kIssueBound><<<(unsigned)blocks, kLeafThreads, 0, stream>>>(g);
         return cudaGetLastError();
     }
     const cudaError_t e = launch_norm_keys(g, (uint64_t)num_sms, stream);
@@ -765,7 +768,7 @@ extern "C" cm_status cm_fragment_id_static(const cm_fragment *frag, int32_t rout
         int device = 0, num_sms = 0;
         e = cudaGetDevice(&device);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, device);
-        if (e == cudaSuccess) e = launch_leaf_hash_group(g, true, num_sms, cs);
+        if (e == cudaSuccess) e = launch_leaf_hash_group(g, LeafMode::kWithNorms, num_sms, cs);
         if (e != cudaSuccess) return report_error(CM_ERR_CUDA, cudaGetErrorString(e));
         TreeTop top;
         std::memset(&top, 0, sizeof top);

@@ -150,10 +150,11 @@ struct cm_context {
     // launch parameters of the render kernel (about 31 KB), reused by every launch
     std::unique_ptr<cm::RenderParams> render_params;
     int32_t render_warps = 16;   // warps per render CTA (cm_context_set_render_warps)
-    // cm_ingest_render: the stream its overlapped render runs on and the two events that
-    // order it after the caller's stream and the caller's stream after it (made on first use)
+    // cm_ingest_render: the stream its overlapped render runs on and the events that order
+    // it after the caller's stream (or its leaf hash) and the caller's stream after it (made on
+    // first use)
     cudaStream_t side = nullptr;
-    cudaEvent_t side_begin = nullptr, side_end = nullptr, side_keys = nullptr;
+    cudaEvent_t side_begin = nullptr, side_end = nullptr, side_keys = nullptr, leaves_end = nullptr;
     int32_t overlap = 1;         // cm_context_set_overlap: 1 render beside the hash when possible
     bool dedup_bytes = false;    // re-delivery fast path (cm_context_set_dedup_by_bytes)
 };
@@ -366,13 +367,14 @@ cm::LeafLaunch leaf_launch(const cm_context *ctx, const cm_fragment *f, const cm
 }
 
 // Enqueues a planned pass on `stream` (the scratch already holds plan.dev_bytes and
-// plan.host_bytes): the leaf launches of up to kMaxLeafGroup fragments each, beside their norm
-// keys (with_norms; without, those run ahead of a render that starts beside the leaves), then
-// the tree levels above the leaves (level 1, then the levels
+// plan.host_bytes): the leaf launches of up to kMaxLeafGroup fragments each, by mode beside
+// their norm keys, then (after the event leaves_end, if any) the tree levels above the leaves (level 1, then the levels
 // above it: one or two launches per kMaxGroup fragments). When the pinned buffer is mapped,
 // the kernels store the roots and norm keys there; otherwise they are copied.
 cm_status enqueue_digest(cm_context *ctx, const DigestPlan &plan, const cm_fragment *const *frags,
-                         size_t n, cudaStream_t stream, bool with_norms) {
+                         size_t n, cudaStream_t stream, cm::LeafMode mode,
+                         cudaEvent_t leaves_end = nullptr) {
+    const bool with_norms = mode == cm::LeafMode::kWithNorms;
     uint8_t *base = ctx->d_scratch;
     uint8_t *results = ctx->h_pinned_dev ? static_cast<uint8_t *>(ctx->h_pinned_dev) : base;
     std::unique_ptr<cm::LeafGroup> grp(new cm::LeafGroup);
@@ -394,11 +396,12 @@ cm_status enqueue_digest(cm_context *ctx, const DigestPlan &plan, const cm_fragm
         if (grp->block_begin[gn] > 0x7FFFFFFFull)
             return fail(CM_ERR_UNSUPPORTED, "leaf-hash launch exceeds 2^31 - 1 blocks");
         CM_CUDA_TRY(timed_launch(ctx, kTimeLeaf, stream,
-                                 [&] { return cm::launch_leaf_hash_group(*grp, with_norms, ctx->num_sms, stream); }),
+                                 [&] { return cm::launch_leaf_hash_group(*grp, mode, ctx->num_sms, stream); }),
                     "leaf hash launch");
         if (ctx->timing) ctx->leaf_fragments += (int64_t)gn;
         if (ctx->timing && with_norms) ++ctx->aux_launches;
     }
+    if (leaves_end) CM_CUDA_TRY(cudaEventRecord(leaves_end, stream), "leaf event");
     std::unique_ptr<cm::TreeTop> top(new cm::TreeTop);
     std::memset(top.get(), 0, sizeof(cm::TreeTop));
     auto flush = [&]() -> cudaError_t {
@@ -454,7 +457,7 @@ cm_status fragments_digest(cm_context *ctx, const cm_fragment *const *frags, siz
     DigestPlan plan;
     cm_status st = plan_digest(ctx, frags, n, plan);
     if (st == CM_OK) st = ensure_scratch(ctx, plan.dev_bytes, plan.host_bytes);
-    if (st == CM_OK) st = enqueue_digest(ctx, plan, frags, n, stream, true);
+    if (st == CM_OK) st = enqueue_digest(ctx, plan, frags, n, stream, cm::LeafMode::kWithNorms);
     if (st != CM_OK) return st;
     CM_CUDA_TRY(cudaStreamSynchronize(stream), "ingest synchronisation");
     collect_digest(ctx, plan, frags, n, ids, Qs);
@@ -1082,6 +1085,7 @@ cm_status cm_context_destroy(cm_context *ctx) {
         if (ctx->side_begin) cudaEventDestroy(ctx->side_begin);
         if (ctx->side_end) cudaEventDestroy(ctx->side_end);
         if (ctx->side_keys) cudaEventDestroy(ctx->side_keys);
+        if (ctx->leaves_end) cudaEventDestroy(ctx->leaves_end);
         for (const auto &pe : ctx->pending) {
             cudaEventDestroy(pe.start);
             cudaEventDestroy(pe.end);
@@ -1350,10 +1354,15 @@ std::vector<Slot> canonical_slots(const cm_set *set, void *k_out, void *v_out, i
     return slots;
 }
 
-// A render beside the leaf hash (cm_ingest_render) whose fragments hold at least this
-// many bytes takes the 4-warp TMA kernel, a smaller one the register kernel with one CTA
-// per SM: measured on the Qwen3 shapes, the register kernel was the faster neighbour of
-// the hash for 0.3 GB of fragments, the TMA kernel from 1.2 GB on.
+// When cm_ingest_render's render starts, and how wide. From this many bytes of fragments on it
+// runs beside the leaf hash as the 4-warp TMA kernel; a smaller one whose leaf hash fills the
+// GPU starts as the leaves end, beside the tree levels (whose few warps leave it the memory),
+// as the register kernel with two CTAs per SM, and one whose leaf hash leaves room on every SM
+// starts at once beside it, as the register kernel with one. Measured (us, on the Qwen3 shapes;
+// beside with one CTA, beside as the TMA kernel, after the leaves): 2 x 512 tokens 146, -, 152;
+// 2 x 700 192, -, 182; 4 x 512 306, 364, 281; 4 x 850 (505 MB) 475, 494, 457; 3 x 1500
+// (663 MB) -, 533, 590; 3 x 2000 -, 666, 777. One or three CTAs after the leaves: 4 x 512
+// 330, 292.
 constexpr uint64_t kBesideLargeBytes = 512ull << 20;
 
 cm_status ensure_side_stream(cm_context *ctx) {
@@ -1365,12 +1374,8 @@ cm_status ensure_side_stream(cm_context *ctx) {
         CM_CUDA_TRY(cudaStreamCreateWithPriority(&ctx->side, cudaStreamNonBlocking, greatest),
                     "side stream");
     }
-    if (!ctx->side_begin)
-        CM_CUDA_TRY(cudaEventCreateWithFlags(&ctx->side_begin, cudaEventDisableTiming), "side event");
-    if (!ctx->side_end)
-        CM_CUDA_TRY(cudaEventCreateWithFlags(&ctx->side_end, cudaEventDisableTiming), "side event");
-    if (!ctx->side_keys)
-        CM_CUDA_TRY(cudaEventCreateWithFlags(&ctx->side_keys, cudaEventDisableTiming), "side event");
+    for (cudaEvent_t *e : {&ctx->side_begin, &ctx->side_end, &ctx->side_keys, &ctx->leaves_end})
+        if (!*e) CM_CUDA_TRY(cudaEventCreateWithFlags(e, cudaEventDisableTiming), "side event");
     return CM_OK;
 }
 
@@ -1490,17 +1495,31 @@ cm_status ingest_render_impl(cm_set *const *sets, const cm_fragment *frags, int3
         if (e != cudaSuccess && prior == CM_OK) return cuda_fail(e, "side stream ordering");
         return prior;
     };
-    // The norm keys decide when the render can start. A leaf grid that leaves a block's room
-    // on every SM (one partial wave) is launched first: the hash starts a few launches
-    // earlier and the norm-key blocks still start at once beside it. A larger grid would
-    // take every SM and hold back norm keys launched after it until its first wave retires.
+    // The norm keys decide when a render beside the leaf hash can start. A leaf grid that leaves
+    // a block's room on every SM (one partial wave) is launched first: the hash starts a few
+    // launches earlier and the norm-key blocks still start at once beside it. A larger grid
+    // would take every SM and hold back norm keys launched after it until its first wave
+    // retires, which a render that waits for the leaves anyway can afford.
     uint64_t leaf_blocks = 0;
     for (const DigestPlan::Frag &l : plan.f) leaf_blocks += ceil_div(l.sizes[0], (uint64_t)cm::kLeafBlockThreads);
-    const bool digest_first =
+    const bool partial_wave =
         ctx->leaf_blocks_per_sm > 1 &&
         leaf_blocks <= (uint64_t)(ctx->leaf_blocks_per_sm - 1) * (uint64_t)ctx->num_sms;
+    int64_t most_tokens = 0;   // of the prospective set, repeats included
+    for (const auto &kv : target->items) most_tokens += kv.second->T;
+    for (const cm_set *src : sources)
+        for (const auto &kv : src->items) most_tokens += kv.second->T;
+    for (const cm_fragment *f : fp) most_tokens += f->seq_len;
+    const uint64_t token_bytes = 4ull * (uint64_t)L * (uint64_t)H * (uint64_t)d;
+    const bool after_leaves = !partial_wave && (uint64_t)most_tokens * token_bytes < kBesideLargeBytes;
+    const bool digest_first = partial_wave || after_leaves;
+    auto digest = [&]() -> cm_status {
+        return enqueue_digest(ctx, plan, fp.data(), fp.size(), cs,
+                              after_leaves ? cm::LeafMode::kAlone : cm::LeafMode::kBesideRender,
+                              after_leaves ? ctx->leaves_end : nullptr);
+    };
     if (digest_first) {
-        st = enqueue_digest(ctx, plan, fp.data(), fp.size(), cs, false);
+        st = digest();
         if (st != CM_OK) return join(st);
     }
     st = enqueue_norm_keys(ctx, fp.data(), fp.size(), ctx->side, q_dev, q_host, q_off, q_bytes);
@@ -1508,7 +1527,7 @@ cm_status ingest_render_impl(cm_set *const *sets, const cm_fragment *frags, int3
     cudaError_t e = cudaEventRecord(ctx->side_keys, ctx->side);
     if (e != cudaSuccess) return join(cuda_fail(e, "side stream ordering"));
     if (!digest_first) {
-        st = enqueue_digest(ctx, plan, fp.data(), fp.size(), cs, false);
+        st = digest();
         if (st != CM_OK) return join(st);
     }
     e = cudaEventSynchronize(ctx->side_keys);
@@ -1575,12 +1594,15 @@ cm_status ingest_render_impl(cm_set *const *sets, const cm_fragment *frags, int3
                 spec_slots.push_back({x.k, x.v, x.T, s, k_out, v_out, capacity});
                 s += x.T;
             }
-            // beside the leaf hash: a narrow render, its kernel chosen by size
-            const uint64_t frag_bytes = 2ull * (uint64_t)total * (uint64_t)L * (uint64_t)H * (uint64_t)d * 2;
-            const cm::RenderWidth beside = frag_bytes >= kBesideLargeBytes
-                                               ? cm::RenderWidth::kBeside
-                                               : cm::RenderWidth::kBesideSmall;
-            st = launch_slots(ctx, spec_slots, L, H, d, ctx->side, 0, nullptr, &beside);
+            const cm::RenderWidth width = after_leaves ? cm::RenderWidth::kAfterLeaves
+                                          : (uint64_t)total * token_bytes >= kBesideLargeBytes
+                                              ? cm::RenderWidth::kBeside
+                                              : cm::RenderWidth::kBesideSmall;
+            if (after_leaves) {
+                e = cudaStreamWaitEvent(ctx->side, ctx->leaves_end, 0);
+                if (e != cudaSuccess) return join(cuda_fail(e, "side stream ordering"));
+            }
+            st = launch_slots(ctx, spec_slots, L, H, d, ctx->side, 0, nullptr, &width);
             if (st != CM_OK) return join(st);
         }
     }

@@ -67,10 +67,12 @@ struct RenderParams {
 //   kBeside       the TMA kernel, one CTA of 4 warps (6 stages each) per SM: a large render
 //                 beside the leaf hash of the same merge (cm_ingest_render)
 //   kBesideSmall  the register kernel, one 8-warp CTA per SM: a small render beside the leaf hash
+//   kAfterLeaves  the register kernel, two 8-warp CTAs per SM: a middling render that starts as
+//                 the leaf hash ends and leaves the tree levels room on every SM
 // A launch group's work items are row chunks of render_item_bytes(w) bytes of one source
 // plane; render_grid gives the launch's CTA count for `chunks` items. render_prepare() once
 // per device before the first launch.
-enum class RenderWidth { kFull, kHalf, kBeside, kBesideSmall };
+enum class RenderWidth { kFull, kHalf, kBeside, kBesideSmall, kAfterLeaves };
 cudaError_t launch_render(const RenderParams &p, int grid, RenderWidth w, cudaStream_t stream);
 cudaError_t render_prepare();
 uint32_t render_item_bytes(RenderWidth w);

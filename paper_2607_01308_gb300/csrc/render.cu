@@ -23,7 +23,7 @@
 // second half: 8 (x, y) pairs that share the lane's 8 (cos, sin) values. A render that
 // runs beside the content address (cm_ingest_render) takes a narrower width still: the
 // TMA kernel with one CTA of 4 warps and 6 stages per SM for large renders, the register
-// kernel with one 8-warp CTA per SM for small ones (see RenderWidth).
+// kernel with one or two 8-warp CTAs per SM for smaller ones (see RenderWidth).
 //
 // Rounding. The result must equal round-to-nearest-even-bf16 of
 // fl64(fl64(x c) - fl64(y s)) (and fl64(fl64(y c) + fl64(x s))), c and s the fp64
@@ -926,7 +926,9 @@ int render_grid(uint64_t chunks, int num_sms, RenderWidth w) {
     if (w == RenderWidth::kHalf || w == RenderWidth::kBeside)
         return (int)std::max<uint64_t>(1, std::min<uint64_t>(chunks, (uint64_t)num_sms));
     const uint64_t ctas = (chunks / 2 + kRegThreads / 32 - 1) / (kRegThreads / 32);
-    const uint64_t per_sm = w == RenderWidth::kFull ? (uint64_t)kRegBlocksPerSm : 1;
+    const uint64_t per_sm = w == RenderWidth::kFull           ? (uint64_t)kRegBlocksPerSm
+                            : w == RenderWidth::kAfterLeaves ? 2
+                                                             : 1;
     return (int)std::max<uint64_t>(1, std::min<uint64_t>(ctas, per_sm * num_sms));
 }
 
@@ -945,7 +947,7 @@ cudaError_t launch_render(const RenderParams &p, int grid, RenderWidth w, cudaSt
             else
                 render_kernel<false, 4, 6, 4><<<grid, 4 * 32, dyn_smem<4, 6>(), stream>>>(p);
             break;
-        default:   // kFull, kBesideSmall: the register kernel (grid sizes differ)
+        default:   // kFull, kBesideSmall, kAfterLeaves: the register kernel (grid sizes differ)
             if (p.paged)
                 render_reg_kernel<true><<<grid, kRegThreads, 0, stream>>>(p);
             else

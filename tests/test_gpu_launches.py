@@ -1,0 +1,92 @@
+"""The edges of the content address's launches: heads per norm-key thread, tree levels at the
+edge of a warp (whose lanes hand digests to their parents) with several fragments in one
+launch, and the sizes at which cm_ingest_render starts its render beside the leaf hash, as
+the leaves end, or beside it again. Ids and norm keys equal the oracle's; the merges' bytes
+equal those of the separate calls."""
+import numpy as np
+import pytest
+import torch
+
+from parity_util import THETA, empty_out, oracle_fragment
+
+pytestmark = pytest.mark.gpu
+
+cm = pytest.importorskip("paper_2607_01308_gb300")
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    c = cm.Context(0, THETA)
+    yield c
+    c.close()
+
+
+def _fragment(seed, L, H, T, d):
+    g = torch.Generator(device="cuda:0").manual_seed(seed)
+    shape = (L, H, T, d)
+    return tuple((torch.randn(shape, generator=g, device="cuda:0") * s).to(torch.bfloat16)
+                 for s in (0.7 + 0.01 * (seed % 50), 1.0))
+
+
+# 128 threads to a norm block: H < 32 gives 128 // H tokens of H threads, more heads loop
+@pytest.mark.parametrize("H,T", [(1, 127), (1, 129), (3, 42), (3, 43), (12, 10), (12, 11),
+                                 (31, 5), (32, 4), (33, 9), (70, 3)])
+def test_norm_key_over_head_counts(ctx, H, T):
+    K, V = _fragment(H * 100 + T, 2, H, T, 16)
+    fid, Q = ctx.fragment_id(K, V)
+    ref = oracle_fragment(K, V)
+    assert fid == ref.fid and np.array_equal(np.array(Q, dtype=np.uint64), ref.Q)
+    # the allocation-free call takes the same launches
+    out = torch.zeros(16, dtype=torch.uint8, device="cuda:0")
+    key = torch.full((T,), -1, dtype=torch.int64, device="cuda:0")
+    cm.cm_fragment_id_static(cm.fragment_from_tensors(K, V), out.data_ptr(), key.data_ptr())
+    torch.cuda.synchronize()
+    assert bytes(out.cpu().numpy()) == ref.fid
+    assert np.array_equal(key.cpu().numpy().view(np.uint64), ref.Q)
+
+
+# a token is 1 KiB = one leaf here, so T tokens have ceil(T / 16) level-1 nodes
+@pytest.mark.parametrize("lengths", [(1, 16, 17), (256, 257, 255), (511, 512, 513),
+                                     (8191, 1, 8193), (4096, 4097, 300)])
+def test_tree_levels_at_warp_edges(ctx, lengths):
+    frags = [_fragment(7 * T + i, 1, 1, T, 256) for i, T in enumerate(lengths)]
+    S = cm.FragmentSet(ctx)
+    res = S.ingest_batch(frags)
+    assert [fid for fid, _ in res] == [oracle_fragment(K, V).fid for K, V in frags]
+    S.close()
+
+
+# 114,688 bytes a token: 1,216 leaf blocks (one partial wave) up to about 1,389 tokens;
+# 512 MiB at 4,681 tokens
+@pytest.mark.parametrize("lengths,prior", [((690, 690), 0), ((700, 705), 0), ((1500, 1500, 1600), 0),
+                                           ((1500, 1500, 1700), 0), ((800, 810), 400), ((800, 810), 3100)])
+def test_ingest_render_start_rules_give_the_separate_calls_bytes(ctx, lengths, prior):
+    frags = [_fragment(31 * T + i, 28, 8, T, 128) for i, T in enumerate(lengths)]
+    old = [_fragment(5, 28, 8, prior, 128)] if prior else []
+    total = sum(lengths) + prior
+    half = (len(frags) + 1) // 2
+    outs = []
+    for fused in (True, False):
+        A, B = cm.FragmentSet(ctx), cm.FragmentSet(ctx)
+        if old:
+            A.ingest_batch(old)
+        k, v = empty_out(28, 8, total, 128, fill=0x3C3C)
+        where = [A.handle] * half + [B.handle] * (len(frags) - half)
+        fd = [cm.fragment_from_tensors(K, V) for K, V in frags]
+        if fused:
+            _, n, order, overlapped = cm.cm_ingest_render(where, fd, A.handle, k.data_ptr(),
+                                                          v.data_ptr(), total)
+            assert overlapped
+        else:
+            cm.cm_ingest_many(where, fd)
+            A.union(B)
+            n, order = A.render(k, v)
+        torch.cuda.synchronize()
+        assert n == total
+        outs.append((order, k.view(torch.int16), v.view(torch.int16)))
+        A.close()
+        B.close()
+    assert outs[0][0] == outs[1][0]
+    assert torch.equal(outs[0][1], outs[1][1]) and torch.equal(outs[0][2], outs[1][2])
