@@ -248,9 +248,10 @@ cm_status cm_render(const cm_set *set, void *k_out, void *v_out, int64_t capacit
  * pairwise distinct, the canonical order of Algorithm 1 does not depend on the ids: the
  * render starts on a stream of the context, with narrow CTAs, while the content address
  * runs on `stream`: at once, or (middling sizes) as its first level ends. When the ids are
- * known the set is checked to hold exactly the fragments rendered, in that order (different fragments taken for one, or sharing
- * an address, which the paper's collision assumption excludes, fail the check; then the
- * target is rendered again after the first render, so the result is still exact). With
+ * known the set is checked to hold exactly the fragments rendered, in that order (different
+ * fragments taken for one, or sharing an address, which the paper's collision assumption
+ * excludes, fail the check; then the target is rendered again after the first render, so the
+ * result is still exact). With
  * a tie of S between members that differ in length or norm keys, with the re-delivery
  * fast path on, or with an output the render would refuse, the steps run one after the
  * other.

@@ -245,8 +245,8 @@ __device__ __forceinline__ void norm_block(const LeafLaunch &a, uint32_t block) 
 }
 
 // Cursor over the fragment's byte stream K[0] V[0] K[1] V[1] ...: every segment
-// (one layer of K or of V) is plane_bytes long, a multiple of 32, so a 16-byte
-// vector never straddles two segments.
+// (one layer of K or of V) is plane_bytes long, a multiple of 32, so 32 bytes of the stream
+// from a multiple of 32 never straddle two segments.
 struct StreamCursor {
     const uint8_t *ptr;
     uint64_t left;       // bytes left in the current segment
@@ -266,20 +266,17 @@ __device__ __forceinline__ StreamCursor cursor_at(const LeafLaunch &a, uint64_t 
     return c;
 }
 
+// The next 32 bytes.
 __device__ __forceinline__ const uint8_t *cursor_next(const LeafLaunch &a, StreamCursor &c) {
     if (c.left == 0) {
-        if (c.in_v) {
-            c.in_v = false;
-            ++c.layer;
-        } else {
-            c.in_v = true;
-        }
+        if (c.in_v) ++c.layer;
+        c.in_v = !c.in_v;
         c.ptr = (c.in_v ? a.v : a.k) + (uint64_t)c.layer * a.plane_bytes;
         c.left = a.plane_bytes;
     }
     const uint8_t *p = c.ptr;
-    c.ptr += 16;
-    c.left -= 16;
+    c.ptr += 32;
+    c.left -= 32;
     return p;
 }
 
@@ -296,7 +293,12 @@ __device__ __forceinline__ void allow_next_launch() {
 
 constexpr int kLeafThreads = kLeafBlockThreads;
 
-template <uint32_t kFmaMask>
+// kWhole: every plane of the group is a multiple of a leaf, so each leaf is 1 KiB of one
+// segment. Otherwise a leaf may run into the next segments and a fragment's last leaf may be
+// short (a multiple of 64 bytes, as 2 L planes are): every leaf then walks its blocks in
+// halves of 32 bytes, one loop for all, so that a warp never hashes its straddling leaves
+// after the others (as it once did: the tiny merge's leaves took 42 us, now 21).
+template <uint32_t kFmaMask, bool kWhole>
 __global__ void __launch_bounds__(kLeafThreads)
 leaf_hash_kernel(const __grid_constant__ LeafGroup grp) {
     // the blocks after the leaf blocks, one per fragment, zero its tree levels' arrival counters
@@ -317,47 +319,33 @@ leaf_hash_kernel(const __grid_constant__ LeafGroup grp) {
     const uint64_t leaf = (uint64_t)(x - grp.block_begin[fi]) * kLeafThreads + threadIdx.x;
     if (leaf >= a.num_leaves) return;
     const uint64_t begin = leaf * kLeafBytes;
-    const uint64_t rem = a.stream_bytes - begin;
-    const uint32_t len = rem < (uint64_t)kLeafBytes ? (uint32_t)rem : (uint32_t)kLeafBytes;
-    const uint32_t nblocks = (len + 63) / 64;
     const bool last_node = leaf + 1 == a.num_leaves;
-
     uint32_t h[8];
     node_init(h, a.tree, leaf, 0);
     StreamCursor cur = cursor_at(a, begin);
-
-    if (len == (uint32_t)kLeafBytes && cur.left >= (uint64_t)kLeafBytes) {
-        // the whole leaf lies in one K or V segment
+    if (kWhole) {
         const uint8_t *p = cur.ptr;
         if (!in_fragment(a, p, kLeafBytes)) return;
 #pragma unroll 1
-        for (uint32_t b = 0; b < 16; ++b) {
-            const uint4 w0 = load_nc(p + 64 * b), w1 = load_nc(p + 64 * b + 16),
-                        w2 = load_nc(p + 64 * b + 32), w3 = load_nc(p + 64 * b + 48);
+        for (uint32_t at = 0; at < (uint32_t)kLeafBytes; at += 64) {
+            const uint4 w0 = load_nc(p + at), w1 = load_nc(p + at + 16), w2 = load_nc(p + at + 32),
+                        w3 = load_nc(p + at + 48);
             const uint32_t m[16] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w,
                                     w2.x, w2.y, w2.z, w2.w, w3.x, w3.y, w3.z, w3.w};
-            compress<kFmaMask>(h, m, (b + 1) * 64, b == 15, last_node);
+            compress<kFmaMask>(h, m, at + 64, at + 64 == (uint32_t)kLeafBytes, last_node);
         }
-        if (CM_IN_BOUNDS(a.digests + leaf * kDigestBytes, kDigestBytes, a.digests,
-                         a.num_leaves * kDigestBytes))
-            store_digest(a.digests + leaf * kDigestBytes, h);
-        return;
-    }
-
-    for (uint32_t b = 0; b < nblocks; ++b) {
-        uint4 w[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            w[q] = make_uint4(0, 0, 0, 0);
-            if (b * 64 + q * 16 < len) {
-                const uint8_t *ptr = cursor_next(a, cur);
-                if (in_fragment(a, ptr, 16)) w[q] = load_nc(ptr);
-            }
+    } else {
+        const uint64_t rem = a.stream_bytes - begin;
+        const uint32_t nblocks = rem < (uint64_t)kLeafBytes ? (uint32_t)rem / 64 : (uint32_t)kLeafBytes / 64;
+#pragma unroll 1
+        for (uint32_t b = 0; b < nblocks; ++b) {
+            const uint8_t *p = cursor_next(a, cur), *q = cursor_next(a, cur);
+            if (!in_fragment(a, p, 32) || !in_fragment(a, q, 32)) return;
+            const uint4 w0 = load_nc(p), w1 = load_nc(p + 16), w2 = load_nc(q), w3 = load_nc(q + 16);
+            const uint32_t m[16] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w,
+                                    w2.x, w2.y, w2.z, w2.w, w3.x, w3.y, w3.z, w3.w};
+            compress<kFmaMask>(h, m, (b + 1) * 64, b + 1 == nblocks, last_node);
         }
-        const uint32_t m[16] = {w[0].x, w[0].y, w[0].z, w[0].w, w[1].x, w[1].y, w[1].z, w[1].w,
-                                w[2].x, w[2].y, w[2].z, w[2].w, w[3].x, w[3].y, w[3].z, w[3].w};
-        const uint32_t end = (b + 1) * 64 < len ? (b + 1) * 64 : len;
-        compress<kFmaMask>(h, m, end, b + 1 == nblocks, last_node);
     }
     if (CM_IN_BOUNDS(a.digests + leaf * kDigestBytes, kDigestBytes, a.digests,
                      a.num_leaves * kDigestBytes))
@@ -555,7 +543,7 @@ CM_DEFINE_BOUNDS_READER(take_hash_bounds_violations)
 
 int leaf_hash_blocks_per_sm() {
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, leaf_hash_kernel<kIssueBound>, kLeafThreads, 0) != cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, leaf_hash_kernel<kIssueBound, true>, kLeafThreads, 0) != cudaSuccess)
         return 0;
     return n;
 }
@@ -588,16 +576,17 @@ cudaError_t launch_leaf_hash_group(const LeafGroup &g, LeafMode mode, int num_sm
     if (g.count == 0) return cudaSuccess;
     const uint64_t blocks = g.block_begin[g.count] + g.count;   // leaves, then arrival counters
     if (blocks > 0x7FFFFFFFull) return cudaErrorInvalidValue;
+    bool whole = true;
+    for (uint32_t i = 0; i < g.count; ++i) whole = whole && g.frag[i].plane_bytes % kLeafBytes == 0;
+    void (*const alone)(LeafGroup) = whole ? leaf_hash_kernel<kIssueBound, true> : leaf_hash_kernel<kIssueBound, false>;
     if (mode != LeafMode::kWithNorms) {
-        if (mode == LeafMode::kBesideRender)
-            leaf_hash_kernel<kBesideRender><<<(unsigned)blocks, kLeafThreads, 0, stream>>>(g);
-        else
-            leaf_hash_kernel<kIssueBound><<<(unsigned)blocks, kLeafThreads, 0, stream>>>(g);
+        void (*const beside)(LeafGroup) =
+            whole ? leaf_hash_kernel<kBesideRender, true> : leaf_hash_kernel<kBesideRender, false>;
+        (mode == LeafMode::kBesideRender ? beside : alone)<<<(unsigned)blocks, kLeafThreads, 0, stream>>>(g);
         return cudaGetLastError();
     }
     const cudaError_t e = launch_norm_keys(g, (uint64_t)num_sms, stream);
-    if (e != cudaSuccess) return e;
-    return launch_after(leaf_hash_kernel<kIssueBound>, blocks, kLeafThreads, stream, g);
+    return e != cudaSuccess ? e : launch_after(alone, blocks, kLeafThreads, stream, g);
 }
 
 cudaError_t launch_norm_keys(const LeafGroup &in, uint64_t max_blocks, cudaStream_t stream) {

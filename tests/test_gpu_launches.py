@@ -90,3 +90,21 @@ def test_ingest_render_start_rules_give_the_separate_calls_bytes(ctx, lengths, p
         B.close()
     assert outs[0][0] == outs[1][0]
     assert torch.equal(outs[0][1], outs[1][1]) and torch.equal(outs[0][2], outs[1][2])
+
+
+# planes that are no multiple of a 1 KiB leaf: leaves that run into one or many further
+# segments, short last leaves, alone and in one launch with whole ones
+@pytest.mark.parametrize("shape", [(2, 1, 1, 16), (40, 1, 1, 16), (9, 1, 3, 32), (3, 3, 11, 16),
+                                   (4, 2, 37, 64), (5, 1, 63, 128), (6, 3, 5, 512)])
+def test_leaves_that_straddle_segments(ctx, shape):
+    L, H, T, d = shape
+    K, V = _fragment(sum(shape), L, H, T, d)
+    whole = _fragment(3, L, H, 1024, d)   # 1024 rows to a head: every plane whole leaves
+    S = cm.FragmentSet(ctx)
+    res = S.ingest_batch([(K, V)])
+    assert res[0][0] == oracle_fragment(K, V).fid
+    both = cm.FragmentSet(ctx)
+    res = both.ingest_batch([whole, (K, V)])
+    assert [fid for fid, _ in res] == [oracle_fragment(*whole).fid, oracle_fragment(K, V).fid]
+    S.close()
+    both.close()
