@@ -156,19 +156,50 @@ def _check(status: int) -> None:
         raise CMError(status, cm_last_error_message())
 
 
+def _torch_current_stream():
+    """The current torch stream's handle; bound to a cheaper lookup once torch has a device."""
+    global _torch_current_stream
+    try:
+        import torch
+    except ImportError:
+        return 0
+    if not torch.cuda.is_available():
+        return 0
+    device, raw = torch.cuda.current_device, getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        _torch_current_stream = lambda: torch.cuda.current_stream().cuda_stream   # noqa: E731
+    else:
+        _torch_current_stream = lambda: raw(device())   # noqa: E731
+    return _torch_current_stream()
+
+
 def _stream_handle(stream) -> Optional[int]:
     """None -> torch's current stream if torch is loaded with CUDA, else the legacy default."""
     if stream is None:
-        try:
-            import torch
-            if torch.cuda.is_available():
-                return torch.cuda.current_stream().cuda_stream or None
-        except ImportError:
-            pass
-        return None
+        return _torch_current_stream() or None
     if isinstance(stream, int):
         return stream or None
     return stream.cuda_stream or None
+
+
+def _id_list(ids, n: int) -> List[bytes]:
+    """The first n entries of a cm_id array."""
+    raw = bytes(ids)
+    return [raw[i:i + 16] for i in range(0, 16 * n, 16)]
+
+
+def _id_array(ids: Sequence[bytes]):
+    """A cm_id array of at least one entry holding `ids` (16 bytes each)."""
+    arr = (cm_id * max(len(ids), 1))()
+    for i, fid in enumerate(ids):
+        if len(fid) != 16:
+            raise ValueError("an id has 16 bytes")
+        ctypes.memmove(ctypes.byref(arr, 16 * i), bytes(fid), 16)
+    return arr
+
+
+def _deliveries(ids, absorbed, n: int) -> List[Tuple[bytes, bool]]:
+    return [(fid, flag != 0) for fid, flag in zip(_id_list(ids, n), absorbed)]
 
 
 def cm_context_create(device: int = 0, rope_theta: float = 1.0e6, routing_layer: int = -1,
@@ -235,7 +266,7 @@ def cm_ingest_batch(s: int, frags: Sequence[cm_fragment], stream=None) -> List[T
     ids = (cm_id * max(n, 1))()
     absorbed = (ctypes.c_int32 * max(n, 1))()
     _check(lib.cm_ingest_batch(s, arr, n, _stream_handle(stream), ids, absorbed))
-    return [(ids[i].to_bytes(), bool(absorbed[i])) for i in range(n)]
+    return _deliveries(ids, absorbed, n)
 
 
 def cm_ingest_many(sets: Sequence[int], frags: Sequence[cm_fragment],
@@ -248,7 +279,7 @@ def cm_ingest_many(sets: Sequence[int], frags: Sequence[cm_fragment],
     ids = (cm_id * max(n, 1))()
     absorbed = (ctypes.c_int32 * max(n, 1))()
     _check(lib.cm_ingest_many(set_arr, arr, n, _stream_handle(stream), ids, absorbed))
-    return [(ids[i].to_bytes(), bool(absorbed[i])) for i in range(n)]
+    return _deliveries(ids, absorbed, n)
 
 
 def cm_ingest_render(sets: Sequence[int], frags: Sequence[cm_fragment], target: int, k_out: int,
@@ -275,8 +306,7 @@ def cm_ingest_render(sets: Sequence[int], frags: Sequence[cm_fragment], target: 
                                 _stream_handle(stream), ids, absorbed, ctypes.byref(seq), order,
                                 ctypes.byref(ovl)))
     size = cm_set_size(target)
-    return ([(ids[i].to_bytes(), bool(absorbed[i])) for i in range(n)], seq.value,
-            [order[i].to_bytes() for i in range(size)], bool(ovl.value))
+    return _deliveries(ids, absorbed, n), seq.value, _id_list(order, size), bool(ovl.value)
 
 
 def cm_render_many(jobs: Sequence[cm_render_job], stream=None) -> List[int]:
@@ -289,9 +319,7 @@ def cm_render_many(jobs: Sequence[cm_render_job], stream=None) -> List[int]:
 
 def cm_set_contains(s: int, ids: Sequence[bytes]) -> List[bool]:
     n = len(ids)
-    arr = (cm_id * max(n, 1))()
-    for i, fid in enumerate(ids):
-        arr[i].b[:] = list(fid)
+    arr = _id_array(ids)
     out = (ctypes.c_uint8 * max(n, 1))()
     _check(lib.cm_set_contains(s, arr, n, out))
     return [bool(out[i]) for i in range(n)]
@@ -352,7 +380,7 @@ def cm_set_ids(s: int) -> List[bytes]:
     n = cm_set_size(s)
     arr = (cm_id * max(n, 1))()
     _check(lib.cm_set_ids(s, arr, n))
-    return [arr[i].to_bytes() for i in range(n)]
+    return _id_list(arr, n)
 
 
 def cm_render(s: int, k_out: int, v_out: int, capacity_tokens: int,
@@ -367,22 +395,20 @@ def cm_render(s: int, k_out: int, v_out: int, capacity_tokens: int,
     order = (cm_id * max(n, 1))()
     _check(lib.cm_render(s, k_out, v_out, capacity_tokens, _stream_handle(stream),
                          ctypes.byref(seq), order))
-    return seq.value, [order[i].to_bytes() for i in range(n)]
+    return seq.value, _id_list(order, n)
 
 
 def cm_render_incremental(s: int, k_out: int, v_out: int, capacity_tokens: int,
                           prev_order: Sequence[bytes], stream=None) -> Tuple[int, List[bytes], int]:
     n = cm_set_size(s)
     order = (cm_id * max(n, 1))()
-    prev = (cm_id * max(len(prev_order), 1))()
-    for i, fid in enumerate(prev_order):
-        prev[i].b[:] = list(fid)
+    prev = _id_array(prev_order)
     seq = ctypes.c_int64()
     reused = ctypes.c_int64()
     _check(lib.cm_render_incremental(s, k_out, v_out, capacity_tokens, prev, len(prev_order),
                                      _stream_handle(stream), ctypes.byref(seq), order,
                                      ctypes.byref(reused)))
-    return seq.value, [order[i].to_bytes() for i in range(n)], reused.value
+    return seq.value, _id_list(order, n), reused.value
 
 
 def cm_render_paged(s: int, cache: cm_paged_cache, stream=None) -> Tuple[int, List[bytes]]:
@@ -391,7 +417,7 @@ def cm_render_paged(s: int, cache: cm_paged_cache, stream=None) -> Tuple[int, Li
     seq = ctypes.c_int64()
     _check(lib.cm_render_paged(s, ctypes.byref(cache), _stream_handle(stream), ctypes.byref(seq),
                                order))
-    return seq.value, [order[i].to_bytes() for i in range(n)]
+    return seq.value, _id_list(order, n)
 
 
 def cm_bagmerge(ctx: int, frags: Sequence[cm_fragment], k_out: int, v_out: int,
@@ -408,12 +434,13 @@ def cm_bagmerge(ctx: int, frags: Sequence[cm_fragment], k_out: int, v_out: int,
 def fragment_from_tensors(K, V) -> cm_fragment:
     """Descriptor of a fragment held in two bf16 CUDA tensors [L, H, T, d] (contiguous)."""
     import torch
-    if K.shape != V.shape or K.dim() != 4:
+    shape = K.shape
+    if shape != V.shape or len(shape) != 4:
         raise ValueError("K and V must both be [layers, kv_heads, seq_len, head_dim]")
     for t in (K, V):
         if t.dtype != torch.bfloat16 or not t.is_cuda or not t.is_contiguous():
             raise ValueError("K and V must be contiguous bf16 CUDA tensors")
-    L, H, T, d = K.shape
+    L, H, T, d = shape
     return cm_fragment(L, H, T, d, K.data_ptr(), V.data_ptr())
 
 
