@@ -368,10 +368,10 @@ cm_status cm_context_check(cm_context *ctx, cm_stream_t stream);
  * pointers count as equal without reading them). A delivery found equal takes that
  * fragment's id and norm key and is not hashed; the others are hashed as usual. Results
  * (ids, absorption, the set) are identical with the path on or off. The candidates'
- * first 4 KiB are compared first; only the first candidate whose prefix matches is then
- * compared in full, reading both fragments at HBM speed. This costs one more stream
- * synchronisation per call that has candidates (two if a prefix matches): turn it on
- * where re-deliveries are common (gossip, retries). The paper has no counterpart. */
+ * first 4 KiB are compared first; then each delivery with one candidate whose prefix
+ * matched, in full, at HBM speed and beside the hashing of the others. This costs one more
+ * stream synchronisation per call that has candidates (two if a matching prefix misled):
+ * turn it on where re-deliveries are common (gossip, retries). The paper has no counterpart. */
 cm_status cm_context_set_dedup_by_bytes(cm_context *ctx, int32_t enable);
 
 /* Whether cm_ingest_render may run its render beside the content address (a scheduling

@@ -9,30 +9,48 @@
 
 namespace cm {
 
-constexpr int kMaxComparePairs = 128;         // pairs per launch
+constexpr int kMaxComparePairs = 128;         // pairs (members) per launch
 constexpr uint64_t kCompareChunkVecs = 2048;   // 16-byte vectors of each array per chunk
 
-// Two fragments of one shape: the K and V arrays of a delivery (a) and of a candidate (b),
-// each `vecs` 16-byte vectors long. All four pointers are 16-byte aligned.
+// Two fragments of one shape, told apart by their K arrays' first 4 KiB: `vecs` 16-byte
+// vectors long. All pointers below are 16-byte aligned.
 struct ComparePair {
-    const uint4 *a_k, *a_v, *b_k, *b_v;
+    const uint4 *a_k, *b_k;
     uint64_t vecs;
 };
-
-struct CompareLaunch {
+struct ComparePrefix {
     uint32_t count;                               // pairs, <= kMaxComparePairs
     uint32_t pad_;
-    // prefix sums of the pairs' chunk counts: 2 ceil(vecs / kCompareChunkVecs) per pair
-    uint64_t chunk_begin[kMaxComparePairs + 1];
     ComparePair pair[kMaxComparePairs];
-    uint32_t *differ;                             // device, one word per pair, zeroed before
+    uint32_t *differ;                             // one word per pair; may be mapped host memory
 };
 
-// differ[p] |= 1 if the first 4 KiB of the pair's K arrays differ (one block per pair).
-cudaError_t launch_compare_prefix(const CompareLaunch &c, cudaStream_t stream);
+// Deliveries (members) that may equal one candidate (the group's base): each group's K and V
+// arrays are `vecs` 16-byte vectors long.
+struct CompareMember {
+    const uint4 *k, *v;
+};
+struct CompareGroup {
+    const uint4 *k, *v;                           // the base
+    uint64_t vecs;
+    uint32_t begin, end;                          // its members
+};
+struct CompareFull {
+    uint32_t groups;                              // <= members <= kMaxComparePairs
+    uint32_t pad_;
+    // prefix sums of the groups' chunk counts: 2 ceil(vecs / kCompareChunkVecs) per group
+    uint64_t chunk_begin[kMaxComparePairs + 1];
+    CompareGroup group[kMaxComparePairs];
+    CompareMember member[kMaxComparePairs];
+    uint32_t *differ;                             // device, one word per member, zeroed before
+};
 
-// differ[p] |= 1 if the pair's K or V arrays differ anywhere (a persistent grid over all
-// chunks of all pairs; the chunks of a pair already found to differ are skipped).
-cudaError_t launch_compare_full(const CompareLaunch &c, int num_sms, cudaStream_t stream);
+// differ[p] = 1 if the first 4 KiB of pair p's K arrays differ, else 0 (one block per pair).
+cudaError_t launch_compare_prefix(const ComparePrefix &c, cudaStream_t stream);
+
+// differ[m] |= 1 if member m's K or V array differs from its group's base anywhere (a
+// persistent grid of blocks_per_sm blocks per SM over all chunks of all groups; a member
+// already found to differ is skipped).
+cudaError_t launch_compare_full(const CompareFull &c, int num_sms, int blocks_per_sm, cudaStream_t stream);
 
 }  // namespace cm

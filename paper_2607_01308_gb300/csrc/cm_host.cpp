@@ -16,12 +16,14 @@
 #include <cstdio>
 #include <cstddef>
 #include <cstring>
+#include <functional>
 #include <map>
 #include <memory>
 #include <mutex>
 #include <new>
 #include <string>
 #include <unordered_map>
+#include <utility>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -217,16 +219,16 @@ cm_status ensure_scratch(cm_context *ctx, size_t dev_bytes, size_t host_bytes) {
     return CM_OK;
 }
 
-// Reads a small device result (`bytes` at `src`) into ctx->h_pinned, enqueued on `stream`:
-// stored by the SMs through the buffer's mapped address when everything is 4-byte granular
-// (so the read does not wait behind bulk device-to-host copies of other streams on the copy
-// engine), else by a copy.
-cudaError_t read_small(cm_context *ctx, const void *src, size_t bytes, cudaStream_t stream) {
-    if (ctx->h_pinned_dev && bytes % 4 == 0 && (reinterpret_cast<uintptr_t>(src) & 3u) == 0) {
+// Reads a small device result (`bytes` at `src`) into ctx->h_pinned + host_off, enqueued on
+// `stream`: stored by the SMs through the buffer's mapped address when everything is 4-byte
+// granular (so the read does not wait behind bulk device-to-host copies of other streams on
+// the copy engine), else by a copy.
+cudaError_t read_small(cm_context *ctx, size_t host_off, const void *src, size_t bytes, cudaStream_t stream) {
+    if (ctx->h_pinned_dev && bytes % 4 == 0 && host_off % 4 == 0 && (reinterpret_cast<uintptr_t>(src) & 3u) == 0) {
         if (ctx->timing) ++ctx->aux_launches;
-        return cm::launch_readback(ctx->h_pinned_dev, src, bytes, stream);
+        return cm::launch_readback(static_cast<uint8_t *>(ctx->h_pinned_dev) + host_off, src, bytes, stream);
     }
-    return cudaMemcpyAsync(ctx->h_pinned, src, bytes, cudaMemcpyDeviceToHost, stream);
+    return cudaMemcpyAsync(ctx->h_pinned + host_off, src, bytes, cudaMemcpyDeviceToHost, stream);
 }
 
 // BLAKE2s parameter block (32 bytes) of the tree, node offset and depth zero,
@@ -262,6 +264,11 @@ cm::TreeParams tree_params(int32_t L, int32_t H, int32_t d, int32_t T) {
 }
 
 uint64_t ceil_div(uint64_t a, uint64_t b) { return (a + b - 1) / b; }
+
+// 16-byte vectors of a fragment's K (= of its V).
+uint64_t plane_vecs(const cm_fragment *f) {
+    return (uint64_t)f->num_layers * f->num_kv_heads * f->seq_len * f->head_dim * 2 / 16;
+}
 
 enum { kTimeLeaf = 0, kTimeInner = 1, kTimeRender = 2 };
 
@@ -498,7 +505,7 @@ cm_status enqueue_norm_keys(cm_context *ctx, const cm_fragment *const *frags, si
 cm_status take_device_error(cm_context *ctx, cudaStream_t stream) {
     cm_status st = ensure_scratch(ctx, 0, 16);
     if (st != CM_OK) return st;
-    CM_CUDA_TRY(read_small(ctx, ctx->d_error, sizeof(unsigned int), stream),
+    CM_CUDA_TRY(read_small(ctx, 0, ctx->d_error, sizeof(unsigned int), stream),
                 "error word copy");
     CM_CUDA_TRY(cudaStreamSynchronize(stream), "error word synchronisation");
     unsigned int e;
@@ -524,7 +531,7 @@ cm_status bytes_equal(cm_context *ctx, const cm_fragment *f, const Record &r, cu
     CM_CUDA_TRY(cudaMemsetAsync(flag, 0, sizeof(unsigned int), stream), "flag reset");
     CM_CUDA_TRY(cm::launch_compare(f->k, r.k, bytes, flag, stream), "compare launch");
     CM_CUDA_TRY(cm::launch_compare(f->v, r.v, bytes, flag, stream), "compare launch");
-    CM_CUDA_TRY(read_small(ctx, flag, sizeof(unsigned int), stream),
+    CM_CUDA_TRY(read_small(ctx, 0, flag, sizeof(unsigned int), stream),
                 "flag copy");
     CM_CUDA_TRY(cudaStreamSynchronize(stream), "compare synchronisation");
     unsigned int h;
@@ -708,25 +715,29 @@ cm_status guarded(F &&f) {
 // a fragment their set already holds or to an earlier delivery of the call. A
 // delivery is compared with at most kMaxCandidates fragments of its shape and length
 // (the set's records first, then the call's earlier deliveries, the latest first):
-// their first 4 KiB in one pass, then all bytes of the first candidate whose prefix
-// matched; identical (k, v) pointers count as equal without a comparison. Results:
-// rec[i] is the equal record, else from[i] the equal earlier delivery, else neither
-// (hash it).
+// their first 4 KiB in one pass, then all bytes of one candidate whose prefix
+// matched; identical (k, v) pointers count as equal without a comparison.
 constexpr int kMaxCandidates = 16;
 
-cm_status find_redeliveries(cm_context *ctx, cm_set *const *sets,
-                            const std::vector<const cm_fragment *> &fp, cudaStream_t stream,
-                            std::vector<std::shared_ptr<const Record>> &rec,
-                            std::vector<int32_t> &from) {
+struct Candidate {
+    size_t delivery;
+    std::shared_ptr<const Record> r;   // a record, or null for delivery `other`
+    size_t other;
+};
+
+// The first pass (synchronising `stream` if there is anything to compare): rec[i] / from[i]
+// for identical pointers; `chosen` gets, for each delivery with a candidate whose prefix
+// matched, the first such record or else the earliest such delivery (one full comparison
+// suffices, and copies of one fragment are then all compared with the same one).
+cm_status match_prefixes(cm_context *ctx, cm_set *const *sets,
+                         const std::vector<const cm_fragment *> &fp, cudaStream_t stream,
+                         std::vector<std::shared_ptr<const Record>> &rec,
+                         std::vector<int32_t> &from, std::vector<Candidate> &chosen) {
     const size_t n = fp.size();
     rec.assign(n, nullptr);
     from.assign(n, -1);
-    struct Cand {
-        size_t delivery;
-        std::shared_ptr<const Record> r;   // a record, or null for delivery `other`
-        size_t other;
-    };
-    std::vector<Cand> cands;
+    chosen.clear();
+    std::vector<Candidate> cands;
     auto same_shape = [](const cm_fragment *f, int32_t L, int32_t H, int32_t T, int32_t d) {
         return f->num_layers == L && f->num_kv_heads == H && f->seq_len == T && f->head_dim == d;
     };
@@ -764,71 +775,78 @@ cm_status find_redeliveries(cm_context *ctx, cm_set *const *sets,
             while (!cands.empty() && cands.back().delivery == i) cands.pop_back();
     }
     if (cands.empty()) return CM_OK;
-    // one comparison pass over a list of candidate pairs: differ[c] = 1 if pair c differs
-    // (its first 4 KiB of K only, or all of it)
-    auto compare = [&](const std::vector<size_t> &which, bool full,
-                       std::vector<uint32_t> &differ) -> cm_status {
-        differ.assign(which.size(), 1u);
-        cm_status st = ensure_scratch(ctx, which.size() * 4, which.size() * 4);
-        if (st != CM_OK) return st;
-        auto *d_differ = reinterpret_cast<uint32_t *>(ctx->d_scratch);
-        CM_CUDA_TRY(cudaMemsetAsync(d_differ, 0, which.size() * 4, stream), "comparison flags reset");
-        for (size_t c0 = 0; c0 < which.size(); c0 += (size_t)cm::kMaxComparePairs) {
-            cm::CompareLaunch cl;
-            std::memset(&cl, 0, sizeof cl);
-            const size_t cn = std::min(which.size() - c0, (size_t)cm::kMaxComparePairs);
-            for (size_t q = 0; q < cn; ++q) {
-                const Cand &c = cands[which[c0 + q]];
-                const cm_fragment *f = fp[c.delivery];
-                const void *bk = c.r ? c.r->k : fp[c.other]->k;
-                const void *bv = c.r ? c.r->v : fp[c.other]->v;
-                const uint64_t vecs =
-                    (uint64_t)f->num_layers * f->num_kv_heads * f->seq_len * f->head_dim * 2 / 16;
-                cl.pair[q] = {static_cast<const uint4 *>(f->k), static_cast<const uint4 *>(f->v),
-                              static_cast<const uint4 *>(bk), static_cast<const uint4 *>(bv), vecs};
-                cl.chunk_begin[q + 1] =
-                    cl.chunk_begin[q] + 2 * ceil_div(vecs, (uint64_t)cm::kCompareChunkVecs);
-            }
-            cl.count = (uint32_t)cn;
-            cl.differ = d_differ + c0;
-            CM_CUDA_TRY(full ? cm::launch_compare_full(cl, ctx->num_sms, stream)
-                             : cm::launch_compare_prefix(cl, stream),
-                        "comparison launch");
-            if (ctx->timing) ++ctx->aux_launches;
+    const size_t bytes = cands.size() * 4;
+    cm_status st = ensure_scratch(ctx, bytes, bytes);
+    if (st != CM_OK) return st;
+    auto *differ = reinterpret_cast<uint32_t *>(ctx->h_pinned_dev ? ctx->h_pinned_dev : ctx->d_scratch);
+    std::unique_ptr<cm::ComparePrefix> cl(new cm::ComparePrefix);
+    for (size_t c0 = 0; c0 < cands.size(); c0 += (size_t)cm::kMaxComparePairs) {
+        const size_t cn = std::min(cands.size() - c0, (size_t)cm::kMaxComparePairs);
+        std::memset(cl.get(), 0, sizeof(cm::ComparePrefix));
+        for (size_t q = 0; q < cn; ++q) {
+            const Candidate &c = cands[c0 + q];
+            const cm_fragment *f = fp[c.delivery];
+            cl->pair[q] = {static_cast<const uint4 *>(f->k),
+                           static_cast<const uint4 *>(c.r ? c.r->k : fp[c.other]->k), plane_vecs(f)};
         }
-        CM_CUDA_TRY(read_small(ctx, d_differ, which.size() * 4, stream),
+        cl->count = (uint32_t)cn;
+        cl->differ = differ + c0;
+        CM_CUDA_TRY(cm::launch_compare_prefix(*cl, stream), "comparison launch");
+        if (ctx->timing) ++ctx->aux_launches;
+    }
+    if (!ctx->h_pinned_dev)
+        CM_CUDA_TRY(cudaMemcpyAsync(ctx->h_pinned, differ, bytes, cudaMemcpyDeviceToHost, stream),
                     "comparison flags copy");
-        CM_CUDA_TRY(cudaStreamSynchronize(stream), "comparison synchronisation");
-        std::memcpy(differ.data(), ctx->h_pinned, which.size() * 4);
-        return CM_OK;
-    };
-    // first the 4 KiB prefixes of every pair, then the whole of one pair per delivery:
-    // its first candidate whose prefix matched (one full comparison suffices, and
-    // re-deliveries of one fragment would otherwise all be compared with each other)
-    std::vector<size_t> all(cands.size());
-    for (size_t c = 0; c < cands.size(); ++c) all[c] = c;
-    std::vector<uint32_t> prefix_differ, full_differ;
-    cm_status st = compare(all, false, prefix_differ);
-    if (st != CM_OK) return st;
-    std::vector<size_t> chosen;
-    std::vector<bool> has_choice(n, false);
+    CM_CUDA_TRY(cudaStreamSynchronize(stream), "comparison synchronisation");
+    const auto *flags = reinterpret_cast<const uint32_t *>(ctx->h_pinned);
     for (size_t c = 0; c < cands.size(); ++c) {
-        const size_t i = cands[c].delivery;
-        if (prefix_differ[c] != 0 || has_choice[i]) continue;
-        has_choice[i] = true;
-        chosen.push_back(c);
+        if (flags[c] != 0) continue;
+        if (chosen.empty() || chosen.back().delivery != cands[c].delivery)
+            chosen.push_back(cands[c]);
+        else if (!chosen.back().r)
+            chosen.back() = cands[c];   // an earlier delivery
     }
-    if (chosen.empty()) return CM_OK;
-    st = compare(chosen, true, full_differ);
-    if (st != CM_OK) return st;
-    for (size_t q = 0; q < chosen.size(); ++q) {
-        if (full_differ[q] != 0) continue;
-        const Cand &c = cands[chosen[q]];
-        if (c.r)
-            rec[c.delivery] = c.r;
-        else
-            from[c.delivery] = (int32_t)c.other;
+    return CM_OK;
+}
+
+// Enqueues the full comparisons of `chosen` on `stream`, one launch per kMaxComparePairs of
+// them, and sorts it by the fragment that each is compared with, so that the copies of one
+// fragment are compared together; their flags (one word each, in device scratch at dev_off) go to the pinned buffer at host_off. Both offsets are
+// multiples of 16 and the scratch already reaches there.
+cm_status enqueue_comparisons(cm_context *ctx, const std::vector<const cm_fragment *> &fp,
+                              std::vector<Candidate> &chosen, cudaStream_t stream,
+                              int blocks_per_sm, size_t dev_off, size_t host_off) {
+    auto base = [&](const Candidate &c) {
+        return c.r ? std::make_pair(c.r->k, c.r->v) : std::make_pair(fp[c.other]->k, fp[c.other]->v);
+    };
+    std::stable_sort(chosen.begin(), chosen.end(), [&](const Candidate &a, const Candidate &b) {
+        return std::less<std::pair<const void *, const void *>>()(base(a), base(b));
+    });
+    auto *differ = reinterpret_cast<uint32_t *>(ctx->d_scratch + dev_off);
+    CM_CUDA_TRY(cudaMemsetAsync(differ, 0, chosen.size() * 4, stream), "comparison flags reset");
+    std::unique_ptr<cm::CompareFull> cl(new cm::CompareFull);
+    for (size_t c0 = 0; c0 < chosen.size(); c0 += (size_t)cm::kMaxComparePairs) {
+        const size_t cn = std::min(chosen.size() - c0, (size_t)cm::kMaxComparePairs);
+        std::memset(cl.get(), 0, sizeof(cm::CompareFull));
+        for (size_t m = 0; m < cn; ++m) {
+            const Candidate &c = chosen[c0 + m];
+            const cm_fragment *f = fp[c.delivery];
+            cl->member[m] = {static_cast<const uint4 *>(f->k), static_cast<const uint4 *>(f->v)};
+            // one fragment's copies share its shape, so also the group's
+            if (m == 0 || base(chosen[c0 + m - 1]) != base(c)) {
+                cl->group[cl->groups] = {static_cast<const uint4 *>(base(c).first),
+                                         static_cast<const uint4 *>(base(c).second), plane_vecs(f), (uint32_t)m, 0};
+                cl->chunk_begin[cl->groups + 1] = cl->chunk_begin[cl->groups] +
+                    2 * ceil_div(plane_vecs(f), (uint64_t)cm::kCompareChunkVecs);
+                ++cl->groups;
+            }
+            cl->group[cl->groups - 1].end = (uint32_t)m + 1;
+        }
+        cl->differ = differ + c0;
+        CM_CUDA_TRY(cm::launch_compare_full(*cl, ctx->num_sms, blocks_per_sm, stream), "comparison launch");
+        if (ctx->timing) ++ctx->aux_launches;
     }
+    CM_CUDA_TRY(read_small(ctx, host_off, differ, chosen.size() * 4, stream), "comparison flags copy");
     return CM_OK;
 }
 
@@ -959,6 +977,68 @@ cm_status insert_deliveries(cm_context *ctx, cm_set *const *sets,
     return CM_OK;
 }
 
+cm_status ensure_side_stream(cm_context *ctx) {
+    if (!ctx->side) {
+        // the highest priority: the render's CTAs, launched while the leaf hash's grid is
+        // already queued, are dispatched as soon as any of its blocks retire
+        int least = 0, greatest = 0;
+        CM_CUDA_TRY(cudaDeviceGetStreamPriorityRange(&least, &greatest), "stream priorities");
+        CM_CUDA_TRY(cudaStreamCreateWithPriority(&ctx->side, cudaStreamNonBlocking, greatest),
+                    "side stream");
+    }
+    for (cudaEvent_t *e : {&ctx->side_begin, &ctx->side_end, &ctx->side_keys, &ctx->leaves_end})
+        if (!*e) CM_CUDA_TRY(cudaEventCreateWithFlags(e, cudaEventDisableTiming), "side event");
+    return CM_OK;
+}
+
+// Orders a stream after the context's side stream on every way out of a scope (a C++ exception
+// included): explicitly through run(), else in the destructor.
+struct SideJoin {
+    cm_context *ctx;
+    cudaStream_t cs;
+    bool done = false;
+    cudaError_t run() {
+        done = true;
+        cudaError_t e = cudaEventRecord(ctx->side_end, ctx->side);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(cs, ctx->side_end, 0);
+        return e;
+    }
+    ~SideJoin() {
+        if (!done) run();
+    }
+};
+
+// The full comparisons of `chosen` (match_prefixes) beside the content address of `hash`: the
+// comparisons are bound by HBM and run on the context's side stream, two blocks per SM, the
+// hash by the integer pipes on `cs`, which is synchronised. Results: differ (one flag per entry
+// of `chosen`, which is sorted anew), ids and Qs of `hash`.
+cm_status compare_and_digest(cm_context *ctx, const std::vector<const cm_fragment *> &fp,
+                             std::vector<Candidate> &chosen, const std::vector<const cm_fragment *> &hash,
+                             cudaStream_t cs, std::vector<uint32_t> &differ, cm_id *ids,
+                             std::vector<uint64_t> *Qs) {
+    DigestPlan plan;
+    cm_status st = plan_digest(ctx, hash.data(), hash.size(), plan);
+    if (st != CM_OK) return st;
+    const size_t dev_off = (plan.dev_bytes + 255) & ~(size_t)255, host_off = (plan.host_bytes + 255) & ~(size_t)255;
+    st = ensure_scratch(ctx, dev_off + chosen.size() * 4, host_off + chosen.size() * 4);
+    if (st == CM_OK) st = ensure_side_stream(ctx);
+    if (st != CM_OK) return st;
+    CM_CUDA_TRY(cudaEventRecord(ctx->side_begin, cs), "side stream ordering");
+    CM_CUDA_TRY(cudaStreamWaitEvent(ctx->side, ctx->side_begin, 0), "side stream ordering");
+    SideJoin side_join{ctx, cs};
+    if (!chosen.empty()) st = enqueue_comparisons(ctx, fp, chosen, ctx->side, hash.empty() ? 6 : 2, dev_off, host_off);
+    if (st == CM_OK && !hash.empty())
+        st = enqueue_digest(ctx, plan, hash.data(), hash.size(), cs, cm::LeafMode::kWithNorms);
+    const cudaError_t e = side_join.run();
+    if (st == CM_OK && e != cudaSuccess) st = cuda_fail(e, "side stream ordering");
+    if (st != CM_OK) return st;
+    CM_CUDA_TRY(cudaStreamSynchronize(cs), "ingest synchronisation");
+    differ.resize(chosen.size());
+    if (!chosen.empty()) std::memcpy(differ.data(), ctx->h_pinned + host_off, chosen.size() * 4);
+    collect_digest(ctx, plan, hash.data(), hash.size(), ids, Qs);
+    return CM_OK;
+}
+
 // Ingest (Algorithm 2) of the validated deliveries fp, delivery i into sets[i]: one GPU
 // pass for all of them (after the re-delivery fast path, when it is on), then the
 // insertions in delivery order. Caller holds ctx->mu and the device scope.
@@ -966,29 +1046,60 @@ cm_status ingest_validated(cm_context *ctx, cm_set *const *sets,
                            const std::vector<const cm_fragment *> &fp, cudaStream_t cs,
                            cm_id *out_ids, int32_t *out_absorbed) {
     const size_t n = fp.size();
+    if (!ctx->dedup_bytes) {
+        const DeliverySources src = hash_everything(n, fp);
+        std::vector<cm_id> ids(n);
+        std::vector<std::vector<uint64_t>> Q(n);
+        cm_status st = fragments_digest(ctx, fp.data(), n, cs, ids.data(), Q.data());
+        if (st != CM_OK) return st;
+        return insert_deliveries(ctx, sets, fp, cs, src, ids, Q, out_ids, out_absorbed);
+    }
+    // deliveries byte-identical to a known fragment take its id and norm key and are not
+    // hashed: those with no candidate left after the prefix pass are hashed while the
+    // candidates are compared in full, those found to differ there afterwards
     DeliverySources src;
-    if (ctx->dedup_bytes) {
-        // deliveries byte-identical to a known fragment take its id and norm key and are
-        // not hashed
-        cm_status st = find_redeliveries(ctx, sets, fp, cs, src.rec, src.from);
-        if (st != CM_OK) return st;
-        src.hashed_as.assign(n, 0);
-        for (size_t i = 0; i < n; ++i)
-            if (!src.rec[i] && src.from[i] < 0) {
-                src.hashed_as[i] = src.to_hash.size();
-                src.to_hash.push_back(fp[i]);
-            }
-    } else {
-        src = hash_everything(n, fp);
+    std::vector<Candidate> chosen;
+    cm_status st = match_prefixes(ctx, sets, fp, cs, src.rec, src.from, chosen);
+    if (st != CM_OK) return st;
+    src.hashed_as.assign(n, 0);
+    auto hash_later = [&](size_t i) {
+        src.hashed_as[i] = src.to_hash.size();
+        src.to_hash.push_back(fp[i]);
+    };
+    size_t next = 0;   // chosen is in delivery order
+    for (size_t i = 0; i < n; ++i) {
+        if (next < chosen.size() && chosen[next].delivery == i)
+            ++next;
+        else if (!src.rec[i] && src.from[i] < 0)
+            hash_later(i);
     }
-    std::vector<cm_id> hashed_ids(src.to_hash.size());
-    std::vector<std::vector<uint64_t>> hashed_Q(src.to_hash.size());
-    if (!src.to_hash.empty()) {
-        cm_status st = fragments_digest(ctx, src.to_hash.data(), src.to_hash.size(), cs,
-                                        hashed_ids.data(), hashed_Q.data());
+    const size_t first = src.to_hash.size();
+    std::vector<cm_id> ids(first);
+    std::vector<std::vector<uint64_t>> Q(first);
+    if (!chosen.empty()) {
+        std::vector<uint32_t> differ;
+        st = compare_and_digest(ctx, fp, chosen, src.to_hash, cs, differ, ids.data(), Q.data());
+        if (st != CM_OK) return st;
+        for (size_t q = 0; q < chosen.size(); ++q) {
+            if (differ[q] != 0)
+                hash_later(chosen[q].delivery);
+            else if (chosen[q].r)
+                src.rec[chosen[q].delivery] = chosen[q].r;
+            else
+                src.from[chosen[q].delivery] = (int32_t)chosen[q].other;
+        }
+    } else if (first != 0) {
+        st = fragments_digest(ctx, src.to_hash.data(), first, cs, ids.data(), Q.data());
         if (st != CM_OK) return st;
     }
-    return insert_deliveries(ctx, sets, fp, cs, src, hashed_ids, hashed_Q, out_ids, out_absorbed);
+    const size_t more = src.to_hash.size() - first;
+    if (more != 0) {
+        ids.resize(first + more);
+        Q.resize(first + more);
+        st = fragments_digest(ctx, src.to_hash.data() + first, more, cs, ids.data() + first, Q.data() + first);
+        if (st != CM_OK) return st;
+    }
+    return insert_deliveries(ctx, sets, fp, cs, src, ids, Q, out_ids, out_absorbed);
 }
 
 // Ingest (Algorithm 2) of n deliveries, delivery i into sets[i] (several entries
@@ -1365,20 +1476,6 @@ std::vector<Slot> canonical_slots(const cm_set *set, void *k_out, void *v_out, i
 // 330, 292.
 constexpr uint64_t kBesideLargeBytes = 512ull << 20;
 
-cm_status ensure_side_stream(cm_context *ctx) {
-    if (!ctx->side) {
-        // the highest priority: the render's CTAs, launched while the leaf hash's grid is
-        // already queued, are dispatched as soon as any of its blocks retire
-        int least = 0, greatest = 0;
-        CM_CUDA_TRY(cudaDeviceGetStreamPriorityRange(&least, &greatest), "stream priorities");
-        CM_CUDA_TRY(cudaStreamCreateWithPriority(&ctx->side, cudaStreamNonBlocking, greatest),
-                    "side stream");
-    }
-    for (cudaEvent_t *e : {&ctx->side_begin, &ctx->side_end, &ctx->side_keys, &ctx->leaves_end})
-        if (!*e) CM_CUDA_TRY(cudaEventCreateWithFlags(e, cudaEventDisableTiming), "side event");
-    return CM_OK;
-}
-
 // cm_ingest_render (see include/cm.h). The norm keys of the deliveries are computed on
 // the context's side stream while the content address runs on `stream`. Equal bytes give
 // equal norm keys, so members of the prospective set whose integer tail sums S (Eq. rho),
@@ -1474,22 +1571,8 @@ cm_status ingest_render_impl(cm_set *const *sets, const cm_fragment *frags, int3
     if (st != CM_OK) return st;
     CM_CUDA_TRY(cudaEventRecord(ctx->side_begin, cs), "side stream ordering");
     CM_CUDA_TRY(cudaStreamWaitEvent(ctx->side, ctx->side_begin, 0), "side stream ordering");
-    // from here on, every way out (a C++ exception included) orders the caller's stream
-    // after the side stream's work: explicitly through join(), else in the destructor
-    struct SideJoin {
-        cm_context *ctx;
-        cudaStream_t cs;
-        bool done = false;
-        cudaError_t run() {
-            done = true;
-            cudaError_t e = cudaEventRecord(ctx->side_end, ctx->side);
-            if (e == cudaSuccess) e = cudaStreamWaitEvent(cs, ctx->side_end, 0);
-            return e;
-        }
-        ~SideJoin() {
-            if (!done) run();
-        }
-    } side_join{ctx, cs};
+    // from here on, every way out orders the caller's stream after the side stream's work
+    SideJoin side_join{ctx, cs};
     auto join = [&](cm_status prior) -> cm_status {
         const cudaError_t e = side_join.run();
         if (e != cudaSuccess && prior == CM_OK) return cuda_fail(e, "side stream ordering");

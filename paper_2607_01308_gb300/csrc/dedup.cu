@@ -13,71 +13,74 @@ namespace {
 constexpr int kThreads = 256;
 constexpr uint64_t kPrefixVecs = 256;                   // 4 KiB
 constexpr uint64_t kChunkVecs = kCompareChunkVecs;      // 32 KiB of each array per chunk
-static_assert(kChunkVecs == (uint64_t)kThreads * 8, "a chunk is 8 vectors per thread");
-static_assert(sizeof(CompareLaunch) <= 32764, "comparison parameters exceed the kernel parameter limit");
+constexpr int kStepVecs = 4;                            // vectors per thread at a time
+static_assert(kChunkVecs % ((uint64_t)kThreads * kStepVecs) == 0, "a chunk is a number of whole steps");
+static_assert(sizeof(CompareFull) <= 32764, "comparison parameters exceed the kernel parameter limit");
 
 __device__ __forceinline__ uint32_t diff4(const uint4 &x, const uint4 &y) {
     return (x.x ^ y.x) | (x.y ^ y.y) | (x.z ^ y.z) | (x.w ^ y.w);
 }
 
 // One block per pair: the first 4 KiB of K.
-__global__ void __launch_bounds__(kThreads) prefix_kernel(const __grid_constant__ CompareLaunch c) {
+__global__ void __launch_bounds__(kThreads) prefix_kernel(const __grid_constant__ ComparePrefix c) {
     const ComparePair &p = c.pair[blockIdx.x];
     const uint64_t n = p.vecs < kPrefixVecs ? p.vecs : kPrefixVecs;
     uint32_t d = 0;
     for (uint64_t i = threadIdx.x; i < n; i += kThreads) d |= diff4(__ldg(p.a_k + i), __ldg(p.b_k + i));
-    if (__syncthreads_or(d != 0) && threadIdx.x == 0) atomicOr(c.differ + blockIdx.x, 1u);
+    const int any = __syncthreads_or(d != 0);
+    if (threadIdx.x == 0) c.differ[blockIdx.x] = any ? 1u : 0u;
 }
 
-// Persistent grid over the chunks of all pairs (K then V of each); a block skips the
-// chunks of a pair that another block has already found to differ.
-__global__ void __launch_bounds__(kThreads) full_kernel(const __grid_constant__ CompareLaunch c) {
-    const uint64_t total = c.chunk_begin[c.count];
-    __shared__ uint32_t skip;
-    for (uint64_t g = blockIdx.x; g < total; g += gridDim.x) {
-        uint32_t pi = 0;
-        while (pi + 1 < c.count && g >= c.chunk_begin[pi + 1]) ++pi;
-        const ComparePair &p = c.pair[pi];
-        if (threadIdx.x == 0) skip = __ldcg(c.differ + pi);
-        __syncthreads();
-        const bool done = skip != 0;
-        __syncthreads();                                   // everyone has read `skip`
-        if (done) {
-            // jump to this block's first chunk past the pair: g + k gridDim with
-            // k = ceil((end - g) / gridDim) >= 1 (the loop adds the last gridDim)
-            const uint64_t end = c.chunk_begin[pi + 1];
-            g += ((end - g + gridDim.x - 1) / gridDim.x - 1) * (uint64_t)gridDim.x;
-            continue;
-        }
-        // chunk index within the pair: the K chunks, then the V chunks
-        const uint64_t per_array = (p.vecs + kChunkVecs - 1) / kChunkVecs;
-        const uint64_t local = g - c.chunk_begin[pi];
+// Persistent grid over the chunks of all groups (K then V of each): a warp loads its part of
+// the base's chunk and compares every member's with it, so the base is read once for all its
+// members (bound by HBM: (members + 1) reads of a fragment instead of 2 per member). Members
+// that another warp has found to differ are skipped.
+__global__ void __launch_bounds__(kThreads) full_kernel(const __grid_constant__ CompareFull c) {
+    const uint64_t total = c.chunk_begin[c.groups];
+    uint32_t gi = 0;
+    for (uint64_t x = blockIdx.x; x < total; x += gridDim.x) {
+        while (x >= c.chunk_begin[gi + 1]) ++gi;
+        const CompareGroup &g = c.group[gi];
+        // chunk index within the group: the K chunks, then the V chunks
+        const uint64_t per_array = (g.vecs + kChunkVecs - 1) / kChunkVecs;
+        const uint64_t local = x - c.chunk_begin[gi];
         const bool is_v = local >= per_array;
-        const uint64_t base = (is_v ? local - per_array : local) * kChunkVecs;
-        const uint4 *a = is_v ? p.a_v : p.a_k;
-        const uint4 *b = is_v ? p.b_v : p.b_k;
-        uint32_t d = 0;
+        const uint64_t begin = (is_v ? local - per_array : local) * kChunkVecs;
+        const uint64_t end = begin + kChunkVecs < g.vecs ? begin + kChunkVecs : g.vecs;
+        const uint4 *base = is_v ? g.v : g.k;
+#pragma unroll 1
+        for (uint64_t i = begin + threadIdx.x; i < end; i += (uint64_t)kThreads * kStepVecs) {
+            uint4 b[kStepVecs];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const uint64_t i = base + (uint64_t)u * kThreads + threadIdx.x;
-            if (i < p.vecs) d |= diff4(__ldcs(a + i), __ldcs(b + i));
+            for (int u = 0; u < kStepVecs; ++u)
+                b[u] = i + (uint64_t)u * kThreads < end ? __ldcs(base + i + (uint64_t)u * kThreads)
+                                                        : make_uint4(0, 0, 0, 0);
+            for (uint32_t m = g.begin; m < g.end; ++m) {
+                if (__ldcg(c.differ + m) != 0) continue;
+                const uint4 *a = is_v ? c.member[m].v : c.member[m].k;
+                uint32_t d = 0;
+#pragma unroll
+                for (int u = 0; u < kStepVecs; ++u)
+                    if (i + (uint64_t)u * kThreads < end) d |= diff4(__ldcs(a + i + (uint64_t)u * kThreads), b[u]);
+                if (d != 0) atomicOr(c.differ + m, 1u);
+            }
         }
-        if (__syncthreads_or(d != 0) && threadIdx.x == 0) atomicOr(c.differ + pi, 1u);
     }
 }
 
 }  // namespace
 
-cudaError_t launch_compare_prefix(const CompareLaunch &c, cudaStream_t stream) {
+cudaError_t launch_compare_prefix(const ComparePrefix &c, cudaStream_t stream) {
     if (c.count == 0) return cudaSuccess;
     prefix_kernel<<<c.count, kThreads, 0, stream>>>(c);
     return cudaGetLastError();
 }
 
-cudaError_t launch_compare_full(const CompareLaunch &c, int num_sms, cudaStream_t stream) {
-    if (c.count == 0) return cudaSuccess;
-    const uint64_t total = c.chunk_begin[c.count];
-    const uint64_t grid = total < (uint64_t)num_sms * 8 ? total : (uint64_t)num_sms * 8;
+cudaError_t launch_compare_full(const CompareFull &c, int num_sms, int blocks_per_sm, cudaStream_t stream) {
+    if (c.groups == 0) return cudaSuccess;
+    const uint64_t total = c.chunk_begin[c.groups];
+    const uint64_t most = (uint64_t)num_sms * (uint64_t)blocks_per_sm;
+    const uint64_t grid = total < most ? total : most;
     if (grid == 0) return cudaSuccess;
     full_kernel<<<(unsigned)grid, kThreads, 0, stream>>>(c);
     return cudaGetLastError();
