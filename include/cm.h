@@ -398,7 +398,7 @@ typedef struct cm_kernel_times {
                                      the norm keys beside it included */
     int64_t leaf_hash_launches;
     double inner_hash_ms;         /* content address, tree levels above the leaves (one
-                                     kernel per call, or two when the call has 32,768 or
+                                     kernel per call, or two when the call has 16,384 or
                                      more level-1 nodes: level 1, then the levels above) */
     int64_t inner_hash_launches;
     double render_ms;             /* render / BagMerge */

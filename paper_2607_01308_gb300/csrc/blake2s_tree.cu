@@ -39,7 +39,7 @@ __device__ __forceinline__ uint32_t rotr7(uint32_t x) { return __funnelshift_r(x
 //
 // a + b + x: x is added first. b is the last word that the previous half of G produced, so
 // this leaves one addition instead of two on G's chain of dependent operations: one warp
-// alone took 0.89 instead of 1.08 us per compression (the tree levels run few warps).
+// alone took 0.89 instead of 1.08 us per compression.
 //
 // The rotation by 16 can move as well: x * 2^16 is its upper half, and a two-way 16-bit dot
 // product with (0, 1) adds its lower half: two multiply-type instructions for one byte
@@ -63,12 +63,11 @@ __device__ __forceinline__ uint32_t rotr16_fma(uint32_t x) {
 }
 
 // Which G's rotate by 16 on the FMA pipe (bit g of kMask: the round's G number g): five of
-// the eight in the leaf kernel, none in kernels that run few warps (bound by the chain of
-// dependent operations, which the dot product lengthens).
+// the eight in the leaf kernel and for level 1 of many nodes.
 // Beside a render (kBesideRender), whose own instructions take issue slots and the FMA pipe,
 // three: the Qwen3-4B-shaped merge of 4 x 4096 tokens took 1.71 ms with 3, 1.71 with 2, 1.72
 // with none or one and 1.77 with 5; the arity merge 0.77, 0.79, 0.80 and 0.78.
-constexpr uint32_t kIssueBound = 0xD6u, kBesideRender = 0x52u, kLatencyBound = 0u;
+constexpr uint32_t kIssueBound = 0xD6u, kBesideRender = 0x52u;
 template <uint32_t kMask, int kG>
 __device__ __forceinline__ uint32_t rotate16(uint32_t x) {
     return (kMask >> kG) & 1u ? rotr16_fma(x) : rotr16(x);
@@ -280,6 +279,102 @@ __device__ __forceinline__ const uint8_t *cursor_next(const LeafLaunch &a, Strea
     return p;
 }
 
+// Four lanes to a node, for levels with few nodes, where the chain of dependent operations
+// bounds a compression: lane q holds column q of the state (words q, q + 4, q + 8, q + 12) and
+// does one G of every half round, so the chain is G's twelve operations and not four G's taking
+// turns on the half-rate ALU pipe. Between the halves the diagonals are lined up by moving a, c
+// and d to the lanes that hold their b: b is the last word that G produces, and the moves of the
+// others hide behind it. One warp alone takes 0.61 us per compression this way, 0.89 with a
+// lane to a node.
+//
+// The message words lie in shared memory; g_schedule[q][r] holds, a byte each, the offsets of
+// the words that lane q's two G's of round r add (RFC 7693, Section 2.7: column G q, then
+// diagonal G q - 1, whose b is in column q).
+#define CM_Q4(x0, y0, x1, y1) (4u * (x0) | 4u * (y0) << 8 | 4u * (x1) << 16 | 4u * (y1) << 24)
+#define CM_QUAD(s0, s1, s2, s3, s4, s5, s6, s7, s8, s9, s10, s11, s12, s13, s14, s15)          \
+    {CM_Q4(s0, s1, s14, s15), CM_Q4(s2, s3, s8, s9), CM_Q4(s4, s5, s10, s11), CM_Q4(s6, s7, s12, s13)}
+__constant__ uint32_t g_schedule[10][4] = {
+    CM_QUAD(0, 1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14, 15),
+    CM_QUAD(14, 10, 4, 8, 9, 15, 13, 6, 1, 12, 0, 2, 11, 7, 5, 3),
+    CM_QUAD(11, 8, 12, 0, 5, 2, 15, 13, 10, 14, 3, 6, 7, 1, 9, 4),
+    CM_QUAD(7, 9, 3, 1, 13, 12, 11, 14, 2, 6, 5, 10, 4, 0, 15, 8),
+    CM_QUAD(9, 0, 5, 7, 2, 4, 10, 15, 14, 1, 11, 12, 6, 8, 3, 13),
+    CM_QUAD(2, 12, 6, 10, 0, 11, 8, 3, 4, 13, 7, 5, 15, 14, 1, 9),
+    CM_QUAD(12, 5, 1, 15, 14, 13, 4, 10, 0, 7, 6, 3, 9, 2, 8, 11),
+    CM_QUAD(13, 11, 7, 14, 12, 1, 3, 9, 5, 0, 15, 4, 8, 6, 2, 10),
+    CM_QUAD(6, 15, 14, 9, 11, 3, 0, 8, 12, 2, 13, 7, 1, 4, 10, 5),
+    CM_QUAD(10, 2, 8, 4, 7, 6, 1, 5, 15, 11, 9, 14, 3, 12, 13, 0),
+};
+#undef CM_QUAD
+#undef CM_Q4
+__constant__ uint32_t g_iv[8] = {kIV0, kIV1, kIV2, kIV3, kIV4, kIV5, kIV6, kIV7};
+
+struct QuadLane {
+    uint32_t q, before, after, across;   // lane in its node, and the node's lanes q - 1, q + 1, q + 2
+    uint32_t iv_c, iv_d;
+    uint32_t schedule[10];
+};
+
+__device__ __forceinline__ QuadLane quad_lane(uint32_t lane) {
+    QuadLane l;
+    l.q = lane & 3u;
+    const uint32_t base = lane & 28u;
+    l.before = base | ((l.q + 3u) & 3u);
+    l.after = base | ((l.q + 1u) & 3u);
+    l.across = base | (l.q ^ 2u);
+    l.iv_c = g_iv[l.q];
+    l.iv_d = g_iv[4u + l.q];
+#pragma unroll
+    for (int r = 0; r < 10; ++r) l.schedule[r] = g_schedule[r][l.q];
+    return l;
+}
+
+__device__ __forceinline__ uint32_t move(uint32_t x, uint32_t from) { return __shfl_sync(0xFFFFFFFFu, x, (int)from); }
+
+__device__ __forceinline__ void quad_g(uint32_t &a, uint32_t &b, uint32_t &c, uint32_t &d, uint32_t x, uint32_t y) {
+    a = add3(a, b, x);
+    d = rotr16(d ^ a);
+    c = c + d;
+    b = rotr12(b ^ c);
+    a = add3(a, b, y);
+    d = rotr8(d ^ a);
+    c = c + d;
+    b = rotr7(b ^ c);
+}
+
+// One compression by the four lanes of a node: (h0, h1) are words q and q + 4 of the chaining
+// value, the block's words lie at m, t = bytes hashed so far including this block (below 2^32).
+// Every lane of the warp calls.
+__device__ __forceinline__ void quad_compress(const QuadLane &l, uint32_t &h0, uint32_t &h1, const uint8_t *m,
+                                              uint32_t t, bool last_block, bool last_node) {
+    uint32_t a = h0, b = h1, c = l.iv_c, d = l.iv_d;
+    if (l.q == 0) d ^= t;
+    if (l.q == 2 && last_block) d = ~d;
+    if (l.q == 3 && last_block && last_node) d = ~d;
+#pragma unroll
+    for (int r = 0; r < 10; ++r) {
+        const uint32_t s = l.schedule[r];
+        auto word = [&](uint32_t k) {
+            return *reinterpret_cast<const uint32_t *>(m + __byte_perm(s, 0, 0x4440u + k));
+        };
+        quad_g(a, b, c, d, word(0), word(1));
+        a = move(a, l.before), c = move(c, l.after), d = move(d, l.across);
+        quad_g(a, b, c, d, word(2), word(3));
+        a = move(a, l.after), c = move(c, l.before), d = move(d, l.across);
+    }
+    h0 ^= a ^ c;
+    h1 ^= b ^ d;
+}
+
+// Words q and q + 4 of the chaining value that node (offset, depth) starts from.
+__device__ __forceinline__ void quad_init(const QuadLane &l, uint32_t &h0, uint32_t &h1, const TreeParams &tp,
+                                          uint64_t offset, uint32_t depth) {
+    h0 = tp.h_base[l.q];
+    h1 = tp.h_base[4 + l.q];
+    if (l.q == 2) h0 ^= (uint32_t)offset;
+    if (l.q == 3) h0 ^= ((uint32_t)(offset >> 32) & 0xFFFFu) | (depth << 16);
+}
+
 // A launch with programmatic stream serialisation may start while the launch before it on the
 // stream drains: its blocks wait here until that launch has completed and its writes are
 // visible.
@@ -293,6 +388,14 @@ __device__ __forceinline__ void allow_next_launch() {
 
 constexpr int kLeafThreads = kLeafBlockThreads;
 
+// A block of the leaf launch: zeroes a fragment's arrival counters for the tree launch, and ends
+// after the launch before this one, so that the tree launch comes after both.
+__device__ __forceinline__ void zero_arrivals(const LeafLaunch &a) {
+    for (uint32_t i = threadIdx.x; i < a.num_arrivals; i += kLeafThreads)
+        if (CM_IN_BOUNDS(a.arrivals + i, 4, a.arrivals, (uint64_t)a.num_arrivals * 4)) a.arrivals[i] = 0;
+    wait_for_previous_launch();
+}
+
 // kWhole: every plane of the group is a multiple of a leaf, so each leaf is 1 KiB of one
 // segment. Otherwise a leaf may run into the next segments and a fragment's last leaf may be
 // short (a multiple of 64 bytes, as 2 L planes are): every leaf then walks its blocks in
@@ -301,16 +404,12 @@ constexpr int kLeafThreads = kLeafBlockThreads;
 template <uint32_t kFmaMask, bool kWhole>
 __global__ void __launch_bounds__(kLeafThreads)
 leaf_hash_kernel(const __grid_constant__ LeafGroup grp) {
-    // the blocks after the leaf blocks, one per fragment, zero its tree levels' arrival counters
-    // for the tree launch (done by the leaf threads it cost them 8 registers), and end after
-    // the launch before this one, so that the tree launch comes after both
+    // the blocks after the leaf blocks, one per fragment (done by the leaf threads this cost
+    // them 8 registers)
     const uint32_t x = blockIdx.x;
     const uint32_t leaf_blocks = (uint32_t)grp.block_begin[grp.count];
     if (x >= leaf_blocks) {
-        const LeafLaunch &a = grp.frag[x - leaf_blocks];
-        for (uint32_t i = threadIdx.x; i < a.num_arrivals; i += kLeafThreads)
-            if (CM_IN_BOUNDS(a.arrivals + i, 4, a.arrivals, (uint64_t)a.num_arrivals * 4)) a.arrivals[i] = 0;
-        wait_for_previous_launch();
+        zero_arrivals(grp.frag[x - leaf_blocks]);
         return;
     }
     uint32_t fi = 0;                                   // the block's fragment (uniform)
@@ -352,6 +451,62 @@ leaf_hash_kernel(const __grid_constant__ LeafGroup grp) {
         store_digest(a.digests + leaf * kDigestBytes, h);
 }
 
+// Level 0 with four lanes to a leaf, for groups of so few leaves that the chain of a leaf's 16
+// compressions bounds them: kLeafThreads / 4 leaves to a block, so four blocks here for one of
+// block_begin, then the blocks that zero the arrival counters as above. Lane q loads its 16
+// bytes of the next block while this one is hashed.
+__global__ void __launch_bounds__(kLeafThreads)
+leaf_quad_kernel(const __grid_constant__ LeafGroup grp) {
+    constexpr uint32_t kSlotBytes = 2 * 64 + 16;   // two blocks, 16 bytes to spread the leaves over the banks
+    __shared__ __align__(16) uint8_t stage_all[kLeafThreads / 4][kSlotBytes];
+    const uint32_t leaf_blocks = (uint32_t)grp.block_begin[grp.count];
+    const uint32_t x = blockIdx.x >> 2;
+    if (x >= leaf_blocks) {
+        zero_arrivals(grp.frag[blockIdx.x - 4 * leaf_blocks]);
+        return;
+    }
+    uint32_t fi = 0;                                   // the block's fragment (uniform)
+    while (fi + 1 < grp.count && x >= grp.block_begin[fi + 1]) ++fi;
+    const LeafLaunch &a = grp.frag[fi];
+    const QuadLane l = quad_lane(threadIdx.x & 31u);
+    const uint64_t leaf = (uint64_t)(x - grp.block_begin[fi]) * kLeafThreads +
+                          (blockIdx.x & 3u) * (kLeafThreads / 4) + (threadIdx.x >> 2);
+    const uint64_t begin = leaf * kLeafBytes;
+    const uint64_t rem = leaf < a.num_leaves ? a.stream_bytes - begin : 0;
+    const uint32_t nblocks = rem < (uint64_t)kLeafBytes ? (uint32_t)rem / 64 : (uint32_t)kLeafBytes / 64;
+    uint8_t *stage = stage_all[threadIdx.x >> 2];
+    uint64_t pos = begin + 16 * l.q;
+    StreamCursor cur{};
+    auto load = [&](uint32_t n) {   // this lane's part of block n, the block after the last one loaded
+        if (n >= nblocks) return make_uint4(0, 0, 0, 0);
+        if (n == 0 || cur.left <= 64) {
+            cur = cursor_at(a, pos);
+        } else {
+            cur.ptr += 64;
+            cur.left -= 64;
+        }
+        pos += 64;
+        return in_fragment(a, cur.ptr, 16) ? load_nc(cur.ptr) : make_uint4(0, 0, 0, 0);
+    };
+    uint32_t h0, h1;
+    quad_init(l, h0, h1, a.tree, leaf, 0);
+    uint4 next = load(0);
+#pragma unroll 1
+    for (uint32_t n = 0; n < (uint32_t)kLeafBytes / 64; ++n) {
+        if (!__any_sync(0xFFFFFFFFu, n < nblocks)) break;
+        uint8_t *m = stage + 64 * (n & 1u);   // the other half may still be read
+        *reinterpret_cast<uint4 *>(m + 16 * l.q) = next;
+        __syncwarp();
+        next = load(n + 1);
+        const uint32_t k0 = h0, k1 = h1;
+        quad_compress(l, h0, h1, m, (n + 1) * 64, n + 1 == nblocks, leaf + 1 == a.num_leaves);
+        if (n >= nblocks) h0 = k0, h1 = k1;
+    }
+    uint8_t *out = a.digests + leaf * kDigestBytes + 4 * l.q;
+    if (leaf < a.num_leaves && CM_IN_BOUNDS(out, 4, a.digests, a.num_leaves * kDigestBytes))
+        *reinterpret_cast<uint32_t *>(out) = h0;
+}
+
 // The norm keys of a group: the blocks walk over the group's norm blocks. Ahead of a leaf
 // launch they are at most one to an SM (the FP64 pipe bounds them, the ALU and FMA pipes the
 // leaves), and the leaves start as soon as they run.
@@ -367,56 +522,12 @@ norm_key_kernel(const __grid_constant__ LeafGroup grp) {
     }
 }
 
-constexpr int kInnerThreads = 32;
-
-// Digest of node j of a tree level from its 16 * min(16, num_children - 16 j) bytes of
-// children's digests, at most four 64-byte blocks, staged in the thread's 256-byte slice of
-// shared memory so that one copy of the compression loop serves every level (the tree top
-// runs few warps per SM; unrolled copies of the compression would not fit the instruction
-// cache).
-__device__ __forceinline__ uint4 node_digest(const uint4 *stage, uint32_t len, uint64_t j,
-                                             uint64_t num_nodes, uint32_t depth,
-                                             const TreeParams &tp) {
-    const uint32_t nblocks = (len + 63) / 64;
-    const bool last_node = j + 1 == num_nodes;
-    uint32_t h[8];
-    node_init(h, tp, j, depth);
-#pragma unroll 1
-    for (uint32_t b = 0; b < nblocks; ++b) {
-        const uint4 w0 = stage[4 * b], w1 = stage[4 * b + 1], w2 = stage[4 * b + 2],
-                    w3 = stage[4 * b + 3];
-        const uint32_t m[16] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w,
-                                w2.x, w2.y, w2.z, w2.w, w3.x, w3.y, w3.z, w3.w};
-        const uint32_t end = (b + 1) * 64 < len ? (b + 1) * 64 : len;
-        compress<kLatencyBound>(h, m, end, b + 1 == nblocks, last_node);
-    }
-    return make_uint4(h[0], h[1], h[2], h[3]);
-}
+constexpr int kTopThreads = 64;   // of a tree-top block
 
 // Bytes of children under node j of a level above one of num_children nodes.
 __device__ __forceinline__ uint32_t child_bytes(uint64_t num_children, uint64_t j) {
     const uint64_t left = num_children - j * kFanout;
     return (left < (uint64_t)kFanout ? (uint32_t)left : (uint32_t)kFanout) * kDigestBytes;
-}
-
-// Loads node j's children (zero-padded to 256 bytes) into `stage`; returns their length. Read
-// through L2 (ld.global.cg): other threads of this launch, or of the launch that this one
-// overlaps, wrote them.
-__device__ __forceinline__ uint32_t stage_children(uint4 *stage, const uint8_t *children,
-                                                   uint64_t num_children, uint64_t j) {
-    static_assert(kFanout * kDigestBytes <= 256, "an inner node must fit four blocks");
-    const uint32_t len = child_bytes(num_children, j);
-    const uint4 *src = reinterpret_cast<const uint4 *>(children + j * kFanout * kDigestBytes);
-    uint4 w[16];
-#pragma unroll
-    for (int q = 0; q < 16; ++q) {
-        const bool in = (uint32_t)(q * 16) < len &&
-                        CM_IN_BOUNDS(src + q, 16, children, num_children * kDigestBytes);
-        w[q] = in ? __ldcg(src + q) : make_uint4(0, 0, 0, 0);
-    }
-#pragma unroll
-    for (int q = 0; q < 16; ++q) stage[q] = w[q];
-    return len;
 }
 
 __device__ __forceinline__ uint32_t arrive_acq_rel(uint32_t *counter) {
@@ -465,64 +576,103 @@ level1_kernel(const __grid_constant__ TreeTop t) {
         store_digest(f.level[1] + j * kDigestBytes, h);
 }
 
+// Digest of a node by the four lanes that call with its arguments (the warp's lanes all call,
+// with `blocks` the most of any): lane q's word of it. The node's len bytes of children's digests
+// lie at `stage`, zero-padded to whole blocks.
+__device__ __forceinline__ uint32_t quad_digest(const QuadLane &l, const uint8_t *stage, uint32_t len,
+                                                uint32_t blocks, uint64_t j, uint64_t num_nodes,
+                                                uint32_t depth, const TreeParams &tp) {
+    const uint32_t mine = (len + 63) / 64;
+    uint32_t h0, h1;
+    quad_init(l, h0, h1, tp, j, depth);
+#pragma unroll 1
+    for (uint32_t n = 0; n < blocks; ++n) {
+        const uint32_t k0 = h0, k1 = h1, end = (n + 1) * 64 < len ? (n + 1) * 64 : len;
+        quad_compress(l, h0, h1, stage + 64 * n, end, n + 1 == mine, j + 1 == num_nodes);
+        if (n >= mine) h0 = k0, h1 = k1;
+    }
+    return h0;
+}
+
+constexpr uint32_t kStageBytes = kFanout * kDigestBytes + 16;   // 16 to spread the nodes over the banks
+
 // Levels kStart and up (node_begin: prefix sums of the level-kStart sizes, each rounded up to
-// a warp, 0 for a fragment without that level): one thread per level-kStart node hashes it,
-// and lanes 0 and 16 then hash the two parents whose children the warp just hashed (a warp's
-// 32 nodes are those of two parents), handed over in shared memory; from there, level by
-// level, the thread that completes a parent's last child hashes the parent. The chain of
-// levels bounds it: about 0.9 us per compression, four to a node, and between levels a
-// store, an arrival and the loads of 16 digests, which the hand-over saves once.
+// the children of one parent, 0 for a fragment without that level): a block hashes the level-
+// kStart nodes of one parent, four lanes each, then its first warp the parent, handed over in
+// shared memory; from there, level by level, the warp that completes a parent's last child
+// hashes the parent. The chain of levels bounds it: four compressions to a node, and between
+// levels a store, an arrival and the loads of 16 digests, which the hand-over saves once.
 template <int kStart>
-__global__ void __launch_bounds__(kInnerThreads)
+__global__ void __launch_bounds__(kTopThreads)
 tree_top_kernel(const __grid_constant__ TreeTop t) {
-    static_assert(kInnerThreads == 32, "a block is one warp: its lanes hand digests over");
-    __shared__ uint4 stage_all[kInnerThreads][16];
-    wait_for_previous_launch();
-    const uint32_t lane = threadIdx.x;
-    const uint64_t g = (uint64_t)blockIdx.x * kInnerThreads + lane;
-    uint32_t fi = 0;                                   // the warp's fragment (uniform)
+    static_assert(kTopThreads == 4 * kFanout, "a block hashes the children of one parent");
+    static_assert(kFanout * kDigestBytes == 256, "an inner node is at most four blocks");
+    __shared__ __align__(16) uint8_t stage_all[kFanout][kStageBytes];
+    __shared__ __align__(16) uint8_t stage_parent[kStageBytes];
+    const QuadLane l = quad_lane(threadIdx.x & 31u);
+    const uint64_t g = (uint64_t)blockIdx.x * kFanout;
+    uint32_t fi = 0;
     while (fi + 1 < t.count && g >= t.node_begin[fi + 1]) ++fi;
     const TreeTopFragment &f = t.frag[fi];
-    uint64_t j = g - t.node_begin[fi];
+    const uint32_t slot = threadIdx.x >> 2;
+    uint64_t j = (g - t.node_begin[fi]) / kFanout;   // the parent
     uint32_t k = kStart;
-    const bool mine = j < f.size[k];
-    uint4 digest = make_uint4(0, 0, 0, 0);
-    if (mine) {
-        const uint32_t len = stage_children(stage_all[lane], f.level[k - 1], f.size[k - 1], j);
-        digest = node_digest(stage_all[lane], len, j, f.size[k], k, f.tree);
-    }
-    if (k + 1 < f.levels) {
-        // lane l's digest is child l % 16 of the parent that lane 16 (l / 16) hashes
+    wait_for_previous_launch();
+    {
+        const uint64_t node = j * kFanout + slot;
+        const bool mine = node < f.size[k];
+        const uint32_t len = mine ? child_bytes(f.size[k - 1], node) : 0;
+        const uint8_t *src = f.level[k - 1] + node * kFanout * kDigestBytes;
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {   // read through L2: the launch that this one overlaps wrote them
+            const uint32_t at = 64 * v + 16 * l.q;
+            const uint4 w = at < len && CM_IN_BOUNDS(src + at, 16, f.level[k - 1], f.size[k - 1] * kDigestBytes)
+                                ? __ldcg(reinterpret_cast<const uint4 *>(src + at))
+                                : make_uint4(0, 0, 0, 0);
+            *reinterpret_cast<uint4 *>(stage_all[slot] + at) = w;
+        }
         __syncwarp();
-        stage_all[lane & 16u][lane & 15u] = digest;
-        __syncwarp();
-        if (!mine || (lane & 15u) != 0) return;
-        const uint32_t len = child_bytes(f.size[k], j / kFanout);
-        j /= kFanout;
-        ++k;
-        digest = node_digest(stage_all[lane], len, j, f.size[k], k, f.tree);
-    } else if (!mine) {
-        return;
+        const uint32_t word = quad_digest(l, stage_all[slot], len, 4, node, f.size[k], k, f.tree);
+        if (k + 1 == f.levels) {   // the root
+            if (mine && CM_IN_BOUNDS(f.level[k] + 4 * l.q, 4, f.level[k], kDigestBytes))
+                reinterpret_cast<uint32_t *>(f.level[k])[l.q] = word;
+            return;
+        }
+        *reinterpret_cast<uint32_t *>(stage_parent + slot * kDigestBytes + 4 * l.q) = mine ? word : 0;
     }
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    uint32_t len = child_bytes(f.size[k], j);
     for (;;) {
+        ++k;
+        // every four lanes hash the same node
+        const uint32_t word = quad_digest(l, stage_parent, len, (len + 63) / 64, j, f.size[k], k, f.tree);
         uint8_t *out = f.level[k] + j * kDigestBytes;
-        if (CM_IN_BOUNDS(out, kDigestBytes, f.level[k], f.size[k] * kDigestBytes))
-            *reinterpret_cast<uint4 *>(out) = digest;
-        if (k + 1 >= f.levels) break;
-        // this thread finished node j of level k; the one that finishes the last child of
+        if (threadIdx.x < 4 && CM_IN_BOUNDS(out + 4 * l.q, 4, f.level[k], f.size[k] * kDigestBytes))
+            reinterpret_cast<uint32_t *>(out)[l.q] = word;
+        if (k + 1 >= f.levels) return;
+        // this warp finished node j of level k; the one that finishes the last child of
         // parent j / 16 hashes the parent
         const uint64_t parent = j / kFanout;
-        const uint32_t len = child_bytes(f.size[k], parent);
-        // one acquire-release add: it publishes this node's digest and, for the thread
+        len = child_bytes(f.size[k], parent);
+        __syncwarp();
+        // one acquire-release add: it publishes this node's digest and, for the warp
         // that counts the last sibling, makes every sibling's digest visible
-        if (!CM_IN_BOUNDS(f.arrivals[k + 1] + parent, 4, f.arrivals[k + 1], f.size[k + 1] * 4))
-            return;
-        const uint32_t done = arrive_acq_rel(f.arrivals[k + 1] + parent) + 1;
+        uint32_t done = 0;
+        if (threadIdx.x == 0 && CM_IN_BOUNDS(f.arrivals[k + 1] + parent, 4, f.arrivals[k + 1], f.size[k + 1] * 4))
+            done = arrive_acq_rel(f.arrivals[k + 1] + parent) + 1;
+        done = __shfl_sync(0xFFFFFFFFu, done, 0);
+        __syncwarp();   // lane 0's acquire comes before the other lanes' loads
         if (done * kDigestBytes != len) return;
         j = parent;
-        stage_children(stage_all[lane], f.level[k], f.size[k], j);
-        ++k;
-        digest = node_digest(stage_all[lane], len, j, f.size[k], k, f.tree);
+        if (threadIdx.x < (uint32_t)kFanout) {
+            const uint8_t *src = f.level[k] + (j * kFanout + threadIdx.x) * kDigestBytes;
+            const uint4 w = threadIdx.x * kDigestBytes < len && CM_IN_BOUNDS(src, 16, f.level[k], f.size[k] * kDigestBytes)
+                                ? __ldcg(reinterpret_cast<const uint4 *>(src))
+                                : make_uint4(0, 0, 0, 0);
+            *reinterpret_cast<uint4 *>(stage_parent + threadIdx.x * kDigestBytes) = w;
+        }
+        __syncwarp();
     }
 }
 
@@ -574,15 +724,21 @@ cudaError_t launch_after(void (*kernel)(P), uint64_t blocks, int threads, cudaSt
 cudaError_t launch_leaf_hash_group(const LeafGroup &g, LeafMode mode, int num_sms, cudaStream_t stream) {
     if (g.count > (uint32_t)kMaxLeafGroup) return cudaErrorInvalidValue;
     if (g.count == 0) return cudaSuccess;
-    const uint64_t blocks = g.block_begin[g.count] + g.count;   // leaves, then arrival counters
+    // four lanes to a leaf up to half a leaf block per SM (two such warps per scheduler; beyond,
+    // they take more issue slots than the chain leaves free): tiny merge 63 -> 58 us, one
+    // 60-token ingest of the Qwen3-4B shape 56 -> 54.5, but of 100 tokens 56 -> 61
+    const bool few = g.block_begin[g.count] * 2 <= (uint64_t)num_sms;
+    const uint64_t blocks = (few ? 4 : 1) * g.block_begin[g.count] + g.count;   // leaves, then arrival counters
     if (blocks > 0x7FFFFFFFull) return cudaErrorInvalidValue;
     bool whole = true;
     for (uint32_t i = 0; i < g.count; ++i) whole = whole && g.frag[i].plane_bytes % kLeafBytes == 0;
-    void (*const alone)(LeafGroup) = whole ? leaf_hash_kernel<kIssueBound, true> : leaf_hash_kernel<kIssueBound, false>;
+    void (*const alone)(LeafGroup) = few     ? leaf_quad_kernel
+                                     : whole ? leaf_hash_kernel<kIssueBound, true>
+                                             : leaf_hash_kernel<kIssueBound, false>;
     if (mode != LeafMode::kWithNorms) {
         void (*const beside)(LeafGroup) =
             whole ? leaf_hash_kernel<kBesideRender, true> : leaf_hash_kernel<kBesideRender, false>;
-        (mode == LeafMode::kBesideRender ? beside : alone)<<<(unsigned)blocks, kLeafThreads, 0, stream>>>(g);
+        (mode == LeafMode::kBesideRender && !few ? beside : alone)<<<(unsigned)blocks, kLeafThreads, 0, stream>>>(g);
         return cudaGetLastError();
     }
     const cudaError_t e = launch_norm_keys(g, (uint64_t)num_sms, stream);
@@ -620,12 +776,12 @@ int tree_top_kernels(const TreeTop &t) {
 
 namespace {
 
-// node_begin for one thread per node of level `k`: each fragment's nodes rounded up to whole
-// warps, so that no warp holds nodes of two fragments.
+// node_begin for level `k`: each fragment's nodes rounded up to the children of one parent, so
+// that no tree-top block holds nodes of two.
 void count_level(TreeTop &t, uint32_t k) {
     for (uint32_t i = 0; i < t.count; ++i) {
         const uint64_t nodes = k < t.frag[i].levels ? t.frag[i].size[k] : 0;
-        t.node_begin[i + 1] = t.node_begin[i] + (nodes + kInnerThreads - 1) / kInnerThreads * kInnerThreads;
+        t.node_begin[i + 1] = t.node_begin[i] + (nodes + kFanout - 1) / kFanout * kFanout;
     }
 }
 
@@ -641,12 +797,12 @@ cudaError_t launch_tree_top(const TreeTop &in, cudaStream_t stream) {
     if (level1_nodes(in) < kSplitLevel1Nodes)
         // one launch from level 1: the level-2 parents are hashed by the warps that hash their
         // children, with no second launch
-        return launch_after(tree_top_kernel<1>, total1 / kInnerThreads, kInnerThreads, stream, t);
+        return launch_after(tree_top_kernel<1>, total1 / kFanout, kTopThreads, stream, t);
     const cudaError_t e = launch_after(level1_kernel, (total1 + kLevel1Threads - 1) / kLevel1Threads,
                                        kLevel1Threads, stream, t);
     if (e != cudaSuccess || kernels == 1) return e;
     count_level(t, 2);
-    return launch_after(tree_top_kernel<2>, t.node_begin[t.count] / kInnerThreads, kInnerThreads, stream, t);
+    return launch_after(tree_top_kernel<2>, t.node_begin[t.count] / kFanout, kTopThreads, stream, t);
 }
 
 cudaError_t launch_compare(const void *a, const void *b, uint64_t bytes, unsigned int *flag,

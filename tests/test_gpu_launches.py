@@ -1,6 +1,6 @@
 """The edges of the content address's launches: heads per norm-key thread, tree levels at the
-edge of a warp (whose lanes hand digests to their parents) with several fragments in one
-launch, and the sizes at which cm_ingest_render starts its render beside the leaf hash, as
+edge of a block (which hands its digests to their parent) with several fragments in one
+launch, leaves on both sides of the switch from four lanes each to one, and the sizes at which cm_ingest_render starts its render beside the leaf hash, as
 the leaves end, or beside it again. Ids and norm keys equal the oracle's; the merges' bytes
 equal those of the separate calls."""
 import numpy as np
@@ -48,9 +48,9 @@ def test_norm_key_over_head_counts(ctx, H, T):
 
 
 # a token is 1 KiB = one leaf here, so T tokens have ceil(T / 16) level-1 nodes
-@pytest.mark.parametrize("lengths", [(1, 16, 17), (256, 257, 255), (511, 512, 513),
+@pytest.mark.parametrize("lengths", [(1, 16, 17), (256, 257, 255), (511, 512, 513), (9600, 128), (9600, 129),
                                      (8191, 1, 8193), (4096, 4097, 300)])
-def test_tree_levels_at_warp_edges(ctx, lengths):
+def test_tree_levels_at_block_edges(ctx, lengths):
     frags = [_fragment(7 * T + i, 1, 1, T, 256) for i, T in enumerate(lengths)]
     S = cm.FragmentSet(ctx)
     res = S.ingest_batch(frags)
@@ -95,11 +95,13 @@ def test_ingest_render_start_rules_give_the_separate_calls_bytes(ctx, lengths, p
 # planes that are no multiple of a 1 KiB leaf: leaves that run into one or many further
 # segments, short last leaves, alone and in one launch with whole ones
 @pytest.mark.parametrize("shape", [(2, 1, 1, 16), (40, 1, 1, 16), (9, 1, 3, 32), (3, 3, 11, 16),
-                                   (4, 2, 37, 64), (5, 1, 63, 128), (6, 3, 5, 512)])
+                                   (4, 2, 37, 64), (5, 1, 63, 128), (6, 3, 5, 512),
+                                   (8, 3, 3201, 64)])
 def test_leaves_that_straddle_segments(ctx, shape):
     L, H, T, d = shape
     K, V = _fragment(sum(shape), L, H, T, d)
     whole = _fragment(3, L, H, 1024, d)   # 1024 rows to a head: every plane whole leaves
+    # (the last shape has more leaves than are hashed by four lanes each)
     S = cm.FragmentSet(ctx)
     res = S.ingest_batch([(K, V)])
     assert res[0][0] == oracle_fragment(K, V).fid
