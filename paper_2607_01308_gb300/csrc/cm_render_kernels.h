@@ -58,17 +58,17 @@ struct RenderParams {
     double cs[2 * kMaxTablePairs];   // (cos a, sin a) of a = s * theta^(-2j/d), interleaved
 };
 
-// How much of each SM a render takes:
-//   kFull         the register kernel, 3 CTAs of 8 warps per SM (cm_context_set_render_warps(16),
-//                 the default): the fastest render alone
-//   kHalf         the TMA kernel, one CTA of 8 warps (3 stages each) per SM
-//                 (cm_context_set_render_warps(8)): half of each SM's registers stay free for
-//                 kernels of other streams
-//   kBeside       the TMA kernel, one CTA of 4 warps (6 stages each) per SM: a large render
-//                 beside the leaf hash of the same merge (cm_ingest_render)
+// How much of each SM a render takes (the TMA kernel's widths are in render.cu):
+//   kFull         the TMA kernel, 20 warps per SM (cm_context_set_render_warps(16), the
+//                 default): the fastest render alone
+//   kHalf         the TMA kernel, 8 warps per SM (cm_context_set_render_warps(8)): half of each
+//                 SM's registers stay free for kernels of other streams
+//   kBeside       the TMA kernel, 4 warps per SM: a large render beside the leaf hash of the same
+//                 merge (cm_ingest_render, contiguous outputs)
 //   kBesideSmall  the register kernel, one 8-warp CTA per SM: a small render beside the leaf hash
+//                 (contiguous outputs)
 //   kAfterLeaves  the register kernel, two 8-warp CTAs per SM: a middling render that starts as
-//                 the leaf hash ends and leaves the tree levels room on every SM
+//                 the leaf hash ends and leaves the tree levels room on every SM (contiguous)
 // A launch group's work items are row chunks of render_item_bytes(w) bytes of one source
 // plane; render_grid gives the launch's CTA count for `chunks` items. render_prepare() once
 // per device before the first launch.

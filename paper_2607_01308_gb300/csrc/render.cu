@@ -10,20 +10,15 @@
 // turned by one constant angle a_j = s * theta^(-2j/d) per frequency j (the delta
 // formula of Section 2.3), pairing element j with element j + d/2.
 //
-// Two kernels move the items. The full-SM render (render_reg_kernel, the default) has
-// every warp take one (K, V) pair of 1 KiB items at a time: its lanes load both items
-// as 16-byte vectors straight into registers, rotate the K rows, and store both with
-// streaming stores; 24 warps per SM keep about 48 KiB of loads in flight, where HBM
-// serves this mix of reads and writes best (more bytes in flight made the same copy
-// slower). The half-SM render (render_kernel, cm_context_set_render_warps(8)) runs one
-// 8-warp CTA per SM that leaves half of the register file to kernels of other
-// streams; its warps keep three 4 KiB items in flight each as 1-D TMA bulk copies
-// into shared memory, which needs fewer warps for the same bytes in flight. For a
-// rotated K item a lane takes vector v of a row's first half and vector v of its
-// second half: 8 (x, y) pairs that share the lane's 8 (cos, sin) values. A render that
-// runs beside the content address (cm_ingest_render) takes a narrower width still: the
-// TMA kernel with one CTA of 4 warps and 6 stages per SM for large renders, the register
-// kernel with one or two 8-warp CTAs per SM for smaller ones (see RenderWidth).
+// Two kernels move the items. In the TMA kernel (render_kernel) every warp keeps its items in
+// flight as 1-D bulk copies into its stages of shared memory; the full-SM render (the default)
+// takes an item from its stage into registers and refills the stage before it rotates and
+// stores, so that a steady 40 KiB of loads per SM is in flight, where HBM serves this mix of
+// reads and writes best (see TmaWidth, which gives its widths and what they measured). The
+// register kernel (render_reg_kernel) loads straight into registers and serves the small and
+// middling merges beside the content address (see RenderWidth). For a rotated K item a lane
+// takes vector v of a row's first half and vector v of its second half: 8 (x, y) pairs that
+// share the lane's 8 (cos, sin) values.
 //
 // Rounding. The result must equal round-to-nearest-even-bf16 of
 // fl64(fl64(x c) - fl64(y s)) (and fl64(fl64(y c) + fl64(x s))), c and s the fp64
@@ -188,38 +183,29 @@ __device__ __noinline__ uint32_t fix_element(float x, float y, float4 t, double 
     return out;
 }
 
-__device__ __forceinline__ uint32_t pick_word(const uint4 &v, int w) {
-    return w == 0 ? v.x : w == 1 ? v.y : w == 2 ? v.z : v.w;
-}
-
-__device__ __forceinline__ void put_half(uint4 &v, int e, uint32_t bits) {
-    const int w = e >> 1;
-    const uint32_t keep = (e & 1) ? 0x0000FFFFu : 0xFFFF0000u;
-    const uint32_t val = (e & 1) ? (bits << 16) : bits;
-    if (w == 0) v.x = (v.x & keep) | val;
-    else if (w == 1) v.y = (v.y & keep) | val;
-    else if (w == 2) v.z = (v.z & keep) | val;
-    else v.w = (v.w & keep) | val;
-}
-
 // Re-evaluates the elements of one vector pair whose masks b0..b3 flag them. Inlined: as a
-// called function its call (argument and result registers, a stack frame) cost the
-// full-SM render 0.80 instead of 0.754 ms on the Qwen3-4B-shaped merge, though only about
-// one warp iteration in twenty takes it.
+// called function its call (argument and result registers, a stack frame) cost the register
+// render 0.80 instead of 0.754 ms on the Qwen3-4B-shaped merge, though only about one warp
+// iteration in twenty takes it.
 __device__ __forceinline__ void fixup_pair(const RenderParams &p, const float4 *tab, int cs_index,
                                         const uint4 &a, const uint4 &b, uint32_t b0, uint32_t b1,
                                         uint32_t b2, uint32_t b3, uint4 &ao, uint4 &bo) {
-    const uint32_t bw[4] = {b0, b1, b2, b3};
-    for (int e = 0; e < 8; ++e) {
-        const uint32_t m = bw[e >> 1] >> ((e & 1) * 16);
-        if ((m & 0xFFFFu) == 0u) continue;
-        const uint32_t xw = pick_word(a, e >> 1), yw = pick_word(b, e >> 1);
-        const float x = (e & 1) ? bf16_hi(xw) : bf16_lo(xw);
-        const float y = (e & 1) ? bf16_hi(yw) : bf16_lo(yw);
-        const uint32_t r = fix_element(x, y, tab[cs_index + e], p.cs[2 * (cs_index + e)],
-                                       p.cs[2 * (cs_index + e) + 1]);
-        put_half(ao, e, r & 0xFFFFu);
-        put_half(bo, e, r >> 16);
+    const uint32_t bw[4] = {b0, b1, b2, b3}, xw[4] = {a.x, a.y, a.z, a.w}, yw[4] = {b.x, b.y, b.z, b.w};
+    uint32_t *ow[4] = {&ao.x, &ao.y, &ao.z, &ao.w}, *pw[4] = {&bo.x, &bo.y, &bo.z, &bo.w};
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+        if (bw[w] == 0u) continue;
+        const int c0 = cs_index + 2 * w;
+        if (bw[w] & 0xFFFFu) {
+            const uint32_t r = fix_element(bf16_lo(xw[w]), bf16_lo(yw[w]), tab[c0], p.cs[2 * c0], p.cs[2 * c0 + 1]);
+            *ow[w] = (*ow[w] & 0xFFFF0000u) | (r & 0xFFFFu);
+            *pw[w] = (*pw[w] & 0xFFFF0000u) | (r >> 16);
+        }
+        if (bw[w] >> 16) {
+            const uint32_t r = fix_element(bf16_hi(xw[w]), bf16_hi(yw[w]), tab[c0 + 1], p.cs[2 * c0 + 2], p.cs[2 * c0 + 3]);
+            *ow[w] = (*ow[w] & 0xFFFFu) | (r << 16);
+            *pw[w] = (*pw[w] & 0xFFFFu) | (r & 0xFFFF0000u);
+        }
     }
 }
 
@@ -286,16 +272,35 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
-constexpr int kStagesDefault = 3;                   // per warp
-constexpr uint32_t kItemBytes = 4096;               // one work item = one stage
-// Per frequency: (c1, c2, s1, s2), then the first-level bound scale k, -s32, c32 and s32
-// (one array of kMaxTablePairs each), so that an item's 8 fp32 (cos, sin) are 4 loads
-constexpr size_t kTableBytes = (sizeof(float4) + 4 * sizeof(float)) * kMaxTablePairs;
-// Dynamic shared memory of a CTA of kW warps: the warps' stages, then the (cos, sin) table.
-template <int kW, int kStages = kStagesDefault>
-constexpr size_t dyn_smem() { return (size_t)kW * kStages * kItemBytes + kTableBytes; }
+// The TMA kernel's widths: warps per CTA (one CTA per SM), bytes of a work item (= of a stage)
+// and stages per warp. More loads in flight per SM than these make HBM serve this mix of reads
+// and writes worse (a plain copy kernel took 0.70 ms for 2.4 GB with 28 to 32 KiB in flight per
+// SM, 0.75 with 40 and more), fewer leave it idle; larger items cost fewer instructions each.
+//   full        20 warps, 2 KiB, through registers: measured for 4 x 4096 tokens / paged 5,208
+//               tokens 716 / 239 us; 16, 19, 21, 24 warps 742 / 258, 747 / 254, 759 / 260,
+//               764 / 267; 4 KiB at 11 warps 715 / 265; not through registers 735 / 277; as the
+//               register kernel below, three CTAs per SM, 752 / 251
+//   half        8 warps, 4 KiB, two stages (paged: three): 750 / 248 us alone, with three
+//               805 / 248, with two 750 / 257; a serving group hashed beside it 5.81 ms with
+//               two, 5.98 with three
+//   beside      4 warps, 16 KiB, two stages: the 4 x 4096-token merge 1.597 ms, 4 x 2048 841 us;
+//               8 KiB x 2 1.599, 849; 8 KiB x 3 1.612, 849; 4 KiB x 6 1.647, 865
+struct TmaWidth {
+    int warps, stages;
+    uint32_t item_bytes;
+};
+constexpr TmaWidth kFullWidth{20, 1, 2048}, kHalfWidth{8, 2, 4096}, kHalfPagedWidth{8, 3, 4096},
+    kBesideWidth{4, 2, 16384};
 
-// One work item: up to kItemBytes of one source plane and where it goes.
+// Per frequency of the launch's slots: (c1, c2, s1, s2), then the first-level bound scale k,
+// -s32, c32 and s32 (one array each), so that an item's 8 fp32 (cos, sin) are 4 loads
+constexpr size_t kTableEntryBytes = sizeof(float4) + 4 * sizeof(float);
+// Dynamic shared memory of a CTA: the warps' stages, then the (cos, sin) table of `entries`.
+constexpr size_t dyn_smem(TmaWidth w, int entries) {
+    return (size_t)w.warps * w.stages * w.item_bytes + kTableEntryBytes * entries;
+}
+
+// One work item: up to an item's bytes of one source plane and where it goes.
 struct Item {
     const uint8_t *src;
     uint8_t *dst;        // contiguous: first output row; paged: pool + (layer, head) offset
@@ -386,37 +391,109 @@ __device__ __forceinline__ uint4 *row_dst(const RenderParams &p, const Item &it,
     return reinterpret_cast<uint4 *>(it.dst + (blk * p.stride_block + o * p.stride_token) * 2);
 }
 
-// Byte copy of one staged item: shared memory -> registers -> 16-byte streaming stores.
-template <bool kPaged>
-__device__ __forceinline__ void copy_from_smem(const RenderParams &p, const Item &it,
-                                               const uint8_t *buf, int lane) {
-    constexpr int kU = kItemBytes / 16 / 32;          // 8 vectors per lane
+// Vectors v0 + lane, v0 + lane + 32, ... of an item from registers to their place in the output,
+// as 16-byte streaming stores.
+template <bool kPaged, int kU>
+__device__ __forceinline__ void copy_from_regs(const RenderParams &p, const Item &it, int v0,
+                                               const uint4 (&r)[kU], int lane) {
     const int n_vec = (int)(it.bytes >> 4);
-    const uint4 *src = reinterpret_cast<const uint4 *>(buf);
     PagedRows pr{};
     if (kPaged) pr = paged_rows(p, it);
-    uint4 r[kU];
+    const int log2_vpr = p.log2_pairs_per_row + 1;     // vectors per row = d / 8
+    const int col_mask = (1 << log2_vpr) - 1;
 #pragma unroll
-    for (int u = 0; u < kU; ++u)
-        if (lane + 32 * u < n_vec) r[u] = src[lane + 32 * u];
-    if (!kPaged) {
-        uint4 *dst = reinterpret_cast<uint4 *>(it.dst);
-#pragma unroll
-        for (int u = 0; u < kU; ++u)
-            if (lane + 32 * u < n_vec && CM_IN_BOUNDS(dst + lane + 32 * u, 16, it.dst_base, it.dst_size))
-                st_stream(dst + lane + 32 * u, r[u]);
-    } else {
-        const int log2_vpr = p.log2_pairs_per_row + 1;     // vectors per row = d / 8
-        const int col_mask = (1 << log2_vpr) - 1;
-#pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            const int v = lane + 32 * u;
-            if (v < n_vec) {
-                uint4 *q = row_dst<true>(p, it, v >> log2_vpr, pr) + (v & col_mask);
-                if (CM_IN_BOUNDS(q, 16, it.dst_base, it.dst_size)) st_stream(q, r[u]);
-            }
+    for (int u = 0; u < kU; ++u) {
+        const int v = v0 + lane + 32 * u;
+        if (v < n_vec) {
+            uint4 *d = kPaged ? row_dst<true>(p, it, v >> log2_vpr, pr) + (v & col_mask)
+                              : reinterpret_cast<uint4 *>(it.dst) + v;
+            if (CM_IN_BOUNDS(d, 16, it.dst_base, it.dst_size)) st_stream(d, r[u]);
         }
     }
+}
+
+// Byte copy of one staged item through registers, 8 vectors per lane at a time.
+template <bool kPaged, uint32_t kItem>
+__device__ __forceinline__ void copy_from_smem(const RenderParams &p, const Item &it,
+                                               const uint8_t *buf, int lane) {
+    constexpr int kU = 8;
+    const int n_vec = (int)(it.bytes >> 4);
+    const uint4 *src = reinterpret_cast<const uint4 *>(buf);
+#pragma unroll
+    for (int v0 = 0; v0 < (int)(kItem / 16); v0 += 32 * kU) {
+        uint4 r[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u)
+            if (v0 + lane + 32 * u < n_vec) r[u] = src[v0 + lane + 32 * u];
+        copy_from_regs<kPaged>(p, it, v0, r, lane);
+    }
+}
+
+// The lane's vectors of a staged item that is copied: lane, lane + 32, ...
+template <int kU>
+__device__ __forceinline__ void vecs_from_smem(const Item &it, const uint8_t *buf, int lane, uint4 (&r)[kU]) {
+    const uint4 *src = reinterpret_cast<const uint4 *>(buf);
+#pragma unroll
+    for (int u = 0; u < kU; ++u)
+        if (lane + 32 * u < (int)(it.bytes >> 4)) r[u] = src[lane + 32 * u];
+}
+
+// The lane's vector pairs of a staged item that is rotated: pairs lane, lane + 32, ..., each the
+// vectors lane_v of a row's first and second half.
+template <int kU>
+__device__ __forceinline__ void pairs_from_smem(const RenderParams &p, const Item &it, const uint8_t *buf,
+                                                int lane, int lane_v, uint4 (&r)[kU]) {
+    const uint4 *src = reinterpret_cast<const uint4 *>(buf);
+    const int half_vecs = p.head_dim >> 4, n_pairs = it.rows * half_vecs;
+#pragma unroll
+    for (int k = 0; k < kU / 2; ++k) {
+        const int q = lane + 32 * k;
+        const int off = (q >> p.log2_pairs_per_row) * 2 * half_vecs + lane_v;
+        if (q < n_pairs) {
+            r[2 * k] = src[off];
+            r[2 * k + 1] = src[off + half_vecs];
+        }
+    }
+}
+
+// A lane's 8 (cos, sin) as fp32, from frequency cs_index on.
+__device__ __forceinline__ void load_cos_sin(const float *c32, const float *s32, int cs_index, float (&c)[8],
+                                             float (&s)[8]) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const float4 cv = *reinterpret_cast<const float4 *>(c32 + cs_index + 4 * h);
+        const float4 sv = *reinterpret_cast<const float4 *>(s32 + cs_index + 4 * h);
+        c[4 * h] = cv.x, c[4 * h + 1] = cv.y, c[4 * h + 2] = cv.z, c[4 * h + 3] = cv.w;
+        s[4 * h] = sv.x, s[4 * h + 1] = sv.y, s[4 * h + 2] = sv.z, s[4 * h + 3] = sv.w;
+    }
+}
+
+// Rotates one vector pair (a from a row's first half, b from its second; frequencies cs_index to
+// cs_index + 7 with cosines c and sines s) into ao and bo.
+__device__ __forceinline__ void rotate_vectors(const RenderParams &p, const float4 *tab, const float *kt,
+                                               const float *nst, int cs_index, const float (&c)[8],
+                                               const float (&s)[8], const uint4 &a, const uint4 &b,
+                                               uint4 &ao, uint4 &bo) {
+    const float4 ka = *reinterpret_cast<const float4 *>(kt + cs_index);
+    const float4 kb = *reinterpret_cast<const float4 *>(kt + cs_index + 4);
+    const float4 na = *reinterpret_cast<const float4 *>(nst + cs_index);
+    const float4 nb = *reinterpret_cast<const float4 *>(nst + cs_index + 4);
+    uint32_t b0, b1, b2, b3;
+    rotate_word(a.x, b.x, c[0], s[0], na.x, ka.x, c[1], s[1], na.y, ka.y, ao.x, bo.x, b0);
+    rotate_word(a.y, b.y, c[2], s[2], na.z, ka.z, c[3], s[3], na.w, ka.w, ao.y, bo.y, b1);
+    rotate_word(a.z, b.z, c[4], s[4], nb.x, kb.x, c[5], s[5], nb.y, kb.y, ao.z, bo.z, b2);
+    rotate_word(a.w, b.w, c[6], s[6], nb.z, kb.z, c[7], s[7], nb.w, kb.w, ao.w, bo.w, b3);
+    if ((b0 | b1 | b2 | b3) != 0u) fixup_pair(p, tab, cs_index, a, b, b0, b1, b2, b3, ao, bo);
+}
+
+// Stores a rotated vector pair of row `row` of an item.
+template <bool kPaged>
+__device__ __forceinline__ void store_pair(const RenderParams &p, const Item &it, const PagedRows &pr, int row,
+                                           int lane_v, const uint4 &ao, const uint4 &bo) {
+    const int half_vecs = p.head_dim >> 4;
+    uint4 *d = row_dst<kPaged>(p, it, row, pr) + lane_v;
+    if (CM_IN_BOUNDS(d, 16, it.dst_base, it.dst_size)) st_stream(d, ao);
+    if (CM_IN_BOUNDS(d + half_vecs, 16, it.dst_base, it.dst_size)) st_stream(d + half_vecs, bo);
 }
 
 // K rows of one staged item: rotate and store. Lane `lane` takes vector pairs
@@ -427,41 +504,45 @@ __device__ __forceinline__ void rotate_from_smem(const RenderParams &p, const fl
                                                  const float *kt, const float *nst, const float *c32,
                                                  const float *s32, const Item &it,
                                                  const uint8_t *buf, int lane, int lane_v) {
-    const int vecs_per_row = p.head_dim >> 3;
     const int half_vecs = p.head_dim >> 4;
     const int n_pairs = it.rows * half_vecs;
     const int cs_index = it.cs_index + 8 * lane_v;
     PagedRows pr{};
     if (kPaged) pr = paged_rows(p, it);
     float c[8], s[8];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const float4 cv = *reinterpret_cast<const float4 *>(c32 + cs_index + 4 * h);
-        const float4 sv = *reinterpret_cast<const float4 *>(s32 + cs_index + 4 * h);
-        c[4 * h] = cv.x, c[4 * h + 1] = cv.y, c[4 * h + 2] = cv.z, c[4 * h + 3] = cv.w;
-        s[4 * h] = sv.x, s[4 * h + 1] = sv.y, s[4 * h + 2] = sv.z, s[4 * h + 3] = sv.w;
-    }
+    load_cos_sin(c32, s32, cs_index, c, s);
     const uint4 *src = reinterpret_cast<const uint4 *>(buf);
 #pragma unroll 1
     for (int q = lane; q < n_pairs; q += 32) {
         const int row = q >> p.log2_pairs_per_row;
-        const int off = row * vecs_per_row + lane_v;
-        const uint4 a = src[off];
-        const uint4 b = src[off + half_vecs];
-        const float4 ka = *reinterpret_cast<const float4 *>(kt + cs_index);
-        const float4 kb = *reinterpret_cast<const float4 *>(kt + cs_index + 4);
-        const float4 na = *reinterpret_cast<const float4 *>(nst + cs_index);
-        const float4 nb = *reinterpret_cast<const float4 *>(nst + cs_index + 4);
+        const int off = row * 2 * half_vecs + lane_v;
+        const uint4 a = src[off], b = src[off + half_vecs];
         uint4 ao, bo;
-        uint32_t b0, b1, b2, b3;
-        rotate_word(a.x, b.x, c[0], s[0], na.x, ka.x, c[1], s[1], na.y, ka.y, ao.x, bo.x, b0);
-        rotate_word(a.y, b.y, c[2], s[2], na.z, ka.z, c[3], s[3], na.w, ka.w, ao.y, bo.y, b1);
-        rotate_word(a.z, b.z, c[4], s[4], nb.x, kb.x, c[5], s[5], nb.y, kb.y, ao.z, bo.z, b2);
-        rotate_word(a.w, b.w, c[6], s[6], nb.z, kb.z, c[7], s[7], nb.w, kb.w, ao.w, bo.w, b3);
-        if ((b0 | b1 | b2 | b3) != 0u) fixup_pair(p, tab, cs_index, a, b, b0, b1, b2, b3, ao, bo);
-        uint4 *d = row_dst<kPaged>(p, it, row, pr) + lane_v;
-        if (CM_IN_BOUNDS(d, 16, it.dst_base, it.dst_size)) st_stream(d, ao);
-        if (CM_IN_BOUNDS(d + half_vecs, 16, it.dst_base, it.dst_size)) st_stream(d + half_vecs, bo);
+        rotate_vectors(p, tab, kt, nst, cs_index, c, s, a, b, ao, bo);
+        store_pair<kPaged>(p, it, pr, row, lane_v, ao, bo);
+    }
+}
+
+// The same for the pairs that pairs_from_smem loaded.
+template <bool kPaged, int kU>
+__device__ __forceinline__ void rotate_from_regs(const RenderParams &p, const float4 *tab,
+                                                 const float *kt, const float *nst, const float *c32,
+                                                 const float *s32, const Item &it,
+                                                 const uint4 (&r)[kU], int lane, int lane_v) {
+    const int n_pairs = it.rows * (p.head_dim >> 4);
+    const int cs_index = it.cs_index + 8 * lane_v;
+    PagedRows pr{};
+    if (kPaged) pr = paged_rows(p, it);
+    float c[8], s[8];
+    load_cos_sin(c32, s32, cs_index, c, s);
+#pragma unroll
+    for (int k = 0; k < kU / 2; ++k) {
+        const int q = lane + 32 * k;
+        if (q >= n_pairs) break;
+        const uint4 a = r[2 * k], b = r[2 * k + 1];   // copies, which the fix-up also reads
+        uint4 ao, bo;
+        rotate_vectors(p, tab, kt, nst, cs_index, c, s, a, b, ao, bo);
+        store_pair<kPaged>(p, it, pr, q >> p.log2_pairs_per_row, lane_v, ao, bo);
     }
 }
 
@@ -602,19 +683,17 @@ __device__ __forceinline__ Item half_item(const Pair &q, bool v) {
     return it;
 }
 
-// Half-SM render: a persistent kernel with one CTA of kW = 8 warps per SM (half of the
-// register file, leaving room for kernels of other streams on the same SMs; kW = 4 with 6
-// stages beside the leaf hash); every warp runs its own pipeline over its own items, with
-// no block-wide barrier after set-up. Items come in (K, V) pairs of the same (slot, layer,
-// head, row chunk); a warp takes pairs warp id + m * total warps and does the K item,
-// then the V item, so rotation work and pure copies alternate within every warp. Lane 0
-// keeps up to kStages items in flight as 1-D TMA bulk loads into the warp's stages
-// (completion on one mbarrier per stage); all lanes wait for an item, move it from shared
-// memory to its place in the output (rotating K rows of slots at a nonzero offset; kPaged:
-// each row's place comes from the block table), and lane 0 refills the stage with the
-// warp's next item. Every wait is bounded: on timeout the warp records an error, waits
-// (bounded) for its own copies in flight and returns.
-template <bool kPaged, int kW, int kStages = kStagesDefault, int kMinBlocks = 16 / kW>
+// The TMA render: a persistent kernel with one CTA of kW warps per SM; every warp runs its own
+// pipeline over its own items, with no block-wide barrier after set-up. Items come in (K, V)
+// pairs of the same (slot, layer, head, row chunk); a warp takes pairs warp id + m * total warps
+// and does the K item, then the V item, so rotation work and pure copies alternate within every
+// warp. Lane 0 keeps up to kStages items in flight as 1-D TMA bulk loads into the warp's stages
+// (completion on one mbarrier per stage); all lanes wait for an item, move it to its place in
+// the output (rotating K rows of slots at a nonzero offset; kPaged: each row's place comes from
+// the block table), and lane 0 refills the stage with the warp's next item, kThroughRegs as
+// soon as the lanes hold the item in registers. Every wait is bounded: on timeout the warp
+// records an error, waits (bounded) for its own copies in flight and returns.
+template <bool kPaged, int kW, int kStages, uint32_t kItem, int kMinBlocks, bool kThroughRegs>
 __global__ void __launch_bounds__(kW * 32, kMinBlocks)
 render_kernel(const __grid_constant__ RenderParams p) {
     constexpr int kThreads = kW * 32;
@@ -625,14 +704,14 @@ render_kernel(const __grid_constant__ RenderParams p) {
     __shared__ __align__(8) uint64_t full[kW][kStages];
     __shared__ Item items[kW][kRing];
     __shared__ PairWalk walks[kW];   // lane 0's position along its warp's pairs
-    float4 *tab = reinterpret_cast<float4 *>(smem + (size_t)kW * kStages * kItemBytes);
-    float *kt = reinterpret_cast<float *>(tab + kMaxTablePairs);
-    float *nst = kt + kMaxTablePairs;
-    float *c32 = nst + kMaxTablePairs;
-    float *s32 = c32 + kMaxTablePairs;
-
     const int half = p.head_dim >> 1;
     const int n_table = p.num_slots * half;
+    float4 *tab = reinterpret_cast<float4 *>(smem + (size_t)kW * kStages * kItem);
+    float *kt = reinterpret_cast<float *>(tab + n_table);
+    float *nst = kt + n_table;
+    float *c32 = nst + n_table;
+    float *s32 = c32 + n_table;
+
     for (int i = threadIdx.x; i < n_table; i += kThreads) {
         const float2 cc = split16(p.cs[2 * i]), ss = split16(p.cs[2 * i + 1]);
         tab[i] = make_float4(cc.x, cc.y, ss.x, ss.y);
@@ -648,12 +727,14 @@ render_kernel(const __grid_constant__ RenderParams p) {
     }
     __syncthreads();
 
-    const uint32_t first = blockIdx.x * kW + warp;
     const uint32_t stride = gridDim.x * kW;
     const uint32_t npairs = p.total_chunks / 2;
+    // neighbouring pairs to neighbouring warps; a launch of fewer pairs than warps spreads over
+    // the SMs first
+    const uint32_t first = npairs < stride ? warp * gridDim.x + blockIdx.x : blockIdx.x * kW + warp;
     const uint32_t n = npairs > first ? 2 * ((npairs - first + stride - 1) / stride) : 0;
     const int lane_v = lane & ((p.head_dim >> 4) - 1);
-    uint8_t *wbuf = smem + (size_t)warp * kStages * kItemBytes;
+    uint8_t *wbuf = smem + (size_t)warp * kStages * kItem;
 
     // Item j: pair j / 2 of the warp (pairs first, first + stride, ...), K if j is even, V if
     // odd. Lane 0 walks the pairs by additions and writes a pair's two Items at once, the V
@@ -690,7 +771,7 @@ render_kernel(const __grid_constant__ RenderParams p) {
         const bool src_ok = CM_IN_BOUNDS(it.src, it.bytes, it.src_base, it.src_size);
         mbar_arrive_expect_tx(&full[warp][s], src_ok ? it.bytes : 0u);
         if (j == 0 && p.withhold_warp == first + 1) return;   // injected: the wait runs out
-        if (src_ok) bulk_load(wbuf + (size_t)s * kItemBytes, it.src, it.bytes, &full[warp][s]);
+        if (src_ok) bulk_load(wbuf + (size_t)s * kItem, it.src, it.bytes, &full[warp][s]);
     };
 
     uint32_t produced = 0;
@@ -707,15 +788,31 @@ render_kernel(const __grid_constant__ RenderParams p) {
             break;
         }
         const Item it = items[warp][i % kRing];
-        const uint8_t *buf = wbuf + (size_t)s * kItemBytes;
-        if (it.rotate)
-            rotate_from_smem<kPaged>(p, tab, kt, nst, c32, s32, it, buf, lane, lane_v);
-        else
-            copy_from_smem<kPaged>(p, it, buf, lane);
-        __syncwarp();                          // every lane is done reading stage s
-        if (lane == 0 && produced < n) {
-            fence_proxy_async_smem();
-            produce(produced++);               // item i + kStages into stage s
+        const uint8_t *buf = wbuf + (size_t)s * kItem;
+        auto refill = [&] {
+            __syncwarp();                      // every lane is done reading stage s
+            if (lane == 0 && produced < n) {
+                fence_proxy_async_smem();
+                produce(produced++);           // item i + kStages into stage s
+            }
+        };
+        if (kThroughRegs) {
+            uint4 r[kItem / 512];
+            if (it.rotate) {
+                pairs_from_smem(p, it, buf, lane, lane_v, r);
+                refill();
+                rotate_from_regs<kPaged>(p, tab, kt, nst, c32, s32, it, r, lane, lane_v);
+            } else {
+                vecs_from_smem(it, buf, lane, r);
+                refill();
+                copy_from_regs<kPaged>(p, it, 0, r, lane);
+            }
+        } else {
+            if (it.rotate)
+                rotate_from_smem<kPaged>(p, tab, kt, nst, c32, s32, it, buf, lane, lane_v);
+            else
+                copy_from_smem<kPaged, kItem>(p, it, buf, lane);
+            refill();
         }
     }
     if (aborted && lane == 0) {
@@ -725,78 +822,44 @@ render_kernel(const __grid_constant__ RenderParams p) {
     }
 }
 
-template <bool kPaged, int kW, int kStages = kStagesDefault, int kMinBlocks = 16 / kW>
-cudaError_t set_smem_attribute() {
-    return cudaFuncSetAttribute(render_kernel<kPaged, kW, kStages, kMinBlocks>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)dyn_smem<kW, kStages>());
+using RenderKernel = void (*)(RenderParams);
+
+// The instance of a TMA width. Minimum CTAs per SM bound the registers: 2 at half width (half of
+// the register file), 4 beside the leaf hash.
+RenderKernel tma_kernel(RenderWidth w, bool paged) {
+    constexpr TmaWidth f = kFullWidth, h = kHalfWidth, hp = kHalfPagedWidth, b = kBesideWidth;
+    switch (w) {
+        case RenderWidth::kHalf:
+            return paged ? render_kernel<true, hp.warps, hp.stages, hp.item_bytes, 2, false>
+                         : render_kernel<false, h.warps, h.stages, h.item_bytes, 2, false>;
+        case RenderWidth::kBeside:   // contiguous outputs only
+            return render_kernel<false, b.warps, b.stages, b.item_bytes, 4, false>;
+        default:
+            return paged ? render_kernel<true, f.warps, f.stages, f.item_bytes, 1, true>
+                         : render_kernel<false, f.warps, f.stages, f.item_bytes, 1, true>;
+    }
 }
 
-// ---------------------------------------------------------------- full-SM render
+TmaWidth tma_width(RenderWidth w, bool paged) {
+    return w == RenderWidth::kHalf ? (paged ? kHalfPagedWidth : kHalfWidth)
+                                   : w == RenderWidth::kBeside ? kBesideWidth : kFullWidth;
+}
+
+bool is_tma(RenderWidth w) { return w != RenderWidth::kBesideSmall && w != RenderWidth::kAfterLeaves; }
+
+// ---------------------------------------------------------------- register render
 
 constexpr int kRegThreads = 256;           // 8 warps per CTA
-constexpr int kRegBlocksPerSm = 3;         // 24 warps per SM
+constexpr int kRegBlocksPerSm = 3;         // at most (80 registers)
 constexpr uint32_t kRegItemBytes = 1024;   // one work item: 2 vectors per lane
 constexpr int kRegVecs = kRegItemBytes / 16 / 32;
 
-// Paged outputs: where the rows of a pair go, for K and V alike (the two halves differ only
-// in their pool). When the block size is a power of two no smaller than the pair's row
-// count, the rows lie in at most two logical blocks: row r goes to half + da + r * stride
-// before the block boundary (r < split), to half + db + r * stride after it, the block
-// table read once per pair; otherwise (fast false) every row looks its block up.
-struct PagedOffsets {
-    int64_t da, db, stride;
-    int split;
-    bool fast;
-};
-
-__device__ __forceinline__ PagedOffsets paged_offsets(const RenderParams &p, int64_t pos0, int rows) {
-    PagedOffsets o;
-    o.fast = p.log2_block_size >= 0 && (int64_t)rows <= p.block_size;
-    o.stride = p.stride_token * 2;
-    o.split = rows;
-    o.da = o.db = 0;
-    if (o.fast) {
-        const int64_t b0 = pos0 >> p.log2_block_size;
-        const int64_t o0 = pos0 & (p.block_size - 1);
-        const int64_t k = p.block_size - o0;                 // rows left in block b0
-        o.da = table_entry(p, b0) * p.stride_block * 2 + o0 * o.stride;
-        if (k < rows) {
-            o.split = (int)k;
-            o.db = table_entry(p, b0 + 1) * p.stride_block * 2 - k * o.stride;
-        }
-    }
-    return o;
-}
-
-// Row r of one half of a pair (half = the half's item).
-template <bool kPaged>
-__device__ __forceinline__ uint4 *pair_row(const RenderParams &p, const Item &half,
-                                           const PagedOffsets &po, int r) {
-    if (!kPaged) return reinterpret_cast<uint4 *>(half.dst) + (int64_t)r * (p.head_dim >> 3);
-    if (po.fast)
-        return reinterpret_cast<uint4 *>(half.dst + (r < po.split ? po.da : po.db) + (int64_t)r * po.stride);
-    PagedRows slow{};
-    slow.fast = false;
-    return row_dst<true>(p, half, r, slow);
-}
-
-// Stores vector v (0 <= v < rows * d / 8) of a copied item.
-template <bool kPaged>
-__device__ __forceinline__ void store_vec(const RenderParams &p, const Item &it,
-                                          const PagedOffsets &po, int v, const uint4 &x) {
-    const int log2_vpr = p.log2_pairs_per_row + 1;   // vectors per row = d / 8
-    uint4 *d = pair_row<kPaged>(p, it, po, v >> log2_vpr) + (v & ((1 << log2_vpr) - 1));
-    if (CM_IN_BOUNDS(d, 16, it.dst_base, it.dst_size)) st_stream(d, x);
-}
-
-// Full-SM render: persistent, kRegBlocksPerSm CTAs of 8 warps per SM, no shared-memory
-// staging and no waits. Per pair, each lane loads its 2 vectors of the K item (for a
-// rotated item: vector v of the first and of the second half of one row, v = lane mod
-// (d/16)) and its 2 vectors of the V item, then stores V, then rotates (slots at a
-// nonzero offset) and stores K. The lane's 8 (cos, sin) values are reloaded only when
-// the slot changes.
-template <bool kPaged>
+// The widths of small and middling merges beside the content address (contiguous outputs):
+// persistent, one or two CTAs of 8 warps per SM, no shared-memory staging and no waits. Per
+// pair, each lane loads its 2 vectors of the K item (for a rotated item: vector v of the first
+// and of the second half of one row, v = lane mod (d/16)) and its 2 vectors of the V item, then
+// stores V, then rotates (slots at a nonzero offset) and stores K. The lane's 8 (cos, sin)
+// values are reloaded only when the slot changes.
 __global__ void __launch_bounds__(kRegThreads, kRegBlocksPerSm)
 render_reg_kernel(const __grid_constant__ RenderParams p) {
     __shared__ float4 tab[kMaxTablePairs];   // (c1, c2, s1, s2) for the second level
@@ -817,7 +880,7 @@ render_reg_kernel(const __grid_constant__ RenderParams p) {
     w.stride = gridDim.x * (kRegThreads / 32);
     w.npairs = p.total_chunks / 2;
     if (w.pr >= w.npairs) return;
-    w.enter<kPaged>(p);
+    w.enter<false>(p);
     const int half_vecs = p.head_dim >> 4;
     const int vecs_per_row = p.head_dim >> 3;
     const int log2_hv = p.log2_pairs_per_row;
@@ -825,7 +888,7 @@ render_reg_kernel(const __grid_constant__ RenderParams p) {
     int cur = -1;
     float c[8], s[8];
     do {
-        const Pair q = pair_of<kPaged>(p, w);
+        const Pair q = pair_of<false>(p, w);
         const int n_vec = q.rows * vecs_per_row;
         const int n_pairs = q.rows * half_vecs;
         const uint4 *ks = reinterpret_cast<const uint4 *>(q.ks);
@@ -857,13 +920,10 @@ render_reg_kernel(const __grid_constant__ RenderParams p) {
             rv[u] = make_uint4(0, 0, 0, 0);
             if (v < n_vec && CM_IN_BOUNDS(vs + v, 16, q.vs_base, q.src_size)) rv[u] = __ldcs(vs + v);
         }
-        PagedOffsets po{};
-        if (kPaged) po = paged_offsets(p, q.pos0, q.rows);
-        const Item vi = half_item(q, true);
-#pragma unroll
-        for (int u = 0; u < kRegVecs; ++u)
-            if (lane + 32 * u < n_vec) store_vec<kPaged>(p, vi, po, lane + 32 * u, rv[u]);
-        const Item ki = half_item(q, false);
+        const uint32_t bytes = (uint32_t)n_vec * 16;
+        Item vi = half_item(q, true), ki = half_item(q, false);
+        vi.bytes = ki.bytes = bytes;
+        copy_from_regs<false>(p, vi, 0, rv, lane);
         if (q.rotate) {
             if (q.cs_index != cur) {
                 cur = q.cs_index;
@@ -880,30 +940,15 @@ render_reg_kernel(const __grid_constant__ RenderParams p) {
                 if (qq < n_pairs) {
                     // copies of the two vectors, which the fix-up also reads
                     const uint4 a = rk[2 * k], b = rk[2 * k + 1];
-                    const float4 ka = *reinterpret_cast<const float4 *>(kt + cur + 8 * lane_v);
-                    const float4 kb = *reinterpret_cast<const float4 *>(kt + cur + 8 * lane_v + 4);
-                    const float4 na = *reinterpret_cast<const float4 *>(nst + cur + 8 * lane_v);
-                    const float4 nb = *reinterpret_cast<const float4 *>(nst + cur + 8 * lane_v + 4);
                     uint4 ao, bo;
-                    uint32_t b0, b1, b2, b3;
-                    rotate_word(a.x, b.x, c[0], s[0], na.x, ka.x, c[1], s[1], na.y, ka.y, ao.x, bo.x, b0);
-                    rotate_word(a.y, b.y, c[2], s[2], na.z, ka.z, c[3], s[3], na.w, ka.w, ao.y, bo.y, b1);
-                    rotate_word(a.z, b.z, c[4], s[4], nb.x, kb.x, c[5], s[5], nb.y, kb.y, ao.z, bo.z, b2);
-                    rotate_word(a.w, b.w, c[6], s[6], nb.z, kb.z, c[7], s[7], nb.w, kb.w, ao.w, bo.w, b3);
-                    if ((b0 | b1 | b2 | b3) != 0u)
-                        fixup_pair(p, tab, cur + 8 * lane_v, a, b, b0, b1, b2, b3, ao, bo);
-                    uint4 *d = pair_row<kPaged>(p, ki, po, qq >> log2_hv) + lane_v;
-                    if (CM_IN_BOUNDS(d, 16, ki.dst_base, ki.dst_size)) st_stream(d, ao);
-                    if (CM_IN_BOUNDS(d + half_vecs, 16, ki.dst_base, ki.dst_size))
-                        st_stream(d + half_vecs, bo);
+                    rotate_vectors(p, tab, kt, nst, cur + 8 * lane_v, c, s, a, b, ao, bo);
+                    store_pair<false>(p, ki, PagedRows{}, qq >> log2_hv, lane_v, ao, bo);
                 }
             }
         } else {
-#pragma unroll
-            for (int u = 0; u < kRegVecs; ++u)
-                if (lane + 32 * u < n_vec) store_vec<kPaged>(p, ki, po, lane + 32 * u, rk[u]);
+            copy_from_regs<false>(p, ki, 0, rk, lane);
         }
-    } while (w.next<kPaged>(p));
+    } while (w.next<false>(p));
 }
 
 }  // namespace
@@ -911,48 +956,37 @@ render_reg_kernel(const __grid_constant__ RenderParams p) {
 CM_DEFINE_BOUNDS_READER(take_render_bounds_violations)
 
 cudaError_t render_prepare() {
-    cudaError_t e = set_smem_attribute<false, 8>();
-    if (e == cudaSuccess) e = set_smem_attribute<true, 8>();
-    if (e == cudaSuccess) e = set_smem_attribute<false, 4, 6, 4>();
-    if (e == cudaSuccess) e = set_smem_attribute<true, 4, 6, 4>();
-    return e;
+    for (RenderWidth w : {RenderWidth::kFull, RenderWidth::kHalf, RenderWidth::kBeside})
+        for (bool paged : {false, true}) {
+            const cudaError_t e = cudaFuncSetAttribute(tma_kernel(w, paged), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       (int)dyn_smem(tma_width(w, paged), kMaxTablePairs));
+            if (e != cudaSuccess) return e;
+        }
+    return cudaSuccess;
 }
 
-uint32_t render_item_bytes(RenderWidth w) {
-    return (w == RenderWidth::kHalf || w == RenderWidth::kBeside) ? kItemBytes : kRegItemBytes;
-}
+uint32_t render_item_bytes(RenderWidth w) { return is_tma(w) ? tma_width(w, false).item_bytes : kRegItemBytes; }
 
 int render_grid(uint64_t chunks, int num_sms, RenderWidth w) {
-    if (w == RenderWidth::kHalf || w == RenderWidth::kBeside)
-        return (int)std::max<uint64_t>(1, std::min<uint64_t>(chunks, (uint64_t)num_sms));
+    const uint64_t sms = (uint64_t)num_sms;
+    if (is_tma(w)) return (int)std::max<uint64_t>(1, std::min<uint64_t>(chunks / 2, sms));   // one CTA per SM
     const uint64_t ctas = (chunks / 2 + kRegThreads / 32 - 1) / (kRegThreads / 32);
-    const uint64_t per_sm = w == RenderWidth::kFull           ? (uint64_t)kRegBlocksPerSm
-                            : w == RenderWidth::kAfterLeaves ? 2
-                                                             : 1;
-    return (int)std::max<uint64_t>(1, std::min<uint64_t>(ctas, per_sm * num_sms));
+    return (int)std::max<uint64_t>(1, std::min<uint64_t>(ctas, (w == RenderWidth::kAfterLeaves ? 2 : 1) * sms));
 }
 
 cudaError_t launch_render(const RenderParams &p, int grid, RenderWidth w, cudaStream_t stream) {
     if (p.total_chunks == 0) return cudaSuccess;
-    switch (w) {
-        case RenderWidth::kHalf:
-            if (p.paged)
-                render_kernel<true, 8><<<grid, 8 * 32, dyn_smem<8>(), stream>>>(p);
-            else
-                render_kernel<false, 8><<<grid, 8 * 32, dyn_smem<8>(), stream>>>(p);
-            break;
-        case RenderWidth::kBeside:
-            if (p.paged)
-                render_kernel<true, 4, 6, 4><<<grid, 4 * 32, dyn_smem<4, 6>(), stream>>>(p);
-            else
-                render_kernel<false, 4, 6, 4><<<grid, 4 * 32, dyn_smem<4, 6>(), stream>>>(p);
-            break;
-        default:   // kFull, kBesideSmall, kAfterLeaves: the register kernel (grid sizes differ)
-            if (p.paged)
-                render_reg_kernel<true><<<grid, kRegThreads, 0, stream>>>(p);
-            else
-                render_reg_kernel<false><<<grid, kRegThreads, 0, stream>>>(p);
-            break;
+    if (is_tma(w)) {
+        const TmaWidth t = tma_width(w, p.paged != 0);
+        // The widths that share their SMs with leaf-hash blocks (1 KiB of shared memory each, which
+        // the system reserves) ask for the whole table whatever they need: of the sizes that an SM
+        // can be set to, the next one up then leaves room for all of the blocks. With 163 KB, 3 KB
+        // short of a size, the merge of 4 x 4096 tokens took 1.76 instead of 1.60 ms.
+        const int entries = w == RenderWidth::kFull ? p.num_slots * (p.head_dim / 2) : kMaxTablePairs;
+        const size_t smem = dyn_smem(t, entries);
+        tma_kernel(w, p.paged != 0)<<<grid, t.warps * 32, smem, stream>>>(p);
+    } else {
+        render_reg_kernel<<<grid, kRegThreads, 0, stream>>>(p);
     }
     return cudaGetLastError();
 }

@@ -110,3 +110,29 @@ def test_leaves_that_straddle_segments(ctx, shape):
     assert [fid for fid, _ in res] == [oracle_fragment(*whole).fid, oracle_fragment(K, V).fid]
     S.close()
     both.close()
+
+
+# item sizes of the renders' widths (2 KiB, 4 KiB and 16 KiB of rows) at, below and above a
+# plane's rows, fewer pairs than warps, and every head_dim, against the oracle
+@pytest.mark.parametrize("L,H,d,lengths", [(1, 1, 128, (8, 7)), (1, 2, 128, (9, 64, 65)), (2, 1, 16, (63, 64, 65)),
+                                           (1, 1, 512, (1, 2, 3)), (3, 2, 64, (16, 17, 31)), (2, 2, 32, (32, 33, 257)),
+                                           (2, 3, 256, (4, 5, 40))])
+@pytest.mark.parametrize("warps", [16, 8])
+def test_render_items_at_their_edges(ctx, L, H, d, lengths, warps):
+    import oracle
+    import synthetic
+    from parity_util import assert_k_parity
+    frags = [_fragment(17 * T + i, L, H, T, d) for i, T in enumerate(lengths)]
+    S = cm.FragmentSet(ctx)
+    S.ingest_batch(frags)
+    k, v = empty_out(L, H, sum(lengths) + 3, d, fill=0x3C3C)
+    cm.cm_context_set_render_warps(ctx.handle, warps)
+    n, order = S.render(k, v)
+    torch.cuda.synchronize()
+    cm.cm_context_set_render_warps(ctx.handle, 16)
+    K_ref, V_ref, o_order = oracle.render(oracle.from_deliveries([oracle_fragment(K, V) for K, V in frags]), THETA)
+    assert n == sum(lengths) and order == [f.fid for f in o_order]
+    assert np.array_equal(synthetic.to_bits(v[:, :, :n]), V_ref)
+    assert assert_k_parity(synthetic.to_bits(k[:, :, :n]), K_ref) == 0
+    assert (k.view(torch.int16)[:, :, n:] == 0x3C3C).all() and (v.view(torch.int16)[:, :, n:] == 0x3C3C).all()
+    S.close()
