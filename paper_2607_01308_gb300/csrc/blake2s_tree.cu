@@ -45,9 +45,9 @@ __device__ __forceinline__ uint32_t rotr7(uint32_t x) { return __funnelshift_r(x
 // product with (0, 1) adds its lower half: two multiply-type instructions for one byte
 // permutation. Moving it in t of the 8 G's of a round leaves (8 - t/8) x 2 ALU cycles,
 // (6 + t/4) x 2 FMA cycles and 14 + t/8 issue cycles per G, balanced at t = 5. Measured over
-// 45 choices of the G's (2.4 GB of leaves, 1.356 ms with the earlier order of additions and
-// no rotation moved): 1.364 ms with t = 0, 1.305 with 3, 1.273 to 1.300 with 5 or 6, 1.330
-// with 8; the choice below is the fastest. ALU 92 %, FMA 89 % and issue 91 % busy.
+// 52 choices of the G's on 2.4 GB of leaves: 1.06 times the best with t = 0, 1.02 with 3, 1.00 to
+// 1.02 with 5 or 6, 1.04 with 8; the choice below 1.259 ms (1.310 with the earlier order of
+// additions and no rotation moved). ALU 92 %, FMA 89 % and issue 91 % busy.
 __constant__ uint32_t g_one = 1, g_64k = 65536, g_upper_half = 0x0100;
 __device__ __forceinline__ uint32_t mad1(uint32_t x, uint32_t y) {
     uint32_t r;
@@ -67,7 +67,7 @@ __device__ __forceinline__ uint32_t rotr16_fma(uint32_t x) {
 // Beside a render (kBesideRender), whose own instructions take issue slots and the FMA pipe,
 // three: the Qwen3-4B-shaped merge of 4 x 4096 tokens took 1.71 ms with 3, 1.71 with 2, 1.72
 // with none or one and 1.77 with 5; the arity merge 0.77, 0.79, 0.80 and 0.78.
-constexpr uint32_t kIssueBound = 0xD6u, kBesideRender = 0x52u;
+constexpr uint32_t kIssueBound = 0xE6u, kBesideRender = 0x52u;
 template <uint32_t kMask, int kG>
 __device__ __forceinline__ uint32_t rotate16(uint32_t x) {
     return (kMask >> kG) & 1u ? rotr16_fma(x) : rotr16(x);
