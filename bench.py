@@ -41,12 +41,15 @@ ROPE_THETA = 1.0e6
 BASE_SEED_REDELIVER = 42 + 997   # delivery order of the re-delivery sweep
 NOMINAL_HBM_GBS = 8000.0
 FALLBACK_HBM_GBS = 6800.0
-# Integer-ALU roofline of the content-address kernel: a BLAKE2s block (64 bytes) is
-# 10 rounds x 8 G x (4 xors + 4 rotates) + 8 xors = 648 ops that must issue on the
-# integer ALU pipe (G's additions are multiply-adds on the FMA pipe); the pipe takes 16
-# lanes per SMSP per clock (4 SMSPs -> 64 ops/clk/SM), so the peak is 152 SMs x 64 x
-# the maximum SM clock.
-HASH_ALU_OPS_PER_BYTE = 648.0 / 64.0
+# Integer-ALU roofline of the content-address kernel: a BLAKE2s block (64 bytes) has
+# 10 rounds x 8 G x (4 xors + 4 rotates) + 8 xors = 648 xors and rotations. Five of a round's
+# rotations by 16 (three when a render runs beside the hash) are dot products on the FMA
+# pipe, as G's additions are multiply-adds there, so 598 (618) issue on the integer ALU pipe;
+# the pipe takes 16 lanes per SMSP per clock (4 SMSPs -> 64 ops/clk/SM), so the peak is
+# 152 SMs x 64 x the maximum SM clock.
+HASH_XOR_ROT_PER_BYTE = 648.0 / 64.0
+HASH_ALU_OPS_PER_BYTE = 598.0 / 64.0
+HASH_ALU_OPS_PER_BYTE_BESIDE = 618.0 / 64.0
 ALU_OPS_PER_CLK_PER_SM = 64
 CLOCK_FIELDS = ("index,clocks.sm,clocks.max.sm,power.draw,clocks_event_reasons.active,"
                 "clocks_event_reasons.hw_slowdown,clocks_event_reasons.hw_thermal_slowdown,"
@@ -677,9 +680,7 @@ def run_serve(args):
 # ---------------------------------------------------------------- GPU arm
 
 # BLAKE2s work per 64-byte block of the content address: 10 rounds x 8 G, each G 6 additions,
-# 4 xors and 4 rotations, then 16 xors of the finalisation: 1136 two-input integer operations,
-# of which the 648 xors and rotations (three-input xors counted once) must issue on the
-# integer ALU pipe.
+# 4 xors and 4 rotations, then 16 xors of the finalisation: 1136 two-input integer operations.
 HASH_INT_OPS_PER_BLOCK = 10 * 8 * (6 + 4 + 4) + 16
 
 
@@ -1146,12 +1147,12 @@ def main():
         render_ms_ovl = ktimes["render_ms"] / max(1, ktimes["render_launches"])
         copy_gbs = copy["median_gbs"]
         render_roof = {
-            "kernel": "render_reg_kernel", "bound": "hbm",
+            "kernel": "render_kernel (20-warp TMA CTAs)", "bound": "hbm",
             "achieved": render_bytes / (kernel_render_ms * 1e-3) / 1e9, "peak": peak,
             "peak_source": f"{peak_src} (MEASURED_PEAKS.json hbm_gbs)" if peak_src == "measured"
             else "fallback 6.8 TB/s", "unit": "GB/s",
             "frac": render_bytes / (kernel_render_ms * 1e-3) / 1e9 / peak,
-            "traffic": profile_traffic("render.cu", "render_reg_kernel_q4b.md"),
+            "traffic": profile_traffic("render.cu", "render_kernel_q4b.md"),
             "algorithmic_bytes_per_launch": render_bytes, "ms_per_launch": kernel_render_ms,
             "timing": "CUDA events on the render's stream around each launch in the sequential "
                       "steps (the full-SM render alone; the stream is idle when the start event is "
@@ -1184,7 +1185,9 @@ def main():
             # measured on this GPU before the timed steps (cm_measure_int_alu): three-input
             # xors alone, and the same compression function on register data alone
             "measured_xor3_tops": xor3_tops, "measured_compress_tops": compress_tops,
-            "frac_of_measured_compress": hash_tops / compress_tops,
+            # (both counted as the 648 xors and rotations of a block)
+            "frac_of_measured_compress":
+                HASH_XOR_ROT_PER_BYTE * frag_bytes / (leaf_ms * 1e-3) / 1e12 / compress_tops,
         }
         per_step = {"leaf_hash": ktimes["leaf_hash_ms"] / args.steps,
                     "inner_hash": ktimes["inner_hash_ms"] / args.steps,
@@ -1194,17 +1197,18 @@ def main():
                         "render": ktimes_seq["render_ms"] / args.steps}
         dominant = max(per_step, key=per_step.get)
         # the dominant kernel of the timed steps as it ran there: the leaf hash, with the
-        # half-SM render of the same merge beside it on the other stream
+        # 4-warp render of the same merge beside it on the other stream
         hash_in_step = dict(hash_roof)
         hash_in_step.update({
-            "achieved": HASH_ALU_OPS_PER_BYTE * frag_bytes / (leaf_ms_ovl * 1e-3) / 1e12,
-            "frac": HASH_ALU_OPS_PER_BYTE * frag_bytes / (leaf_ms_ovl * 1e-3) / 1e12 / alu_peak,
+            "algorithmic_ops_per_launch": HASH_ALU_OPS_PER_BYTE_BESIDE * frag_bytes,
+            "achieved": HASH_ALU_OPS_PER_BYTE_BESIDE * frag_bytes / (leaf_ms_ovl * 1e-3) / 1e12,
+            "frac": HASH_ALU_OPS_PER_BYTE_BESIDE * frag_bytes / (leaf_ms_ovl * 1e-3) / 1e12 / alu_peak,
             "ms_per_launch": leaf_ms_ovl,
             "hash_gbs": frag_bytes / (leaf_ms_ovl * 1e-3) / 1e9,
             "frac_all_int_ops_of_128_lanes":
                 HASH_INT_OPS_PER_BLOCK * blocks / (leaf_ms_ovl * 1e-3) / 1e12 / int_peak,
             "frac_of_measured_compress":
-                HASH_ALU_OPS_PER_BYTE * frag_bytes / (leaf_ms_ovl * 1e-3) / 1e12 / compress_tops,
+                HASH_XOR_ROT_PER_BYTE * frag_bytes / (leaf_ms_ovl * 1e-3) / 1e12 / compress_tops,
             "timing": "CUDA events around each leaf-hash launch in the timed steps, where the "
                       "render of the same merge runs beside it on another stream (cm_ingest_render); "
                       "hash_roofline has the same kernel alone",
