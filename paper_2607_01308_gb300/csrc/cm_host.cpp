@@ -21,6 +21,7 @@
 #include <memory>
 #include <mutex>
 #include <new>
+#include <set>
 #include <string>
 #include <unordered_map>
 #include <utility>
@@ -1465,16 +1466,19 @@ std::vector<Slot> canonical_slots(const cm_set *set, void *k_out, void *v_out, i
     return slots;
 }
 
-// When cm_ingest_render's render starts, and how wide. From this many bytes of fragments on it
-// runs beside the leaf hash as the 4-warp TMA kernel; a smaller one whose leaf hash fills the
-// GPU starts as the leaves end, beside the tree levels (whose few warps leave it the memory),
-// as the register kernel with two CTAs per SM, and one whose leaf hash leaves room on every SM
-// starts at once beside it, as the register kernel with one. Measured (us, on the Qwen3 shapes;
-// beside with one CTA, beside as the TMA kernel, after the leaves): 2 x 512 tokens 146, -, 152;
-// 2 x 700 192, -, 182; 4 x 512 306, 364, 281; 4 x 850 (505 MB) 475, 494, 457; 3 x 1500
-// (663 MB) -, 533, 590; 3 x 2000 -, 666, 777. One or three CTAs after the leaves: 4 x 512
-// 330, 292.
-constexpr uint64_t kBesideLargeBytes = 512ull << 20;
+// When cm_ingest_render's render starts, and how wide. A render of this many bytes of fragments
+// or more starts at once and runs beside the leaf hash as the 4-warp TMA kernel. A smaller one
+// whose leaf hash fills the GPU starts as the leaves end, beside the tree levels (whose few warps
+// leave it the memory), as the register kernel with two CTAs per SM. Measured (us, beside against
+// after the leaves): 253 MB 271, 252; 288 MB 280, 287; 346 MB (head_dim 256) 325, 337; 478 MB 405,
+// 462; 632 MB 501, 587. One or three CTAs after the leaves: 288 MB 330, 292 against 281.
+constexpr uint64_t kBesideLargeBytes = 272ull << 20;
+// The same where the leaf hash leaves room on every SM (few deliveries, perhaps into a set that
+// holds more): smaller renders start at once too, as the register kernel with one CTA per SM.
+// Measured (us, TMA kernel against register kernel): all delivered 65 MB 125, 102; 84 MB 134, 118;
+// 112 MB 130, 128; 129 MB 143, 165; 500 delivered tokens on 100, 300 and 500 held (84, 112, 140 MB)
+// 115, 118, 122 against 102, 116, 128; 60 tokens on 900 (135 MB) 82, 99; on 3000 (430 MB) 183, 248.
+constexpr uint64_t kBesideRoomBytes = 120ull << 20;
 
 // cm_ingest_render (see include/cm.h). The norm keys of the deliveries are computed on
 // the context's side stream while the content address runs on `stream`. Equal bytes give
@@ -1588,18 +1592,29 @@ cm_status ingest_render_impl(cm_set *const *sets, const cm_fragment *frags, int3
     const bool partial_wave =
         ctx->leaf_blocks_per_sm > 1 &&
         leaf_blocks <= (uint64_t)(ctx->leaf_blocks_per_sm - 1) * (uint64_t)ctx->num_sms;
-    int64_t most_tokens = 0;   // of the prospective set, repeats included
-    for (const auto &kv : target->items) most_tokens += kv.second->T;
+    // The prospective set's tokens, re-sent copies not yet told apart: at most all of them, at
+    // least one fragment of each length.
+    int64_t most_tokens = 0, least_tokens = 0;
+    std::set<int64_t> seen_lengths;
+    auto count_tokens = [&](int64_t T) {
+        most_tokens += T;
+        if (seen_lengths.insert(T).second) least_tokens += T;
+    };
+    for (const auto &kv : target->items) count_tokens(kv.second->T);
     for (const cm_set *src : sources)
-        for (const auto &kv : src->items) most_tokens += kv.second->T;
-    for (const cm_fragment *f : fp) most_tokens += f->seq_len;
+        for (const auto &kv : src->items) count_tokens(kv.second->T);
+    for (const cm_fragment *f : fp) count_tokens(f->seq_len);
     const uint64_t token_bytes = 4ull * (uint64_t)L * (uint64_t)H * (uint64_t)d;
-    const bool after_leaves = !partial_wave && (uint64_t)most_tokens * token_bytes < kBesideLargeBytes;
-    const bool digest_first = partial_wave || after_leaves;
+    auto large = [&](int64_t tokens) {
+        return (uint64_t)tokens * token_bytes >= (partial_wave ? kBesideRoomBytes : kBesideLargeBytes);
+    };
+    const bool may_wait = !partial_wave && !large(least_tokens);   // for the leaves to end
+    const bool digest_first = partial_wave || !large(most_tokens);
     auto digest = [&]() -> cm_status {
         return enqueue_digest(ctx, plan, fp.data(), fp.size(), cs,
-                              after_leaves ? cm::LeafMode::kAlone : cm::LeafMode::kBesideRender,
-                              after_leaves ? ctx->leaves_end : nullptr);
+                              partial_wave || large(most_tokens) ? cm::LeafMode::kBesideRender
+                                                                 : cm::LeafMode::kAlone,
+                              may_wait ? ctx->leaves_end : nullptr);
     };
     if (digest_first) {
         st = digest();
@@ -1677,11 +1692,10 @@ cm_status ingest_render_impl(cm_set *const *sets, const cm_fragment *frags, int3
                 spec_slots.push_back({x.k, x.v, x.T, s, k_out, v_out, capacity});
                 s += x.T;
             }
-            const cm::RenderWidth width = after_leaves ? cm::RenderWidth::kAfterLeaves
-                                          : (uint64_t)total * token_bytes >= kBesideLargeBytes
-                                              ? cm::RenderWidth::kBeside
-                                              : cm::RenderWidth::kBesideSmall;
-            if (after_leaves) {
+            const cm::RenderWidth width = large(total)   ? cm::RenderWidth::kBeside
+                                          : partial_wave ? cm::RenderWidth::kBesideSmall
+                                                         : cm::RenderWidth::kAfterLeaves;
+            if (width == cm::RenderWidth::kAfterLeaves) {
                 e = cudaStreamWaitEvent(ctx->side, ctx->leaves_end, 0);
                 if (e != cudaSuccess) return join(cuda_fail(e, "side stream ordering"));
             }

@@ -1,7 +1,8 @@
 """The edges of the content address's launches: heads per norm-key thread, tree levels at the
 edge of a block (which hands its digests to their parent) with several fragments in one
-launch, leaves on both sides of the switch from four lanes each to one, and the sizes at which cm_ingest_render starts its render beside the leaf hash, as
-the leaves end, or beside it again. Ids and norm keys equal the oracle's; the merges' bytes
+launch, leaves on both sides of the switch from four lanes each to one, and the sizes at which
+cm_ingest_render starts its render beside the leaf hash, as the leaves end, or beside it again.
+Ids and norm keys equal the oracle's; the merges' bytes
 equal those of the separate calls."""
 import numpy as np
 import pytest
@@ -58,12 +59,15 @@ def test_tree_levels_at_block_edges(ctx, lengths):
     S.close()
 
 
-# 114,688 bytes a token: 1,216 leaf blocks (one partial wave) up to about 1,389 tokens;
-# 512 MiB at 4,681 tokens
-@pytest.mark.parametrize("lengths,prior", [((690, 690), 0), ((700, 705), 0), ((1500, 1500, 1600), 0),
-                                           ((1500, 1500, 1700), 0), ((800, 810), 400), ((800, 810), 3100)])
-def test_ingest_render_start_rules_give_the_separate_calls_bytes(ctx, lengths, prior):
+# 114,688 bytes a token: 120 MiB at 1,098 tokens, 1,216 leaf blocks (one partial wave) up to
+# about 1,389, 272 MiB at 2,487; the re-sent copies reach that, what is rendered does not
+@pytest.mark.parametrize("lengths,prior,copies", [
+    ((540, 550), 0, ()), ((548, 550), 0, ()), ((690, 690), 0, ()), ((700, 705), 0, ()),
+    ((1240, 1246), 0, ()), ((1240, 1247), 0, ()), ((1500, 1500, 1700), 0, ()), ((300, 300), 400, ()),
+    ((300, 300), 1900, ()), ((800, 810), 400, ()), ((800, 810), 3100, ()), ((600, 700), 0, (1, 0))])
+def test_ingest_render_start_rules_give_the_separate_calls_bytes(ctx, lengths, prior, copies):
     frags = [_fragment(31 * T + i, 28, 8, T, 128) for i, T in enumerate(lengths)]
+    frags += [tuple(x.clone() for x in frags[i]) for i in copies]
     old = [_fragment(5, 28, 8, prior, 128)] if prior else []
     total = sum(lengths) + prior
     half = (len(frags) + 1) // 2
