@@ -65,9 +65,11 @@ __device__ __forceinline__ uint32_t rotr16_fma(uint32_t x) {
 // Which G's rotate by 16 on the FMA pipe (bit g of kMask: the round's G number g): five of
 // the eight in the leaf kernel and for level 1 of many nodes.
 // Beside a render (kBesideRender), whose own instructions take issue slots and the FMA pipe,
-// three: the Qwen3-4B-shaped merge of 4 x 4096 tokens took 1.71 ms with 3, 1.71 with 2, 1.72
-// with none or one and 1.77 with 5; the arity merge 0.77, 0.79, 0.80 and 0.78.
-constexpr uint32_t kIssueBound = 0xE6u, kBesideRender = 0x52u;
+// three: the Qwen3-4B-shaped merge of 4 x 4096 tokens took 1.598 ms with these three, 1.601 to
+// 1.616 with other threes, 1.598 with the best two, 1.605 with one, 1.631 with none, 1.602 with
+// four and 1.633 with five; the merge of five ragged fragments 0.722, 0.725 to 0.732, 0.723,
+// 0.727, 0.743, 0.722 and 0.732.
+constexpr uint32_t kIssueBound = 0xE6u, kBesideRender = 0x94u;
 template <uint32_t kMask, int kG>
 __device__ __forceinline__ uint32_t rotate16(uint32_t x) {
     return (kMask >> kG) & 1u ? rotr16_fma(x) : rotr16(x);
