@@ -26,8 +26,8 @@ cm_status cm_testing_render_withheld_load(const cm_set *set, void *k_out, void *
                                           int64_t capacity_tokens, cm_stream_t stream);
 
 /* Bounds-checked builds of the library (compiled with -DCM_DEBUG_BOUNDS; build.py --bounds
- * writes libcm_bounds.so) test every global access of the render and content-address
- * kernels against the buffer it belongs to (a fragment, an output, a level of the hash
+ * writes libcm_bounds.so) test every global access of the render, content-address
+ * and byte-comparison kernels against the buffer it belongs to (a fragment, an output, a level of the hash
  * tree, the norm key, a paged block table and the lower end of a paged pool, whose size
  * the library is not told); an access outside it is counted and not made, so a wrong index
  * cannot fault. This call synchronises `device` and returns the number of such accesses on

@@ -25,10 +25,11 @@ struct ComparePrefix {
     uint32_t *differ;                             // one word per pair; may be mapped host memory
 };
 
-// Deliveries (members) that may equal one candidate (the group's base): each group's K and V
-// arrays are `vecs` 16-byte vectors long.
+// Deliveries (members) that may equal one candidate (the group's base). K and V arrays are
+// `vecs` 16-byte vectors long, a member's as long as its base's.
 struct CompareMember {
     const uint4 *k, *v;
+    uint64_t vecs;
 };
 struct CompareGroup {
     const uint4 *k, *v;                           // the base
@@ -52,5 +53,9 @@ cudaError_t launch_compare_prefix(const ComparePrefix &c, cudaStream_t stream);
 // persistent grid of blocks_per_sm blocks per SM over all chunks of all groups; a member
 // already found to differ is skipped).
 cudaError_t launch_compare_full(const CompareFull &c, int num_sms, int blocks_per_sm, cudaStream_t stream);
+
+// Bounds-checked builds: reads and zeroes these kernels' violation count on the current device
+// (0 in other builds).
+cudaError_t take_dedup_bounds_violations(unsigned int *out);
 
 }  // namespace cm

@@ -16,7 +16,6 @@
 #include <cstdio>
 #include <cstddef>
 #include <cstring>
-#include <functional>
 #include <map>
 #include <memory>
 #include <mutex>
@@ -30,6 +29,7 @@
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
+#include "cm_dedup_groups.h"
 #include "cm_kernels.h"
 
 namespace {
@@ -265,11 +265,6 @@ cm::TreeParams tree_params(int32_t L, int32_t H, int32_t d, int32_t T) {
 }
 
 uint64_t ceil_div(uint64_t a, uint64_t b) { return (a + b - 1) / b; }
-
-// 16-byte vectors of a fragment's K (= of its V).
-uint64_t plane_vecs(const cm_fragment *f) {
-    return (uint64_t)f->num_layers * f->num_kv_heads * f->seq_len * f->head_dim * 2 / 16;
-}
 
 enum { kTimeLeaf = 0, kTimeInner = 1, kTimeRender = 2 };
 
@@ -788,7 +783,7 @@ cm_status match_prefixes(cm_context *ctx, cm_set *const *sets,
             const Candidate &c = cands[c0 + q];
             const cm_fragment *f = fp[c.delivery];
             cl->pair[q] = {static_cast<const uint4 *>(f->k),
-                           static_cast<const uint4 *>(c.r ? c.r->k : fp[c.other]->k), plane_vecs(f)};
+                           static_cast<const uint4 *>(c.r ? c.r->k : fp[c.other]->k), cm::fragment_vecs(*f)};
         }
         cl->count = (uint32_t)cn;
         cl->differ = differ + c0;
@@ -812,37 +807,28 @@ cm_status match_prefixes(cm_context *ctx, cm_set *const *sets,
 
 // Enqueues the full comparisons of `chosen` on `stream`, one launch per kMaxComparePairs of
 // them, and sorts it by the fragment that each is compared with, so that the copies of one
-// fragment are compared together; their flags (one word each, in device scratch at dev_off) go to the pinned buffer at host_off. Both offsets are
-// multiples of 16 and the scratch already reaches there.
+// fragment are compared together; their flags (one word each, in device scratch at dev_off) go
+// to the pinned buffer at host_off. Both offsets are multiples of 16 and the scratch already
+// reaches there.
 cm_status enqueue_comparisons(cm_context *ctx, const std::vector<const cm_fragment *> &fp,
                               std::vector<Candidate> &chosen, cudaStream_t stream,
                               int blocks_per_sm, size_t dev_off, size_t host_off) {
     auto base = [&](const Candidate &c) {
-        return c.r ? std::make_pair(c.r->k, c.r->v) : std::make_pair(fp[c.other]->k, fp[c.other]->v);
+        return c.r ? cm_fragment{c.r->L, c.r->H, c.r->T, c.r->d, c.r->k, c.r->v} : *fp[c.other];
     };
     std::stable_sort(chosen.begin(), chosen.end(), [&](const Candidate &a, const Candidate &b) {
-        return std::less<std::pair<const void *, const void *>>()(base(a), base(b));
+        return cm::compare_fragments(base(a), base(b)) < 0;
     });
+    std::vector<cm::Comparison> comparisons;
+    comparisons.reserve(chosen.size());
+    for (const Candidate &c : chosen) comparisons.push_back({base(c), *fp[c.delivery]});
     auto *differ = reinterpret_cast<uint32_t *>(ctx->d_scratch + dev_off);
     CM_CUDA_TRY(cudaMemsetAsync(differ, 0, chosen.size() * 4, stream), "comparison flags reset");
     std::unique_ptr<cm::CompareFull> cl(new cm::CompareFull);
     for (size_t c0 = 0; c0 < chosen.size(); c0 += (size_t)cm::kMaxComparePairs) {
         const size_t cn = std::min(chosen.size() - c0, (size_t)cm::kMaxComparePairs);
-        std::memset(cl.get(), 0, sizeof(cm::CompareFull));
-        for (size_t m = 0; m < cn; ++m) {
-            const Candidate &c = chosen[c0 + m];
-            const cm_fragment *f = fp[c.delivery];
-            cl->member[m] = {static_cast<const uint4 *>(f->k), static_cast<const uint4 *>(f->v)};
-            // one fragment's copies share its shape, so also the group's
-            if (m == 0 || base(chosen[c0 + m - 1]) != base(c)) {
-                cl->group[cl->groups] = {static_cast<const uint4 *>(base(c).first),
-                                         static_cast<const uint4 *>(base(c).second), plane_vecs(f), (uint32_t)m, 0};
-                cl->chunk_begin[cl->groups + 1] = cl->chunk_begin[cl->groups] +
-                    2 * ceil_div(plane_vecs(f), (uint64_t)cm::kCompareChunkVecs);
-                ++cl->groups;
-            }
-            cl->group[cl->groups - 1].end = (uint32_t)m + 1;
-        }
+        if (!cm::group_comparisons(comparisons.data() + c0, cn, *cl))
+            return fail(CM_ERR_INVALID_ARG, "a comparison of fragments of different sizes");
         cl->differ = differ + c0;
         CM_CUDA_TRY(cm::launch_compare_full(*cl, ctx->num_sms, blocks_per_sm, stream), "comparison launch");
         if (ctx->timing) ++ctx->aux_launches;
@@ -1853,10 +1839,11 @@ cm_status cm_testing_bounds_violations(int32_t device, uint64_t *out_count, int3
         DeviceScope scope(device);
         if (!scope.ok()) return fail(CM_ERR_CUDA, "cannot select the CUDA device");
         CM_CUDA_TRY(cudaDeviceSynchronize(), "device synchronisation");
-        unsigned int render = 0, hash = 0;
+        unsigned int render = 0, hash = 0, dedup = 0;
         CM_CUDA_TRY(cm::take_render_bounds_violations(&render), "render violation count");
         CM_CUDA_TRY(cm::take_hash_bounds_violations(&hash), "content-address violation count");
-        *out_count = (uint64_t)render + hash;
+        CM_CUDA_TRY(cm::take_dedup_bounds_violations(&dedup), "comparison violation count");
+        *out_count = (uint64_t)render + hash + dedup;
 #ifdef CM_DEBUG_BOUNDS
         *out_enabled = 1;
 #else

@@ -5,6 +5,7 @@
 // a fragment whose address is known or being computed, it need not be hashed. The
 // comparison reads both fragments once at HBM speed; the hash is bound by the
 // integer ALU. Pairs that differ are usually told apart by their first 4 KiB.
+#include "cm_bounds.h"
 #include "cm_dedup_kernels.h"
 
 namespace cm {
@@ -21,12 +22,17 @@ __device__ __forceinline__ uint32_t diff4(const uint4 &x, const uint4 &y) {
     return (x.x ^ y.x) | (x.y ^ y.y) | (x.z ^ y.z) | (x.w ^ y.w);
 }
 
+// Vector i of an array of n.
+__device__ __forceinline__ uint4 load_vec(const uint4 *p, uint64_t i, [[maybe_unused]] uint64_t n) {
+    return CM_IN_BOUNDS(p + i, 16, p, n * 16) ? __ldcs(p + i) : make_uint4(0, 0, 0, 0);
+}
+
 // One block per pair: the first 4 KiB of K.
 __global__ void __launch_bounds__(kThreads) prefix_kernel(const __grid_constant__ ComparePrefix c) {
     const ComparePair &p = c.pair[blockIdx.x];
     const uint64_t n = p.vecs < kPrefixVecs ? p.vecs : kPrefixVecs;
     uint32_t d = 0;
-    for (uint64_t i = threadIdx.x; i < n; i += kThreads) d |= diff4(__ldg(p.a_k + i), __ldg(p.b_k + i));
+    for (uint64_t i = threadIdx.x; i < n; i += kThreads) d |= diff4(load_vec(p.a_k, i, p.vecs), load_vec(p.b_k, i, p.vecs));
     const int any = __syncthreads_or(d != 0);
     if (threadIdx.x == 0) c.differ[blockIdx.x] = any ? 1u : 0u;
 }
@@ -53,7 +59,7 @@ __global__ void __launch_bounds__(kThreads) full_kernel(const __grid_constant__ 
             uint4 b[kStepVecs];
 #pragma unroll
             for (int u = 0; u < kStepVecs; ++u)
-                b[u] = i + (uint64_t)u * kThreads < end ? __ldcs(base + i + (uint64_t)u * kThreads)
+                b[u] = i + (uint64_t)u * kThreads < end ? load_vec(base, i + (uint64_t)u * kThreads, g.vecs)
                                                         : make_uint4(0, 0, 0, 0);
             for (uint32_t m = g.begin; m < g.end; ++m) {
                 if (__ldcg(c.differ + m) != 0) continue;
@@ -61,7 +67,8 @@ __global__ void __launch_bounds__(kThreads) full_kernel(const __grid_constant__ 
                 uint32_t d = 0;
 #pragma unroll
                 for (int u = 0; u < kStepVecs; ++u)
-                    if (i + (uint64_t)u * kThreads < end) d |= diff4(__ldcs(a + i + (uint64_t)u * kThreads), b[u]);
+                    if (i + (uint64_t)u * kThreads < end)
+                        d |= diff4(load_vec(a, i + (uint64_t)u * kThreads, c.member[m].vecs), b[u]);
                 if (d != 0) atomicOr(c.differ + m, 1u);
             }
         }
@@ -69,6 +76,8 @@ __global__ void __launch_bounds__(kThreads) full_kernel(const __grid_constant__ 
 }
 
 }  // namespace
+
+CM_DEFINE_BOUNDS_READER(take_dedup_bounds_violations)
 
 cudaError_t launch_compare_prefix(const ComparePrefix &c, cudaStream_t stream) {
     if (c.count == 0) return cudaSuccess;
@@ -78,6 +87,9 @@ cudaError_t launch_compare_prefix(const ComparePrefix &c, cudaStream_t stream) {
 
 cudaError_t launch_compare_full(const CompareFull &c, int num_sms, int blocks_per_sm, cudaStream_t stream) {
     if (c.groups == 0) return cudaSuccess;
+    for (uint32_t g = 0; g < c.groups; ++g)   // a member of another size would be read past its end
+        for (uint32_t m = c.group[g].begin; m < c.group[g].end; ++m)
+            if (c.member[m].vecs != c.group[g].vecs) return cudaErrorInvalidValue;
     const uint64_t total = c.chunk_begin[c.groups];
     const uint64_t most = (uint64_t)num_sms * (uint64_t)blocks_per_sm;
     const uint64_t grid = total < most ? total : most;

@@ -1,8 +1,8 @@
 """Parity cases run against the bounds-checked build of the library (libcm_bounds.so,
 named by the environment variable CM_LIBRARY; started by test_gpu_bounds.py).
 
-Every global access of the render and content-address kernels is checked against the
-buffer it belongs to in that build. The cases below cover every kernel path (both render
+Every global access of the render, content-address and byte-comparison kernels is checked
+against the buffer it belongs to in that build. The cases below cover every kernel path (both render
 widths, contiguous, paged with power-of-two and other block sizes, both tree-top schemes,
 the allocation-free path, the re-delivery comparison, BagMerge, the incremental render and
 both renders that run beside the leaf hash in cm_ingest_render);
@@ -186,6 +186,17 @@ def main():
     assert [a for _, a in res] == [False, False, True, True]
     assert res[2][0] == res[0][0] == oracle_fragment(*A).fid
     S.close()
+    # fragments that start at one address (a tensor's first layers beside all of them), each
+    # copy compared over its own size
+    from test_gpu_dedup import part_schedules
+    whole = frags_of(22, 3, 1, 128, (4099,))[0]
+    for plan in part_schedules(whole, tuple(x[:2] for x in whole)):
+        P, Q = cm.FragmentSet(c2), cm.FragmentSet(c2)
+        res = cm.ingest_many([((P, Q)[s], *f) for s, f, _ in plan])
+        assert res == [(oracle_fragment(*f).fid, absorbed) for _, f, absorbed in plan]
+        P.close()
+        Q.close()
+        cases += 1
     c2.close()
     cases += 1
 

@@ -1,7 +1,7 @@
 """The bounds-checked testing build (build.py --bounds, libcm_bounds.so; a stand-in for a
 device memory checker): the parity cases of tests/bounds_cases.py run against it in a
-separate process, with every global access of the render and content-address kernels
-checked against the buffer it belongs to. No access may fall outside, the results must
+separate process, with every global access of the render, content-address and
+byte-comparison kernels checked against the buffer it belongs to. No access may fall outside, the results must
 be the oracle's, and a negative block-table entry (an input the host does not check) must
 be counted."""
 import json

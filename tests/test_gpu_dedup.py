@@ -140,6 +140,41 @@ def test_fast_path_with_verify_on_hit():
     ctx.close()
 
 
+def part_schedules(whole, part):
+    """[(set, fragment, absorbed)] deliveries of two fragments that start at one address (`part`:
+    fewer bytes of the same buffers), a copy of each and a copy of the whole that differs in its
+    last element alone, the copies in both orders. Each copy is a buffer of its own."""
+    copies = [(0, _flip(whole, "v", -1), False), (0, _clone(whole), True), (1, _clone(part), True)]
+    return [[(0, whole, False), (1, part, False)] + c for c in (copies, copies[::-1])]
+
+
+# the first two of three layers, and with one layer and head the first 200 of 300 tokens
+@pytest.mark.parametrize("shape,layers,tokens", [((3, 2, 50, 64), 2, 50), ((3, 1, 4099, 128), 2, 4099),
+                                                 ((1, 1, 300, 64), 1, 200)])
+@pytest.mark.parametrize("one_call", [True, False])
+def test_fragments_that_start_at_one_address(ctxs, shape, layers, tokens, one_call):
+    L, H, T, d = shape
+    whole, = _frags(930 + T, [T], L, H, d)
+    part = tuple(x[:layers, :, :tokens] for x in whole)
+    assert all(x.is_contiguous() for x in part)
+    for plan in part_schedules(whole, part):
+        split = len(plan) if one_call else 2      # the originals in the same call, or held already
+        got = []
+        for ctx in ctxs:
+            sets = [cm.FragmentSet(ctx), cm.FragmentSet(ctx)]
+            res = []
+            for deliveries in (plan[:split], plan[split:]):
+                if deliveries:
+                    res += cm.ingest_many([(sets[s], *f) for s, f, _ in deliveries])
+            got.append((res, [S.ids() for S in sets]))
+            for S in sets:
+                S.close()
+        assert got[0] == got[1]
+        res, ids = got[1]
+        assert res == [(oracle_fragment(*f).fid, absorbed) for _, f, absorbed in plan]
+        assert [len(i) for i in ids] == [2, 1]        # the near-copy is a fragment of its own
+
+
 @pytest.mark.parametrize("seed", range(10))
 def test_random_redeliveries_equal_the_path_off(ctxs, seed):
     # seeded random merges (the generator of test_gpu_random.py) with every delivery a
