@@ -554,13 +554,23 @@ struct Slot {
 cm_status launch_slots(cm_context *ctx, const std::vector<Slot> &slots, int32_t L, int32_t H,
                        int32_t d, cudaStream_t stream, uint32_t withhold_warp = 0,
                        const cm_paged_cache *paged = nullptr, const cm::RenderWidth *width = nullptr) {
-    // no width: the context's. The failure-injection hook withholds a TMA copy, so it runs
-    // the half-SM kernel (the TMA kernels are the ones that wait).
-    const cm::RenderWidth warps =
-        withhold_warp ? cm::RenderWidth::kHalf
-                      : width ? *width
-                              : (ctx->render_warps == 8 ? cm::RenderWidth::kHalf : cm::RenderWidth::kFull);
-    const int rows_per_chunk = (int)cm::render_item_bytes(warps) / (2 * d);
+    // no width: the context's, a full one by the launch's size. The failure-injection hook
+    // withholds a TMA copy, so it runs the half-SM kernel (the TMA kernels are the ones that wait).
+    const int reg_rows = (int)cm::render_item_bytes(cm::RenderWidth::kFullRegisters) / (2 * d);
+    auto width_of = [&](const Slot *s, size_t n) {
+        if (withhold_warp) return cm::RenderWidth::kHalf;
+        if (width) return *width;
+        if (ctx->render_warps == 8) return cm::RenderWidth::kHalf;
+        const uint64_t token_bytes = 4ull * (uint64_t)L * (uint64_t)H * (uint64_t)d;
+        cm::RenderLoad load{0, 0, 0, d, paged != nullptr};
+        for (size_t i = 0; i < n; ++i) {
+            const uint64_t T = (uint64_t)s[i].T;
+            load.reg_pairs += ceil_div(T, (uint64_t)reg_rows) * (uint64_t)L * (uint64_t)H;
+            load.bytes += T * token_bytes;
+            if (s[i].offset != 0) load.rotated_bytes += T * token_bytes;
+        }
+        return cm::full_render_width(load, ctx->num_sms);
+    };
     const int half = d / 2;
     const int max_group = std::min<int>(cm::kMaxSlots, cm::kMaxTablePairs / half);
     const uint64_t planes = 2ull * L * H;
@@ -575,6 +585,8 @@ cm_status launch_slots(cm_context *ctx, const std::vector<Slot> &slots, int32_t 
     cm::RenderParams *p = ctx->render_params.get();
     for (size_t g0 = 0; g0 < slots.size(); g0 += (size_t)max_group) {
         const size_t n = std::min(slots.size() - g0, (size_t)max_group);
+        const cm::RenderWidth warps = width_of(slots.data() + g0, n);
+        const int rows_per_chunk = (int)cm::render_item_bytes(warps) / (2 * d);
         // the kernel reads the header, slot[0, n) and the (cos, sin) pairs of those slots
         // that rotate, all written below; the rest of the block keeps older values
         std::memset(p, 0, offsetof(cm::RenderParams, slot));

@@ -61,6 +61,8 @@ struct RenderParams {
 // How much of each SM a render takes (the TMA kernel's widths are in render.cu):
 //   kFull         the TMA kernel, 20 warps per SM (cm_context_set_render_warps(16), the
 //                 default): the fastest render alone
+//   kFullRegisters  the register kernel, three 8-warp CTAs per SM: the renders alone that
+//                 full_render_width gives it
 //   kHalf         the TMA kernel, 8 warps per SM (cm_context_set_render_warps(8)): half of each
 //                 SM's registers stay free for kernels of other streams
 //   kBeside       the TMA kernel, 4 warps per SM: a large render beside the leaf hash of the same
@@ -72,11 +74,20 @@ struct RenderParams {
 // A launch group's work items are row chunks of render_item_bytes(w) bytes of one source
 // plane; render_grid gives the launch's CTA count for `chunks` items. render_prepare() once
 // per device before the first launch.
-enum class RenderWidth { kFull, kHalf, kBeside, kBesideSmall, kAfterLeaves };
+enum class RenderWidth { kFull, kFullRegisters, kHalf, kBeside, kBesideSmall, kAfterLeaves };
 cudaError_t launch_render(const RenderParams &p, int grid, RenderWidth w, cudaStream_t stream);
 cudaError_t render_prepare();
 uint32_t render_item_bytes(RenderWidth w);
 int render_grid(uint64_t chunks, int num_sms, RenderWidth w);
+// kFull or kFullRegisters: the faster full-SM width for a launch group.
+struct RenderLoad {
+    uint64_t reg_pairs;      // (K, V) pairs of items of render_item_bytes(kFullRegisters)
+    uint64_t bytes;          // of K and V
+    uint64_t rotated_bytes;  // of the slots at a nonzero offset
+    int head_dim;
+    bool paged;
+};
+RenderWidth full_render_width(const RenderLoad &l, int num_sms);
 
 // Bounds-checked builds: reads and zeroes the render kernels' violation count on the
 // current device (0 in other builds).

@@ -13,10 +13,11 @@
 // Two kernels move the items. In the TMA kernel (render_kernel) every warp keeps its items in
 // flight as 1-D bulk copies into its stages of shared memory; the full-SM render (the default)
 // takes an item from its stage into registers and refills the stage before it rotates and
-// stores, so that a steady 40 KiB of loads per SM is in flight, where HBM serves this mix of
-// reads and writes best (see TmaWidth, which gives its widths and what they measured). The
-// register kernel (render_reg_kernel) loads straight into registers and serves the small and
-// middling merges beside the content address (see RenderWidth). For a rotated K item a lane
+// stores, so that up to 40 KiB of loads per SM stay in flight while the warps store (see
+// TmaWidth, which gives its widths and what they measured). The register kernel
+// (render_reg_kernel) loads straight into registers and serves the small and middling merges
+// beside the content address (see RenderWidth) and the full-SM renders that full_render_width
+// gives it. For a rotated K item a lane
 // takes vector v of a row's first half and vector v of its second half: 8 (x, y) pairs that
 // share the lane's 8 (cos, sin) values.
 //
@@ -845,7 +846,13 @@ TmaWidth tma_width(RenderWidth w, bool paged) {
                                    : w == RenderWidth::kBeside ? kBesideWidth : kFullWidth;
 }
 
-bool is_tma(RenderWidth w) { return w != RenderWidth::kBesideSmall && w != RenderWidth::kAfterLeaves; }
+bool is_tma(RenderWidth w) {
+    return w == RenderWidth::kFull || w == RenderWidth::kHalf || w == RenderWidth::kBeside;
+}
+
+int reg_blocks_per_sm(RenderWidth w) {
+    return w == RenderWidth::kFullRegisters ? 3 : w == RenderWidth::kAfterLeaves ? 2 : 1;
+}
 
 // ---------------------------------------------------------------- register render
 
@@ -854,12 +861,13 @@ constexpr int kRegBlocksPerSm = 3;         // at most (80 registers)
 constexpr uint32_t kRegItemBytes = 1024;   // one work item: 2 vectors per lane
 constexpr int kRegVecs = kRegItemBytes / 16 / 32;
 
-// The widths of small and middling merges beside the content address (contiguous outputs):
-// persistent, one or two CTAs of 8 warps per SM, no shared-memory staging and no waits. Per
-// pair, each lane loads its 2 vectors of the K item (for a rotated item: vector v of the first
+// The widths of small and middling merges beside the content address (one or two CTAs per SM,
+// contiguous outputs) and of the renders alone that full_render_width gives it (three):
+// persistent, CTAs of 8 warps, no shared-memory staging and no waits. Per pair, each lane loads its 2 vectors of the K item (for a rotated item: vector v of the first
 // and of the second half of one row, v = lane mod (d/16)) and its 2 vectors of the V item, then
 // stores V, then rotates (slots at a nonzero offset) and stores K. The lane's 8 (cos, sin)
 // values are reloaded only when the slot changes.
+template <bool kPaged>
 __global__ void __launch_bounds__(kRegThreads, kRegBlocksPerSm)
 render_reg_kernel(const __grid_constant__ RenderParams p) {
     __shared__ float4 tab[kMaxTablePairs];   // (c1, c2, s1, s2) for the second level
@@ -880,7 +888,7 @@ render_reg_kernel(const __grid_constant__ RenderParams p) {
     w.stride = gridDim.x * (kRegThreads / 32);
     w.npairs = p.total_chunks / 2;
     if (w.pr >= w.npairs) return;
-    w.enter<false>(p);
+    w.enter<kPaged>(p);
     const int half_vecs = p.head_dim >> 4;
     const int vecs_per_row = p.head_dim >> 3;
     const int log2_hv = p.log2_pairs_per_row;
@@ -888,7 +896,7 @@ render_reg_kernel(const __grid_constant__ RenderParams p) {
     int cur = -1;
     float c[8], s[8];
     do {
-        const Pair q = pair_of<false>(p, w);
+        const Pair q = pair_of<kPaged>(p, w);
         const int n_vec = q.rows * vecs_per_row;
         const int n_pairs = q.rows * half_vecs;
         const uint4 *ks = reinterpret_cast<const uint4 *>(q.ks);
@@ -923,8 +931,10 @@ render_reg_kernel(const __grid_constant__ RenderParams p) {
         const uint32_t bytes = (uint32_t)n_vec * 16;
         Item vi = half_item(q, true), ki = half_item(q, false);
         vi.bytes = ki.bytes = bytes;
-        copy_from_regs<false>(p, vi, 0, rv, lane);
+        copy_from_regs<kPaged>(p, vi, 0, rv, lane);
         if (q.rotate) {
+            PagedRows pr{};
+            if (kPaged) pr = paged_rows(p, ki);
             if (q.cs_index != cur) {
                 cur = q.cs_index;
 #pragma unroll
@@ -942,13 +952,13 @@ render_reg_kernel(const __grid_constant__ RenderParams p) {
                     const uint4 a = rk[2 * k], b = rk[2 * k + 1];
                     uint4 ao, bo;
                     rotate_vectors(p, tab, kt, nst, cur + 8 * lane_v, c, s, a, b, ao, bo);
-                    store_pair<false>(p, ki, PagedRows{}, qq >> log2_hv, lane_v, ao, bo);
+                    store_pair<kPaged>(p, ki, pr, qq >> log2_hv, lane_v, ao, bo);
                 }
             }
         } else {
-            copy_from_regs<false>(p, ki, 0, rk, lane);
+            copy_from_regs<kPaged>(p, ki, 0, rk, lane);
         }
-    } while (w.next<false>(p));
+    } while (w.next<kPaged>(p));
 }
 
 }  // namespace
@@ -965,13 +975,32 @@ cudaError_t render_prepare() {
     return cudaSuccess;
 }
 
+// Measured as register kernel / TMA kernel (times in turn; "hot" back to back from L2, "cold"
+// from HBM, "after" right behind the ingest of the same fragments):
+//   pairs for at most one register CTA per SM: head_dim 16 and 32 0.78 to 0.95, 64 0.84 to 1.0,
+//     128 0.88 to 1.05, 512 0.82 to 0.88; with 1.5 times the pairs and head_dim 128 on 1.2 to 1.5
+//   head_dim up to 32 (contiguous): 15 to 60 MB cold 0.86 to 0.97, after 0.87 to 0.97, hot 1.02 to
+//     1.13; paged (items of 2 KiB longer than a 16-token block): up to 40 MB 0.77 to 0.98 on both,
+//     60 MB 1.05 to 1.13
+//   64 to 192 MiB, at most half of the tokens rotated: after 0.84 to 0.99, cold 0.92 to 1.04, hot
+//     0.80 to 1.03; three quarters rotated 0.88 to 1.02 up to head_dim 64, 1.01 to 1.24 above
+// Elsewhere the TMA kernel wins or the three disagree.
+RenderWidth full_render_width(const RenderLoad &l, int num_sms) {
+    constexpr uint64_t kMiB = 1ull << 20;
+    const bool small = l.reg_pairs <= (uint64_t)num_sms * (kRegThreads / 32);
+    const bool short_rows = l.head_dim <= 32 && l.bytes <= (l.paged ? 48 : 192) * kMiB;
+    const bool middling = !l.paged && l.bytes >= 64 * kMiB && l.bytes <= 192 * kMiB &&
+                          (2 * l.rotated_bytes <= l.bytes || l.head_dim <= 64);
+    return small || short_rows || middling ? RenderWidth::kFullRegisters : RenderWidth::kFull;
+}
+
 uint32_t render_item_bytes(RenderWidth w) { return is_tma(w) ? tma_width(w, false).item_bytes : kRegItemBytes; }
 
 int render_grid(uint64_t chunks, int num_sms, RenderWidth w) {
     const uint64_t sms = (uint64_t)num_sms;
     if (is_tma(w)) return (int)std::max<uint64_t>(1, std::min<uint64_t>(chunks / 2, sms));   // one CTA per SM
     const uint64_t ctas = (chunks / 2 + kRegThreads / 32 - 1) / (kRegThreads / 32);
-    return (int)std::max<uint64_t>(1, std::min<uint64_t>(ctas, (w == RenderWidth::kAfterLeaves ? 2 : 1) * sms));
+    return (int)std::max<uint64_t>(1, std::min<uint64_t>(ctas, (uint64_t)reg_blocks_per_sm(w) * sms));
 }
 
 cudaError_t launch_render(const RenderParams &p, int grid, RenderWidth w, cudaStream_t stream) {
@@ -986,7 +1015,7 @@ cudaError_t launch_render(const RenderParams &p, int grid, RenderWidth w, cudaSt
         const size_t smem = dyn_smem(t, entries);
         tma_kernel(w, p.paged != 0)<<<grid, t.warps * 32, smem, stream>>>(p);
     } else {
-        render_reg_kernel<<<grid, kRegThreads, 0, stream>>>(p);
+        (p.paged ? render_reg_kernel<true> : render_reg_kernel<false>)<<<grid, kRegThreads, 0, stream>>>(p);
     }
     return cudaGetLastError();
 }

@@ -140,3 +140,45 @@ def test_render_items_at_their_edges(ctx, L, H, d, lengths, warps):
     assert assert_k_parity(synthetic.to_bits(k[:, :, :n]), K_ref) == 0
     assert (k.view(torch.int16)[:, :, n:] == 0x3C3C).all() and (v.view(torch.int16)[:, :, n:] == 0x3C3C).all()
     S.close()
+
+
+# the lines between the full-SM render's two kernels on 152 SMs: 1,216 pairs of 1 KiB items (8
+# to 152 planes of K at a time), 48, 64 and 192 MiB of fragments, half of the tokens rotated
+@pytest.mark.parametrize("L,H,d,lengths", [
+    (19, 8, 128, (16, 16)), (19, 8, 128, (16, 17)), (19, 8, 128, (33, 7, 65)), (19, 8, 512, (4, 4)), (19, 8, 512, (4, 5)),
+    (19, 8, 64, (31, 34)), (16, 4, 64, (300, 333, 271)), (19, 8, 16, (300, 290)), (8, 4, 256, (39, 41, 43)),
+    (28, 8, 128, (292, 292)), (28, 8, 128, (293, 293)), (28, 8, 128, (293, 292, 5)), (28, 8, 128, (878, 877)),
+    (28, 8, 128, (878, 878)), (12, 12, 64, (1201, 700, 800)), (24, 8, 32, (1100, 948)), (24, 8, 32, (1100, 949))])
+def test_full_width_renders_on_both_sides_of_their_lines(ctx, L, H, d, lengths):
+    frags = [_fragment(13 * T + i, L, H, T, d) for i, T in enumerate(lengths)]
+    S = cm.FragmentSet(ctx)
+    S.ingest_batch(frags)
+    total = sum(lengths)
+    outs = {}
+    for warps in (16, 8):
+        cm.cm_context_set_render_warps(ctx.handle, warps)
+        k, v = empty_out(L, H, total + 1, d, fill=0x3C3C)
+        S.render(k, v)
+        outs[warps] = (k.view(torch.int16), v.view(torch.int16))
+        for block in (16, 24):
+            blocks = -(-total // block)
+            table = torch.randperm(blocks + 2, device="cuda:0")[:blocks].to(torch.int32)
+            pools = [torch.zeros((L, blocks + 2, block, H, d), dtype=torch.bfloat16, device="cuda:0") for _ in range(2)]
+            cm.cm_render_paged(S.handle, cm.cm_paged_cache(
+                pools[0].data_ptr(), pools[1].data_ptr(), table.data_ptr(), blocks, block,
+                pools[0].stride(1), pools[0].stride(0), pools[0].stride(3), pools[0].stride(2)))
+            pos = torch.arange(total, device="cuda:0")
+            for pool, flat in zip(pools, outs[warps]):
+                got = pool[:, table.long()[pos // block], pos % block].permute(0, 2, 1, 3).view(torch.int16)
+                assert torch.equal(got, flat[:, :, :total])
+            del pools
+        assert all((x[:, :, total:] == 0x3C3C).all() for x in outs[warps])
+    cm.cm_context_set_render_warps(ctx.handle, 16)
+    assert all(torch.equal(a, b) for a, b in zip(outs[16], outs[8]))
+    if L * H * total * d < 4 << 20:
+        import oracle
+        import synthetic
+        K_ref, V_ref, _ = oracle.render(oracle.from_deliveries([oracle_fragment(K, V) for K, V in frags]), THETA)
+        assert np.array_equal(synthetic.to_bits(outs[16][1][:, :, :total].view(torch.bfloat16)), V_ref)
+        assert np.array_equal(synthetic.to_bits(outs[16][0][:, :, :total].view(torch.bfloat16)), K_ref)
+    S.close()
