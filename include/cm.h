@@ -367,10 +367,11 @@ cm_status cm_context_check(cm_context *ctx, cm_stream_t stream);
  * records its set holds, then the earlier deliveries of the same call (identical (k, v)
  * pointers count as equal without reading them). A delivery found equal takes that
  * fragment's id and norm key and is not hashed; the others are hashed as usual. Results
- * (ids, absorption, the set) are identical with the path on or off. The candidates'
- * first 4 KiB are compared first; then each delivery with one candidate whose prefix
- * matched, in full, at HBM speed and beside the hashing of the others. This costs one more
- * stream synchronisation per call that has candidates (two if a matching prefix misled):
+ * (ids, absorption, the set) are identical with the path on or off. The candidates
+ * get a first look (8 KiB of each: the start of K and pieces spread over K and V to their
+ * ends); then each delivery is compared with the first that looked the same, in full, at HBM
+ * speed and beside the hashing of the others. This costs one more stream synchronisation per
+ * call that has candidates (two if a look misled):
  * turn it on where re-deliveries are common (gossip, retries). The paper has no counterpart. */
 cm_status cm_context_set_dedup_by_bytes(cm_context *ctx, int32_t enable);
 

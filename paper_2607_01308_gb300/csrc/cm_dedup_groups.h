@@ -31,9 +31,9 @@ inline int compare_fragments(const cm_fragment &a, const cm_fragment &b) {
     return 0;
 }
 
-// Fills the launch of n comparisons (n <= kMaxComparePairs), sorted by their bases: member m
-// is comparison m's, and neighbours of one base form a group. False if a member is not of its
-// base's size.
+// Fills the launch of n comparisons (n <= kMaxComparePairs): member m is comparison m's. A
+// comparison joins the group before it, unless that is full, if they have one base, or (a chain)
+// if it is with that group's last member. False if a member is not of its base's size.
 inline bool group_comparisons(const Comparison *c, size_t n, CompareFull &out) {
     std::memset(&out, 0, sizeof out);
     if (n > (size_t)kMaxComparePairs) return false;
@@ -41,13 +41,20 @@ inline bool group_comparisons(const Comparison *c, size_t n, CompareFull &out) {
         const cm_fragment &b = c[m].base, &f = c[m].member;
         const uint64_t vecs = fragment_vecs(b);
         if (fragment_vecs(f) != vecs) return false;
-        out.member[m] = {static_cast<const uint4 *>(f.k), static_cast<const uint4 *>(f.v), vecs};
-        if (m == 0 || compare_fragments(c[m - 1].base, b) != 0) {
-            const uint32_t g = out.groups++;
-            out.group[g] = {static_cast<const uint4 *>(b.k), static_cast<const uint4 *>(b.v), vecs, (uint32_t)m, 0};
-            out.chunk_begin[g + 1] = out.chunk_begin[g] + 2 * ((vecs + kCompareChunkVecs - 1) / kCompareChunkVecs);
+        out.member[m] = {{static_cast<const uint4 *>(f.k), static_cast<const uint4 *>(f.v)}, vecs};
+        CompareGroup *g = out.groups != 0 ? &out.group[out.groups - 1] : nullptr;
+        if (g != nullptr && g->end - g->begin == kMaxCompareGroup) g = nullptr;
+        const bool one = g != nullptr && g->end - g->begin == 1;   // not yet a chain or not
+        if (g != nullptr && (one || g->chain != 0) && compare_fragments(c[m - 1].member, b) == 0) {
+            g->chain = 1;
+        } else if (g == nullptr || g->chain != 0 || compare_fragments(c[m - 1].base, b) != 0) {
+            g = &out.group[out.groups];
+            *g = {{static_cast<const uint4 *>(b.k), static_cast<const uint4 *>(b.v)}, vecs, (uint32_t)m, 0, 0, 0};
+            out.chunk_begin[out.groups + 1] =
+                out.chunk_begin[out.groups] + 2 * ((vecs + kCompareChunkVecs - 1) / kCompareChunkVecs);
+            ++out.groups;
         }
-        out.group[out.groups - 1].end = (uint32_t)m + 1;
+        g->end = (uint32_t)m + 1;
     }
     return true;
 }

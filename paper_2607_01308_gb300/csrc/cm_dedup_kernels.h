@@ -10,31 +10,34 @@
 namespace cm {
 
 constexpr int kMaxComparePairs = 128;         // pairs (members) per launch
+constexpr uint32_t kMaxCompareGroup = 32;     // members of a group: a lane keeps track of each
 constexpr uint64_t kCompareChunkVecs = 2048;   // 16-byte vectors of each array per chunk
 
-// Two fragments of one shape, told apart by their K arrays' first 4 KiB: `vecs` 16-byte
-// vectors long. All pointers below are 16-byte aligned.
+// Two fragments of one shape, K and V `vecs` 16-byte vectors long each. All pointers below are
+// 16-byte aligned.
 struct ComparePair {
-    const uint4 *a_k, *b_k;
+    const uint4 *a_k, *a_v, *b_k, *b_v;
     uint64_t vecs;
 };
-struct ComparePrefix {
+struct CompareLook {
     uint32_t count;                               // pairs, <= kMaxComparePairs
     uint32_t pad_;
     ComparePair pair[kMaxComparePairs];
     uint32_t *differ;                             // one word per pair; may be mapped host memory
 };
 
-// Deliveries (members) that may equal one candidate (the group's base). K and V arrays are
+// Deliveries (members) that are compared in one walk: each with the group's base, or (a chain)
+// the first with the base and each other one with the member before it. K and V arrays are
 // `vecs` 16-byte vectors long, a member's as long as its base's.
 struct CompareMember {
-    const uint4 *k, *v;
+    const uint4 *kv[2];
     uint64_t vecs;
 };
 struct CompareGroup {
-    const uint4 *k, *v;                           // the base
+    const uint4 *kv[2];                           // the base
     uint64_t vecs;
-    uint32_t begin, end;                          // its members
+    uint32_t begin, end;                          // its members, at most kMaxCompareGroup
+    uint32_t chain, pad_;
 };
 struct CompareFull {
     uint32_t groups;                              // <= members <= kMaxComparePairs
@@ -46,12 +49,14 @@ struct CompareFull {
     uint32_t *differ;                             // device, one word per member, zeroed before
 };
 
-// differ[p] = 1 if the first 4 KiB of pair p's K arrays differ, else 0 (one block per pair).
-cudaError_t launch_compare_prefix(const ComparePrefix &c, cudaStream_t stream);
+// A first look at every pair: differ[p] = 1 if pair p's K arrays differ in their first 4 KiB, or
+// one of 16 pieces of 256 bytes spread over K and V to their ends differs, else 0 (one block per
+// pair). The start alone is the same in fragments whose tokens begin alike; their ends are not.
+cudaError_t launch_compare_look(const CompareLook &c, cudaStream_t stream);
 
-// differ[m] |= 1 if member m's K or V array differs from its group's base anywhere (a
-// persistent grid of blocks_per_sm blocks per SM over all chunks of all groups; a member
-// already found to differ is skipped).
+// differ[m] |= 1 if member m's K or V array differs anywhere from what it is compared with (a
+// persistent grid of blocks_per_sm blocks per SM over all chunks of all groups; what is already
+// known to differ is no longer read).
 cudaError_t launch_compare_full(const CompareFull &c, int num_sms, int blocks_per_sm, cudaStream_t stream);
 
 // Bounds-checked builds: reads and zeroes these kernels' violation count on the current device

@@ -723,8 +723,8 @@ cm_status guarded(F &&f) {
 // a fragment their set already holds or to an earlier delivery of the call. A
 // delivery is compared with at most kMaxCandidates fragments of its shape and length
 // (the set's records first, then the call's earlier deliveries, the latest first):
-// their first 4 KiB in one pass, then all bytes of one candidate whose prefix
-// matched; identical (k, v) pointers count as equal without a comparison.
+// 8 KiB of each in one pass, then all bytes of the first candidate that looked the same;
+// identical (k, v) pointers count as equal without a comparison.
 constexpr int kMaxCandidates = 16;
 
 struct Candidate {
@@ -734,10 +734,9 @@ struct Candidate {
 };
 
 // The first pass (synchronising `stream` if there is anything to compare): rec[i] / from[i]
-// for identical pointers; `chosen` gets, for each delivery with a candidate whose prefix
-// matched, the first such record or else the earliest such delivery (one full comparison
-// suffices, and copies of one fragment are then all compared with the same one).
-cm_status match_prefixes(cm_context *ctx, cm_set *const *sets,
+// for identical pointers; `chosen` gets, for each delivery with a candidate that looked the
+// same, the first such candidate (one full comparison suffices).
+cm_status first_look(cm_context *ctx, cm_set *const *sets,
                          const std::vector<const cm_fragment *> &fp, cudaStream_t stream,
                          std::vector<std::shared_ptr<const Record>> &rec,
                          std::vector<int32_t> &from, std::vector<Candidate> &chosen) {
@@ -787,19 +786,20 @@ cm_status match_prefixes(cm_context *ctx, cm_set *const *sets,
     cm_status st = ensure_scratch(ctx, bytes, bytes);
     if (st != CM_OK) return st;
     auto *differ = reinterpret_cast<uint32_t *>(ctx->h_pinned_dev ? ctx->h_pinned_dev : ctx->d_scratch);
-    std::unique_ptr<cm::ComparePrefix> cl(new cm::ComparePrefix);
+    std::unique_ptr<cm::CompareLook> cl(new cm::CompareLook);
     for (size_t c0 = 0; c0 < cands.size(); c0 += (size_t)cm::kMaxComparePairs) {
         const size_t cn = std::min(cands.size() - c0, (size_t)cm::kMaxComparePairs);
-        std::memset(cl.get(), 0, sizeof(cm::ComparePrefix));
+        std::memset(cl.get(), 0, sizeof(cm::CompareLook));
         for (size_t q = 0; q < cn; ++q) {
             const Candidate &c = cands[c0 + q];
             const cm_fragment *f = fp[c.delivery];
-            cl->pair[q] = {static_cast<const uint4 *>(f->k),
-                           static_cast<const uint4 *>(c.r ? c.r->k : fp[c.other]->k), cm::fragment_vecs(*f)};
+            cl->pair[q] = {static_cast<const uint4 *>(f->k), static_cast<const uint4 *>(f->v),
+                           static_cast<const uint4 *>(c.r ? c.r->k : fp[c.other]->k),
+                           static_cast<const uint4 *>(c.r ? c.r->v : fp[c.other]->v), cm::fragment_vecs(*f)};
         }
         cl->count = (uint32_t)cn;
         cl->differ = differ + c0;
-        CM_CUDA_TRY(cm::launch_compare_prefix(*cl, stream), "comparison launch");
+        CM_CUDA_TRY(cm::launch_compare_look(*cl, stream), "comparison launch");
         if (ctx->timing) ++ctx->aux_launches;
     }
     if (!ctx->h_pinned_dev)
@@ -807,29 +807,30 @@ cm_status match_prefixes(cm_context *ctx, cm_set *const *sets,
                     "comparison flags copy");
     CM_CUDA_TRY(cudaStreamSynchronize(stream), "comparison synchronisation");
     const auto *flags = reinterpret_cast<const uint32_t *>(ctx->h_pinned);
-    for (size_t c = 0; c < cands.size(); ++c) {
-        if (flags[c] != 0) continue;
-        if (chosen.empty() || chosen.back().delivery != cands[c].delivery)
+    for (size_t c = 0; c < cands.size(); ++c)
+        if (flags[c] == 0 && (chosen.empty() || chosen.back().delivery != cands[c].delivery))
             chosen.push_back(cands[c]);
-        else if (!chosen.back().r)
-            chosen.back() = cands[c];   // an earlier delivery
-    }
     return CM_OK;
 }
 
 // Enqueues the full comparisons of `chosen` on `stream`, one launch per kMaxComparePairs of
-// them, and sorts it by the fragment that each is compared with, so that the copies of one
-// fragment are compared together; their flags (one word each, in device scratch at dev_off) go
-// to the pinned buffer at host_off. Both offsets are multiples of 16 and the scratch already
-// reaches there.
+// them, and sorts it so that a fragment's copies are compared in one walk: those of one record,
+// and the chains of deliveries each compared with the one before. Their flags (one word each, in
+// device scratch at dev_off) go to the pinned buffer at host_off. Both offsets are multiples of
+// 16 and the scratch already reaches there.
 cm_status enqueue_comparisons(cm_context *ctx, const std::vector<const cm_fragment *> &fp,
                               std::vector<Candidate> &chosen, cudaStream_t stream,
                               int blocks_per_sm, size_t dev_off, size_t host_off) {
     auto base = [&](const Candidate &c) {
         return c.r ? cm_fragment{c.r->L, c.r->H, c.r->T, c.r->d, c.r->k, c.r->v} : *fp[c.other];
     };
+    std::vector<size_t> chain(fp.size());   // a delivery's chain, named by where it begins
+    for (size_t i = 0; i < chain.size(); ++i) chain[i] = i;
+    for (const Candidate &c : chosen)
+        if (!c.r) chain[c.delivery] = chain[c.other];
     std::stable_sort(chosen.begin(), chosen.end(), [&](const Candidate &a, const Candidate &b) {
-        return cm::compare_fragments(base(a), base(b)) < 0;
+        if (!a.r != !b.r) return !b.r;
+        return a.r ? cm::compare_fragments(base(a), base(b)) < 0 : chain[a.delivery] < chain[b.delivery];
     });
     std::vector<cm::Comparison> comparisons;
     comparisons.reserve(chosen.size());
@@ -1007,7 +1008,7 @@ struct SideJoin {
     }
 };
 
-// The full comparisons of `chosen` (match_prefixes) beside the content address of `hash`: the
+// The full comparisons of `chosen` (first_look) beside the content address of `hash`: the
 // comparisons are bound by HBM and run on the context's side stream, two blocks per SM, the
 // hash by the integer pipes on `cs`, which is synchronised. Results: differ (one flag per entry
 // of `chosen`, which is sorted anew), ids and Qs of `hash`.
@@ -1054,11 +1055,11 @@ cm_status ingest_validated(cm_context *ctx, cm_set *const *sets,
         return insert_deliveries(ctx, sets, fp, cs, src, ids, Q, out_ids, out_absorbed);
     }
     // deliveries byte-identical to a known fragment take its id and norm key and are not
-    // hashed: those with no candidate left after the prefix pass are hashed while the
+    // hashed: those with no candidate left after the first look are hashed while the
     // candidates are compared in full, those found to differ there afterwards
     DeliverySources src;
     std::vector<Candidate> chosen;
-    cm_status st = match_prefixes(ctx, sets, fp, cs, src.rec, src.from, chosen);
+    cm_status st = first_look(ctx, sets, fp, cs, src.rec, src.from, chosen);
     if (st != CM_OK) return st;
     src.hashed_as.assign(n, 0);
     auto hash_later = [&](size_t i) {

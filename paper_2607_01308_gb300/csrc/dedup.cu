@@ -4,7 +4,7 @@
 // is a function of the bytes, shapes and dtype), so once its bytes are shown equal to
 // a fragment whose address is known or being computed, it need not be hashed. The
 // comparison reads both fragments once at HBM speed; the hash is bound by the
-// integer ALU. Pairs that differ are usually told apart by their first 4 KiB.
+// integer ALU. Pairs that differ are usually told apart by a first look at 8 KiB of them.
 #include "cm_bounds.h"
 #include "cm_dedup_kernels.h"
 
@@ -12,7 +12,8 @@ namespace cm {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr uint64_t kPrefixVecs = 256;                   // 4 KiB
+constexpr uint32_t kPieces = 16, kPieceVecs = 16;       // of the first look: 256 bytes each
+static_assert(kPieces * kPieceVecs == (uint32_t)kThreads, "a thread compares one vector of a piece");
 constexpr uint64_t kChunkVecs = kCompareChunkVecs;      // 32 KiB of each array per chunk
 constexpr int kStepVecs = 4;                            // vectors per thread at a time
 static_assert(kChunkVecs % ((uint64_t)kThreads * kStepVecs) == 0, "a chunk is a number of whole steps");
@@ -27,51 +28,81 @@ __device__ __forceinline__ uint4 load_vec(const uint4 *p, uint64_t i, [[maybe_un
     return CM_IN_BOUNDS(p + i, 16, p, n * 16) ? __ldcs(p + i) : make_uint4(0, 0, 0, 0);
 }
 
-// One block per pair: the first 4 KiB of K.
-__global__ void __launch_bounds__(kThreads) prefix_kernel(const __grid_constant__ ComparePrefix c) {
+// One block per pair: a vector of K's first 4 KiB and one of the spread pieces per thread.
+__global__ void __launch_bounds__(kThreads) look_kernel(const __grid_constant__ CompareLook c) {
     const ComparePair &p = c.pair[blockIdx.x];
-    const uint64_t n = p.vecs < kPrefixVecs ? p.vecs : kPrefixVecs;
+    const uint32_t t = threadIdx.x, piece = t / kPieceVecs;
+    const bool in_v = piece >= kPieces / 2;
+    const uint64_t room = p.vecs > kPieceVecs ? p.vecs - kPieceVecs : 0;   // the last piece begins here
+    const uint64_t i = piece % (kPieces / 2) * room / (kPieces / 2 - 1) + t % kPieceVecs;
     uint32_t d = 0;
-    for (uint64_t i = threadIdx.x; i < n; i += kThreads) d |= diff4(load_vec(p.a_k, i, p.vecs), load_vec(p.b_k, i, p.vecs));
+    if (t < p.vecs) d |= diff4(load_vec(p.a_k, t, p.vecs), load_vec(p.b_k, t, p.vecs));
+    if (i < p.vecs) d |= diff4(load_vec(in_v ? p.a_v : p.a_k, i, p.vecs), load_vec(in_v ? p.b_v : p.b_k, i, p.vecs));
     const int any = __syncthreads_or(d != 0);
-    if (threadIdx.x == 0) c.differ[blockIdx.x] = any ? 1u : 0u;
+    if (t == 0) c.differ[blockIdx.x] = any ? 1u : 0u;
 }
 
 // Persistent grid over the chunks of all groups (K then V of each): a warp loads its part of
-// the base's chunk and compares every member's with it, so the base is read once for all its
-// members (bound by HBM: (members + 1) reads of a fragment instead of 2 per member). Members
-// that another warp has found to differ are skipped.
+// the base's chunk and of every member's, so that a fragment is read once for all its copies
+// (bound by HBM: (members + 1) reads instead of 2 per member). What other warps have found to
+// differ is learnt once per chunk, a lane to a member; such a member is read only where the next
+// of its chain is compared with it, and a group whose members all differ is left. Beside the
+// hash, which is bound by issue slots, instructions and registers count: on six copies alone 8
+// vectors a step took 152 us, 4 185, but a merge of nine deliveries hashed beside it 420 and 369.
 __global__ void __launch_bounds__(kThreads) full_kernel(const __grid_constant__ CompareFull c) {
     const uint64_t total = c.chunk_begin[c.groups];
-    uint32_t gi = 0;
+    const uint32_t lane = threadIdx.x % 32;
+    uint32_t gi = 0, closed = 0;   // the group's members known to differ
     for (uint64_t x = blockIdx.x; x < total; x += gridDim.x) {
-        while (x >= c.chunk_begin[gi + 1]) ++gi;
+        for (; x >= c.chunk_begin[gi + 1]; ++gi) closed = 0;
         const CompareGroup &g = c.group[gi];
+        const uint32_t members = g.end - g.begin, all = 0xFFFFFFFFu >> (32 - members);
+        if (closed == all) {
+            // to this block's first chunk past the group: x + k gridDim with
+            // k = ceil((end of group - x) / gridDim) >= 1 (the loop adds the last gridDim)
+            x += ((c.chunk_begin[gi + 1] - x + gridDim.x - 1) / gridDim.x - 1) * (uint64_t)gridDim.x;
+            continue;
+        }
+        const uint32_t found = lane < members ? __ldcg(c.differ + g.begin + lane) : 0u;   // for the next chunk
+        // the members to read, and whether the base
+        const uint32_t open = ~closed & all, read = g.chain != 0 ? open | open >> 1 : open;
+        const bool read_base = g.chain == 0 || (open & 1u) != 0;
         // chunk index within the group: the K chunks, then the V chunks
         const uint64_t per_array = (g.vecs + kChunkVecs - 1) / kChunkVecs;
         const uint64_t local = x - c.chunk_begin[gi];
-        const bool is_v = local >= per_array;
+        const uint32_t is_v = local >= per_array;
         const uint64_t begin = (is_v ? local - per_array : local) * kChunkVecs;
         const uint64_t end = begin + kChunkVecs < g.vecs ? begin + kChunkVecs : g.vecs;
-        const uint4 *base = is_v ? g.v : g.k;
 #pragma unroll 1
-        for (uint64_t i = begin + threadIdx.x; i < end; i += (uint64_t)kThreads * kStepVecs) {
-            uint4 b[kStepVecs];
-#pragma unroll
-            for (int u = 0; u < kStepVecs; ++u)
-                b[u] = i + (uint64_t)u * kThreads < end ? load_vec(base, i + (uint64_t)u * kThreads, g.vecs)
-                                                        : make_uint4(0, 0, 0, 0);
-            for (uint32_t m = g.begin; m < g.end; ++m) {
-                if (__ldcg(c.differ + m) != 0) continue;
-                const uint4 *a = is_v ? c.member[m].v : c.member[m].k;
-                uint32_t d = 0;
+        for (uint64_t at = begin; at < end; at += (uint64_t)kThreads * kStepVecs) {
+            const uint64_t i = at + threadIdx.x;
+            const bool whole = at + (uint64_t)kThreads * kStepVecs <= end;
+            auto load = [&](const uint4 *p, uint64_t vecs, uint4 (&r)[kStepVecs]) {
 #pragma unroll
                 for (int u = 0; u < kStepVecs; ++u)
-                    if (i + (uint64_t)u * kThreads < end)
-                        d |= diff4(load_vec(a, i + (uint64_t)u * kThreads, c.member[m].vecs), b[u]);
-                if (d != 0) atomicOr(c.differ + m, 1u);
+                    r[u] = whole || i + (uint64_t)u * kThreads < end ? load_vec(p, i + (uint64_t)u * kThreads, vecs)
+                                                                     : make_uint4(0, 0, 0, 0);
+            };
+            uint4 b[kStepVecs], a[kStepVecs];
+            if (read_base) load(g.kv[is_v], g.vecs, b);
+            // member m into `a`, compared with `b`, which may be anything if m is known to differ
+            auto member = [&](uint32_t m, const uint4 (&b)[kStepVecs], uint4 (&a)[kStepVecs]) {
+                if ((read >> m & 1u) == 0) return;
+                const CompareMember &f = c.member[g.begin + m];
+                load(f.kv[is_v], f.vecs, a);
+                uint32_t d = 0;
+#pragma unroll
+                for (int u = 0; u < kStepVecs; ++u) d |= diff4(a[u], b[u]);
+                if ((open >> m & 1u) != 0 && __any_sync(0xFFFFFFFFu, d != 0) && lane == 0)
+                    atomicOr(c.differ + g.begin + m, 1u);
+            };
+#pragma unroll 1
+            for (uint32_t m = 0; m < members; ++m) {
+                member(m, b, a);
+                if (g.chain != 0 && ++m < members) member(m, a, b);   // in turn: no copies
             }
         }
+        closed |= __ballot_sync(0xFFFFFFFFu, found != 0);
     }
 }
 
@@ -79,9 +110,9 @@ __global__ void __launch_bounds__(kThreads) full_kernel(const __grid_constant__ 
 
 CM_DEFINE_BOUNDS_READER(take_dedup_bounds_violations)
 
-cudaError_t launch_compare_prefix(const ComparePrefix &c, cudaStream_t stream) {
+cudaError_t launch_compare_look(const CompareLook &c, cudaStream_t stream) {
     if (c.count == 0) return cudaSuccess;
-    prefix_kernel<<<c.count, kThreads, 0, stream>>>(c);
+    look_kernel<<<c.count, kThreads, 0, stream>>>(c);
     return cudaGetLastError();
 }
 

@@ -20,29 +20,39 @@ alignas(16) unsigned char buffers[16][64];   // addresses only: nothing is read
 
 cm_fragment fragment(int k, int L, int H, int T, int d) { return {L, H, T, d, buffers[2 * k], buffers[2 * k + 1]}; }
 
-// Every member in one group, of its own base and size; chunks as long as the sizes say.
-int check(std::vector<cm::Comparison> c, uint32_t want_groups) {
-    std::stable_sort(c.begin(), c.end(), [](const cm::Comparison &a, const cm::Comparison &b) {
-        return cm::compare_fragments(a.base, b.base) < 0;
-    });
+// Every member in one group, compared with its own base (the one before it, in a chain) over its
+// own size; chunks as long as the sizes say.
+int check_in_order(const std::vector<cm::Comparison> &c, uint32_t want_groups, uint32_t want_chains) {
     static cm::CompareFull out;
     CHECK(cm::group_comparisons(c.data(), c.size(), out));
     CHECK(out.groups == want_groups);
     uint32_t m = 0;
     for (uint32_t g = 0; g < out.groups; ++g) {
         const cm::CompareGroup &q = out.group[g];
-        CHECK(q.begin == m && q.end > m);
+        CHECK(q.begin == m && q.end > m && q.end - q.begin <= cm::kMaxCompareGroup);
         for (; m < q.end; ++m) {
             const uint64_t vecs = cm::fragment_vecs(c[m].member);
-            CHECK(q.k == c[m].base.k && q.v == c[m].base.v);
+            const bool first = m == q.begin || q.chain == 0;
+            CHECK((first ? q.kv[0] : out.member[m - 1].kv[0]) == c[m].base.k);
+            CHECK((first ? q.kv[1] : out.member[m - 1].kv[1]) == c[m].base.v);
             CHECK(q.vecs == vecs && out.member[m].vecs == vecs);
-            CHECK(out.member[m].k == c[m].member.k && out.member[m].v == c[m].member.v);
+            CHECK(out.member[m].kv[0] == c[m].member.k && out.member[m].kv[1] == c[m].member.v);
         }
         const uint64_t chunks = 2 * ((q.vecs + cm::kCompareChunkVecs - 1) / cm::kCompareChunkVecs);
         CHECK(out.chunk_begin[g + 1] - out.chunk_begin[g] == chunks);
     }
     CHECK(m == c.size());
+    uint32_t chains = 0;
+    for (uint32_t g = 0; g < out.groups; ++g) chains += out.group[g].chain;
+    CHECK(chains == want_chains);
     return 0;
+}
+
+int check(std::vector<cm::Comparison> c, uint32_t want_groups) {
+    std::stable_sort(c.begin(), c.end(), [](const cm::Comparison &a, const cm::Comparison &b) {
+        return cm::compare_fragments(a.base, b.base) < 0;
+    });
+    return check_in_order(c, want_groups, 0);
 }
 
 }  // namespace
@@ -68,13 +78,22 @@ int main() {
     const cm_fragment a = fragment(0, 3, 2, 50, 64), b = fragment(1, 3, 2, 50, 64);
     if (check({{a, fragment(2, 3, 2, 50, 64)}, {b, fragment(3, 3, 2, 50, 64)}, {a, fragment(4, 3, 2, 50, 64)}}, 2) != 0)
         return 1;
+    // a chain is one group; its end, another chain and a base with several copies are not in it
+    const cm_fragment f[6] = {a, b, fragment(2, 3, 2, 50, 64), fragment(3, 3, 2, 50, 64), fragment(4, 3, 2, 50, 64),
+                              fragment(5, 3, 2, 50, 64)};
+    if (check_in_order({{f[0], f[1]}, {f[1], f[2]}, {f[2], f[3]}}, 1, 1) != 0) return 1;
+    if (check_in_order({{f[0], f[1]}, {f[1], f[2]}, {f[3], f[4]}, {f[4], f[5]}}, 2, 2) != 0) return 1;
+    if (check_in_order({{f[0], f[1]}, {f[0], f[2]}, {f[2], f[3]}, {f[3], f[4]}}, 2, 1) != 0) return 1;
+    if (check_in_order({{f[0], f[1]}, {f[1], f[2]}, {f[1], f[3]}}, 2, 1) != 0) return 1;
+    // (a part of a fragment that ends a chain is another fragment)
+    if (check_in_order({{f[0], f[1]}, {fragment(1, 2, 2, 50, 64), fragment(2, 2, 2, 50, 64)}}, 2, 0) != 0) return 1;
     // sizes that differ are refused, and so are more than a launch holds
     static cm::CompareFull out;
     const cm::Comparison wrong{a, fragment(2, 2, 2, 50, 64)};
     CHECK(!cm::group_comparisons(&wrong, 1, out));
     const std::vector<cm::Comparison> many(cm::kMaxComparePairs + 1, {a, b});
     CHECK(!cm::group_comparisons(many.data(), many.size(), out));
-    CHECK(cm::group_comparisons(many.data(), many.size() - 1, out) && out.groups == 1);
+    CHECK(cm::group_comparisons(many.data(), many.size() - 1, out) && out.groups == 4);   // full ones
     std::printf("ok\n");
     return 0;
 }

@@ -175,6 +175,56 @@ def test_fragments_that_start_at_one_address(ctxs, shape, layers, tokens, one_ca
         assert [len(i) for i in ids] == [2, 1]        # the near-copy is a fragment of its own
 
 
+# thoughts of one prompt (their first tokens' K and V are equal in every layer), and fragments
+# that differ in one bit: re-sent copies of either are recognised, and only the two are hashed
+@pytest.mark.parametrize("bit", [None, ("k", 0), ("k", 20000), ("v", 30000), ("v", -1)])
+def test_copies_of_fragments_that_begin_alike_are_not_hashed(ctxs, bit):
+    off, on = ctxs
+    A, B = _frags(940, [200, 200], 4, 2, 64)
+    if bit is None:
+        for x, y in zip(A, B):
+            y[:, :, :120] = x[:, :, :120]
+    else:
+        B = _flip(A, *bit)
+    for order in ("ABBB", "ABBAA", "BAAABB"):
+        originals, msgs = set(), []
+        for c in order:
+            msgs.append(_clone(A if c == "A" else B) if c in originals else (A if c == "A" else B))
+            originals.add(c)
+        S, T = cm.FragmentSet(on), cm.FragmentSet(off)
+        res, t = _timed(on, lambda: S.ingest_batch(msgs))
+        assert res == T.ingest_batch(msgs)
+        assert [fid for fid, _ in res] == [oracle_fragment(*(A if c == "A" else B)).fid for c in order]
+        # a copy right behind another of its kind is always recognised; one with the other kind in
+        # between where the first look tells the two apart
+        runs = 1 + sum(x != y for x, y in zip(order, order[1:]))
+        assert t["leaf_hash_fragments"] <= (2 if bit in (None, ("k", 0), ("v", -1)) else runs)
+        S.close()
+        T.close()
+
+
+# more copies than a group (32) or a launch (128) of comparisons holds, of a fragment of the call
+# (a chain) and of a record; one in between and the last differ in one bit that the first look misses
+@pytest.mark.parametrize("held", [False, True])
+def test_more_copies_than_a_group_or_a_launch_holds(ctxs, held):
+    off, on = ctxs
+    A, = _frags(950, [120], 4, 2, 64)
+    near = _flip(A, "k", 20000)
+    msgs = [_clone(A) for _ in range(150)]
+    msgs[70], msgs[-1] = near, _clone(near)
+    got = []
+    for ctx in (off, on):
+        S = cm.FragmentSet(ctx)
+        res = S.ingest_batch([A]) if held else []
+        more, t = _timed(ctx, lambda: S.ingest_batch(msgs))
+        got.append((res + more, S.ids()))
+        S.close()
+    assert got[0] == got[1] and len(got[1][1]) == 2
+    # hashed: the first of a chain, what differs from the one before it (from the record); in a
+    # launch's first place a copy is compared with the one before as well
+    assert t["leaf_hash_fragments"] <= (2 if held else 4)
+
+
 @pytest.mark.parametrize("seed", range(10))
 def test_random_redeliveries_equal_the_path_off(ctxs, seed):
     # seeded random merges (the generator of test_gpu_random.py) with every delivery a
