@@ -194,7 +194,10 @@ def _id_array(ids: Sequence[bytes]):
     for i, fid in enumerate(ids):
         if len(fid) != 16:
             raise ValueError("an id has 16 bytes")
-        ctypes.memmove(ctypes.byref(arr, 16 * i), bytes(fid), 16)
+        if isinstance(fid, bytes):
+            ctypes.memmove(ctypes.byref(arr, 16 * i), fid, 16)
+        else:
+            arr[i].b[:] = list(fid)   # entry by entry: the entries may be wider than a byte
     return arr
 
 
