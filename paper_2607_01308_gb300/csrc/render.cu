@@ -203,7 +203,8 @@ __device__ __forceinline__ void fixup_pair(const RenderParams &p, const float4 *
             *pw[w] = (*pw[w] & 0xFFFF0000u) | (r >> 16);
         }
         if (bw[w] >> 16) {
-            const uint32_t r = fix_element(bf16_hi(xw[w]), bf16_hi(yw[w]), tab[c0 + 1], p.cs[2 * c0 + 2], p.cs[2 * c0 + 3]);
+            const uint32_t r = fix_element(bf16_hi(xw[w]), bf16_hi(yw[w]), tab[c0 + 1], p.cs[2 * c0 + 2],
+                                           p.cs[2 * c0 + 3]);
             *ow[w] = (*ow[w] & 0xFFFFu) | (r << 16);
             *pw[w] = (*pw[w] & 0xFFFFu) | (r & 0xFFFF0000u);
         }
@@ -274,16 +275,17 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
 }
 
 // The TMA kernel's widths: warps per CTA (one CTA per SM), bytes of a work item (= of a stage)
-// and stages per warp. More loads in flight per SM than these make HBM serve this mix of reads
-// and writes worse (a plain copy kernel took 0.70 ms for 2.4 GB with 28 to 32 KiB in flight per
-// SM, 0.75 with 40 and more), fewer leave it idle; larger items cost fewer instructions each.
+// and stages per warp. Larger items cost fewer instructions each; more bytes of stages than
+// these (40 KiB per SM alone, 64 and 96 at half width, 128 beside) were slower.
 //   full        20 warps, 2 KiB, through registers: measured for 4 x 4096 tokens / paged 5,208
 //               tokens 716 / 239 us; 16, 19, 21, 24 warps 742 / 258, 747 / 254, 759 / 260,
-//               764 / 267; 4 KiB at 11 warps 715 / 265; not through registers 735 / 277; as the
-//               register kernel below, three CTAs per SM, 752 / 251
+//               764 / 267; 4 KiB at 11 warps 715 / 265; not through registers 735 / 277; the
+//               register kernel, three CTAs per SM, 752 / 251; two stages 652 against 598 us on
+//               2 GB of fragments
 //   half        8 warps, 4 KiB, two stages (paged: three): 750 / 248 us alone, with three
 //               805 / 248, with two 750 / 257; a serving group hashed beside it 5.81 ms with
-//               two, 5.98 with three
+//               two, 5.98 with three (renders of 8 to 60 MB whose inputs are not in L2 are 0 to
+//               7 % faster with three, the others 3 to 13 % with two)
 //   beside      4 warps, 16 KiB, two stages: the 4 x 4096-token merge 1.597 ms, 4 x 2048 841 us;
 //               8 KiB x 2 1.599, 849; 8 KiB x 3 1.612, 849; 4 KiB x 6 1.647, 865
 struct TmaWidth {
@@ -863,10 +865,11 @@ constexpr int kRegVecs = kRegItemBytes / 16 / 32;
 
 // The widths of small and middling merges beside the content address (one or two CTAs per SM,
 // contiguous outputs) and of the renders alone that full_render_width gives it (three):
-// persistent, CTAs of 8 warps, no shared-memory staging and no waits. Per pair, each lane loads its 2 vectors of the K item (for a rotated item: vector v of the first
-// and of the second half of one row, v = lane mod (d/16)) and its 2 vectors of the V item, then
-// stores V, then rotates (slots at a nonzero offset) and stores K. The lane's 8 (cos, sin)
-// values are reloaded only when the slot changes.
+// persistent, CTAs of 8 warps, no shared-memory staging and no waits. Per pair, each lane loads
+// its 2 vectors of the K item (for a rotated item: vector v of the first and of the second half
+// of one row, v = lane mod (d/16)) and its 2 vectors of the V item, then stores V, then rotates
+// (slots at a nonzero offset) and stores K. The lane's 8 (cos, sin) values are reloaded only
+// when the slot changes.
 template <bool kPaged>
 __global__ void __launch_bounds__(kRegThreads, kRegBlocksPerSm)
 render_reg_kernel(const __grid_constant__ RenderParams p) {
@@ -968,8 +971,9 @@ CM_DEFINE_BOUNDS_READER(take_render_bounds_violations)
 cudaError_t render_prepare() {
     for (RenderWidth w : {RenderWidth::kFull, RenderWidth::kHalf, RenderWidth::kBeside})
         for (bool paged : {false, true}) {
-            const cudaError_t e = cudaFuncSetAttribute(tma_kernel(w, paged), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                       (int)dyn_smem(tma_width(w, paged), kMaxTablePairs));
+            const int smem = (int)dyn_smem(tma_width(w, paged), kMaxTablePairs);
+            const cudaError_t e =
+                cudaFuncSetAttribute(tma_kernel(w, paged), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
             if (e != cudaSuccess) return e;
         }
     return cudaSuccess;
@@ -982,14 +986,15 @@ cudaError_t render_prepare() {
 //   head_dim up to 32 (contiguous): 15 to 60 MB cold 0.86 to 0.97, after 0.87 to 0.97, hot 1.02 to
 //     1.13; paged (items of 2 KiB longer than a 16-token block): up to 40 MB 0.77 to 0.98 on both,
 //     60 MB 1.05 to 1.13
-//   64 to 192 MiB, at most half of the tokens rotated: after 0.84 to 0.99, cold 0.92 to 1.04, hot
-//     0.80 to 1.03; three quarters rotated 0.88 to 1.02 up to head_dim 64, 1.01 to 1.24 above
+//   62 (from where fragments and outputs outgrow L2) to 192 MiB, at most half of the tokens
+//     rotated: after 0.84 to 1.03, cold 0.92 to 1.04, hot 0.78 to 1.03 (at 55 MB 1.13 to 1.23);
+//     two thirds or three quarters rotated 0.88 to 1.03 up to head_dim 64, 1.01 to 1.24 above
 // Elsewhere the TMA kernel wins or the three disagree.
 RenderWidth full_render_width(const RenderLoad &l, int num_sms) {
     constexpr uint64_t kMiB = 1ull << 20;
     const bool small = l.reg_pairs <= (uint64_t)num_sms * (kRegThreads / 32);
     const bool short_rows = l.head_dim <= 32 && l.bytes <= (l.paged ? 48 : 192) * kMiB;
-    const bool middling = !l.paged && l.bytes >= 64 * kMiB && l.bytes <= 192 * kMiB &&
+    const bool middling = !l.paged && l.bytes >= 62 * kMiB && l.bytes <= 192 * kMiB &&
                           (2 * l.rotated_bytes <= l.bytes || l.head_dim <= 64);
     return small || short_rows || middling ? RenderWidth::kFullRegisters : RenderWidth::kFull;
 }
@@ -1015,7 +1020,8 @@ cudaError_t launch_render(const RenderParams &p, int grid, RenderWidth w, cudaSt
         const size_t smem = dyn_smem(t, entries);
         tma_kernel(w, p.paged != 0)<<<grid, t.warps * 32, smem, stream>>>(p);
     } else {
-        (p.paged ? render_reg_kernel<true> : render_reg_kernel<false>)<<<grid, kRegThreads, 0, stream>>>(p);
+        const RenderKernel kernel = p.paged ? render_reg_kernel<true> : render_reg_kernel<false>;
+        kernel<<<grid, kRegThreads, 0, stream>>>(p);
     }
     return cudaGetLastError();
 }

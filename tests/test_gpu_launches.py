@@ -143,11 +143,12 @@ def test_render_items_at_their_edges(ctx, L, H, d, lengths, warps):
 
 
 # the lines between the full-SM render's two kernels on 152 SMs: 1,216 pairs of 1 KiB items (8
-# to 152 planes of K at a time), 48, 64 and 192 MiB of fragments, half of the tokens rotated
+# to 152 planes of K at a time), 48, 62 and 192 MiB of fragments, half of the tokens rotated
 @pytest.mark.parametrize("L,H,d,lengths", [
-    (19, 8, 128, (16, 16)), (19, 8, 128, (16, 17)), (19, 8, 128, (33, 7, 65)), (19, 8, 512, (4, 4)), (19, 8, 512, (4, 5)),
-    (19, 8, 64, (31, 34)), (16, 4, 64, (300, 333, 271)), (19, 8, 16, (300, 290)), (8, 4, 256, (39, 41, 43)),
-    (28, 8, 128, (292, 292)), (28, 8, 128, (293, 293)), (28, 8, 128, (293, 292, 5)), (28, 8, 128, (878, 877)),
+    (19, 8, 128, (16, 16)), (19, 8, 128, (16, 17)), (19, 8, 128, (33, 7, 65)), (19, 8, 512, (4, 4)),
+    (19, 8, 512, (4, 5)), (19, 8, 64, (31, 34)), (16, 4, 64, (300, 333, 271)),
+    (19, 8, 16, (300, 290)), (8, 4, 256, (39, 41, 43)),
+    (28, 8, 128, (283, 283)), (28, 8, 128, (284, 283)), (28, 8, 128, (280, 282, 5)), (28, 8, 128, (878, 877)),
     (28, 8, 128, (878, 878)), (12, 12, 64, (1201, 700, 800)), (24, 8, 32, (1100, 948)), (24, 8, 32, (1100, 949))])
 def test_full_width_renders_on_both_sides_of_their_lines(ctx, L, H, d, lengths):
     frags = [_fragment(13 * T + i, L, H, T, d) for i, T in enumerate(lengths)]
