@@ -2,10 +2,11 @@
 named by the environment variable CM_LIBRARY; started by test_gpu_bounds.py).
 
 Every global access of the render, content-address and byte-comparison kernels is checked
-against the buffer it belongs to in that build. The cases below cover every kernel path (both render
-widths, contiguous, paged with power-of-two and other block sizes, both tree-top schemes,
-the allocation-free path, the re-delivery comparison, BagMerge, the incremental render and
-both renders that run beside the leaf hash in cm_ingest_render);
+against the buffer it belongs to in that build. The cases below cover every kernel path (the full-SM
+render by both of its kernels and the half-SM one, contiguous, paged with power-of-two and
+other block sizes, both tree-top schemes, leaves by one lane and by four, whole and straddling
+segments, the allocation-free path, the re-delivery comparison, BagMerge, the incremental
+render and the three renders that cm_ingest_render runs beside the content address);
 their results are checked against the oracle or against each other, and the violation
 count must stay 0. A last case renders into a paged cache whose block table holds a
 negative entry, an input the host does not check: the bounds-checked build must count it
@@ -114,6 +115,31 @@ def main():
         assert torch.equal(kg, kc) and torch.equal(vg, vc)
         cases += 1
 
+    # the same at half width, and renders large enough for the full-SM TMA kernel (2,280 pairs of
+    # 1 KiB items and more), contiguous and paged: items at the ends of planes and blocks
+    cm.cm_context_set_render_warps(ctx.handle, 8)
+    for bs in (16, 12):
+        kg, vg = paged_render(ctx, fr, bs)
+        assert torch.equal(kg, kc) and torch.equal(vg, vc)
+        cases += 1
+    cm.cm_context_set_render_warps(ctx.handle, 16)
+    for d, lengths in ((128, (33, 7, 19)), (512, (5, 6, 4)), (64, (60, 41, 33))):
+        fl = frags_of(12 + d, 19, 8, d, lengths)
+        kl, vl, _ = check_render(ctx, fl)
+        for bs in (16, 12):
+            kg, vg = paged_render(ctx, fl, bs)
+            assert torch.equal(kg, kl) and torch.equal(vg, vl)
+        cases += 3
+
+    # straddling leaves by one lane each (the four-lane kernel takes the smaller launches above),
+    # alone and beside a fragment of whole segments
+    st = frags_of(13, 8, 3, 64, (3201,)) + frags_of(14, 8, 3, 64, (1024,))
+    for part in (st[:1], st):
+        S = cm.FragmentSet(ctx)
+        assert [r[0] for r in S.ingest_batch(part)] == [oracle_fragment(K, V).fid for K, V in part]
+        S.close()
+        cases += 1
+
     # allocation-free content address
     K, V = fr[0]
     L, H, T, d = K.shape
@@ -161,6 +187,26 @@ def main():
     for X in (A, B, S):
         X.close()
     del big, fused_k, fused_v, seq_k, seq_v
+    cases += 1
+    # a middling one (a leaf grid of more than a wave, less than 272 MiB): the register render,
+    # two CTAs per SM, starts as the leaves end
+    mid = frags_of(62, 28, 8, 128, (700, 705, 690))
+    outs = []
+    for fused in (True, False):
+        A = cm.FragmentSet(ctx)
+        km, vm = empty_out(28, 8, 2095, 128)
+        if fused:
+            _, n, _, overlapped = cm.cm_ingest_render([A.handle] * 3, [cm.fragment_from_tensors(K, V) for K, V in mid],
+                                                      A.handle, km.data_ptr(), vm.data_ptr(), 2095)
+            assert overlapped and n == 2095
+        else:
+            A.ingest_batch(mid)
+            A.render(km, vm)
+        torch.cuda.synchronize()
+        outs.append((km.view(torch.int16), vm.view(torch.int16)))
+        A.close()
+    assert all(torch.equal(a, b) for a, b in zip(*outs))
+    del mid, outs, km, vm
     cases += 1
     # a small merge through cm_ingest_render (the register render, one CTA per SM, beside
     # the hash), checked against the oracle
