@@ -6,8 +6,9 @@
 // 1024-byte leaves (depth 0), inner nodes over 16 child digests, 16-byte
 // digests, shapes and dtype in the salt, seq_len in the personalisation.
 //
-// Level 0 runs one thread per leaf: 16 compressions of 64-byte blocks, loaded as
-// 128-bit vectors straight from the fragment buffers. A launch beside it computes the norm key from K[l*]: a row's squared norm in fp64 in ascending element
+// Level 0 runs one thread per leaf (four lanes, where there are few): 16 compressions of
+// 64-byte blocks, loaded as 128-bit vectors straight from the fragment buffers. A launch beside
+// it computes the norm key from K[l*]: a row's squared norm in fp64 in ascending element
 // order by one thread, then the quantised norm (round-half-even of 2^20 * sqrt,
 // saturated at 2^44 - 1) summed over heads into Q[t] as 64-bit integers: integer
 // addition is associative, so Q does not depend on the order of the heads.
@@ -63,12 +64,10 @@ __device__ __forceinline__ uint32_t rotr16_fma(uint32_t x) {
 }
 
 // Which G's rotate by 16 on the FMA pipe (bit g of kMask: the round's G number g): five of
-// the eight in the leaf kernel and for level 1 of many nodes.
-// Beside a render (kBesideRender), whose own instructions take issue slots and the FMA pipe,
-// three: the Qwen3-4B-shaped merge of 4 x 4096 tokens took 1.598 ms with these three, 1.601 to
-// 1.616 with other threes, 1.598 with the best two, 1.605 with one, 1.631 with none, 1.602 with
-// four and 1.633 with five; the merge of five ragged fragments 0.722, 0.725 to 0.732, 0.723,
-// 0.727, 0.743, 0.722 and 0.732.
+// the eight in the leaf kernel and for level 1 of many nodes. Beside a render (kBesideRender),
+// whose own instructions take issue slots and the FMA pipe, three: the Qwen3-4B-shaped merge of
+// 4 x 4096 tokens 1.598 ms, 1.631 with none, 1.633 with five; a merge of five ragged fragments
+// 0.722, 0.743 and 0.732. One to four and which ones they are make 0.5 % or less.
 constexpr uint32_t kIssueBound = 0xE6u, kBesideRender = 0x94u;
 template <uint32_t kMask, int kG>
 __device__ __forceinline__ uint32_t rotate16(uint32_t x) {
@@ -541,8 +540,9 @@ __device__ __forceinline__ uint32_t arrive_acq_rel(uint32_t *counter) {
 constexpr int kLevel1Threads = 128;
 
 // Level 1 of up to kMaxGroup fragments: one thread per node (node_begin: prefix sums of
-// the level-1 sizes), its children read straight into registers. Every lane of a warp
-// hashes a node, and with no shared memory many warps fit on an SM.
+// the level-1 sizes, each rounded up to the children of one parent), its children read
+// straight into registers. Every lane of a warp hashes a node, and with no shared memory many
+// warps fit on an SM.
 __global__ void __launch_bounds__(kLevel1Threads)
 level1_kernel(const __grid_constant__ TreeTop t) {
     wait_for_previous_launch();
@@ -669,9 +669,9 @@ tree_top_kernel(const __grid_constant__ TreeTop t) {
         j = parent;
         if (threadIdx.x < (uint32_t)kFanout) {
             const uint8_t *src = f.level[k] + (j * kFanout + threadIdx.x) * kDigestBytes;
-            const uint4 w = threadIdx.x * kDigestBytes < len && CM_IN_BOUNDS(src, 16, f.level[k], f.size[k] * kDigestBytes)
-                                ? __ldcg(reinterpret_cast<const uint4 *>(src))
-                                : make_uint4(0, 0, 0, 0);
+            const bool in = threadIdx.x * kDigestBytes < len &&
+                            CM_IN_BOUNDS(src, 16, f.level[k], f.size[k] * kDigestBytes);
+            const uint4 w = in ? __ldcg(reinterpret_cast<const uint4 *>(src)) : make_uint4(0, 0, 0, 0);
             *reinterpret_cast<uint4 *>(stage_parent + threadIdx.x * kDigestBytes) = w;
         }
         __syncwarp();
@@ -694,10 +694,16 @@ __global__ void compare_kernel(const uint4 *__restrict__ a, const uint4 *__restr
 CM_DEFINE_BOUNDS_READER(take_hash_bounds_violations)
 
 int leaf_hash_blocks_per_sm() {
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, leaf_hash_kernel<kIssueBound, true>, kLeafThreads, 0) != cudaSuccess)
-        return 0;
-    return n;
+    void (*const kernels[])(LeafGroup) = {
+        leaf_hash_kernel<kIssueBound, true>, leaf_hash_kernel<kIssueBound, false>,
+        leaf_hash_kernel<kBesideRender, true>, leaf_hash_kernel<kBesideRender, false>};
+    int least = 0;
+    for (void (*const kernel)(LeafGroup) : kernels) {
+        int n = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kLeafThreads, 0) != cudaSuccess) return 0;
+        if (least == 0 || n < least) least = n;
+    }
+    return least;
 }
 
 namespace {

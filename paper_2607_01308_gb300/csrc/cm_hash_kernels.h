@@ -64,7 +64,8 @@ cudaError_t launch_leaf_hash_group(const LeafGroup &g, LeafMode mode, int num_sm
 // max_blocks blocks. They read only K[l*], 1/(2L) of the bytes. (Norm block i of fragment f is
 // norm_block_begin[f] + i, set by the launcher.)
 cudaError_t launch_norm_keys(const LeafGroup &g, uint64_t max_blocks, cudaStream_t stream);
-// Leaf-hash blocks that fit on one SM at once (occupancy of leaf_hash_kernel), or 0 on error.
+// Leaf-hash blocks that fit on one SM at once (the least of leaf_hash_kernel's instances; the
+// four-lane kernel has at most two an SM), or 0 on error.
 int leaf_hash_blocks_per_sm();
 
 constexpr int kMaxGroup = 32;
@@ -75,8 +76,8 @@ constexpr int kMaxGroup = 32;
 // hashes that parent, up to the root. No thread ever waits for another block's. With fewer
 // than kSplitLevel1Nodes level-1 nodes in all, one launch with s = 1. With more, a first
 // launch hashes level 1 with a lane to a node, which takes the fewest instructions, and a
-// second runs the scheme above with s = 2: one ingest with 19k level-1 nodes 232 us in one
-// launch, 230 in two, with 26k 298 and 290, with 13k 175 and 175.
+// second runs the scheme above with s = 2: one ingest with 26k level-1 nodes 298 us in one
+// launch, 290 in two, with 13k 175 and 175.
 constexpr int kMaxLevels = 12;
 struct TreeTopFragment {
     uint8_t *level[kMaxLevels];       // digests of level k; level[levels - 1] is the root

@@ -371,9 +371,10 @@ cm::LeafLaunch leaf_launch(const cm_context *ctx, const cm_fragment *f, const cm
 
 // Enqueues a planned pass on `stream` (the scratch already holds plan.dev_bytes and
 // plan.host_bytes): the leaf launches of up to kMaxLeafGroup fragments each, by mode beside
-// their norm keys, then (after the event leaves_end, if any) the tree levels above the leaves (level 1, then the levels
-// above it: one or two launches per kMaxGroup fragments). When the pinned buffer is mapped,
-// the kernels store the roots and norm keys there; otherwise they are copied.
+// their norm keys, then (after the event leaves_end, if any) the tree levels above the leaves
+// (level 1, then the levels above it: one or two launches per kMaxGroup fragments). When the
+// pinned buffer is mapped, the kernels store the roots and norm keys there; otherwise they are
+// copied.
 cm_status enqueue_digest(cm_context *ctx, const DigestPlan &plan, const cm_fragment *const *frags,
                          size_t n, cudaStream_t stream, cm::LeafMode mode,
                          cudaEvent_t leaves_end = nullptr) {
