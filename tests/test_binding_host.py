@@ -15,7 +15,8 @@ def binding():
 
 @pytest.mark.parametrize("form", [bytes, bytearray, memoryview, list, tuple,
                                   lambda b: array.array("I", list(b)), lambda b: memoryview(array.array("H", list(b))),
-                                  lambda b: np.frombuffer(b, dtype=np.uint8), lambda b: np.array(list(b), dtype=np.int64),
+                                  lambda b: np.frombuffer(b, dtype=np.uint8),
+                                  lambda b: np.array(list(b), dtype=np.int64),
                                   lambda b: [x - 256 for x in b]])
 def test_an_id_is_its_sixteen_entries_whatever_their_type(binding, form):
     arr = binding._id_array([form(ID), ID])
