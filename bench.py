@@ -42,14 +42,12 @@ BASE_SEED_REDELIVER = 42 + 997   # delivery order of the re-delivery sweep
 NOMINAL_HBM_GBS = 8000.0
 FALLBACK_HBM_GBS = 6800.0
 # Integer-ALU roofline of the content-address kernel: a BLAKE2s block (64 bytes) has
-# 10 rounds x 8 G x (4 xors + 4 rotates) + 8 xors = 648 xors and rotations. Five of a round's
-# rotations by 16 (three when a render runs beside the hash) are dot products on the FMA
-# pipe, as G's additions are multiply-adds there, so 598 (618) issue on the integer ALU pipe;
-# the pipe takes 16 lanes per SMSP per clock (4 SMSPs -> 64 ops/clk/SM), so the peak is
-# 152 SMs x 64 x the maximum SM clock.
+# 10 rounds x 8 G x (4 xors + 4 rotates) + 8 xors = 648 xors and rotations. Three of a round's
+# rotations by 16 are dot products on the FMA pipe, as G's additions are multiply-adds there, so
+# 618 issue on the integer ALU pipe; the pipe takes 16 lanes per SMSP per clock (4 SMSPs -> 64
+# ops/clk/SM), so the peak is 152 SMs x 64 x the maximum SM clock.
 HASH_XOR_ROT_PER_BYTE = 648.0 / 64.0
-HASH_ALU_OPS_PER_BYTE = 598.0 / 64.0
-HASH_ALU_OPS_PER_BYTE_BESIDE = 618.0 / 64.0
+HASH_ALU_OPS_PER_BYTE = 618.0 / 64.0
 ALU_OPS_PER_CLK_PER_SM = 64
 CLOCK_FIELDS = ("index,clocks.sm,clocks.max.sm,power.draw,clocks_event_reasons.active,"
                 "clocks_event_reasons.hw_slowdown,clocks_event_reasons.hw_thermal_slowdown,"
@@ -1200,9 +1198,8 @@ def main():
         # 4-warp render of the same merge beside it on the other stream
         hash_in_step = dict(hash_roof)
         hash_in_step.update({
-            "algorithmic_ops_per_launch": HASH_ALU_OPS_PER_BYTE_BESIDE * frag_bytes,
-            "achieved": HASH_ALU_OPS_PER_BYTE_BESIDE * frag_bytes / (leaf_ms_ovl * 1e-3) / 1e12,
-            "frac": HASH_ALU_OPS_PER_BYTE_BESIDE * frag_bytes / (leaf_ms_ovl * 1e-3) / 1e12 / alu_peak,
+            "achieved": HASH_ALU_OPS_PER_BYTE * frag_bytes / (leaf_ms_ovl * 1e-3) / 1e12,
+            "frac": HASH_ALU_OPS_PER_BYTE * frag_bytes / (leaf_ms_ovl * 1e-3) / 1e12 / alu_peak,
             "ms_per_launch": leaf_ms_ovl,
             "hash_gbs": frag_bytes / (leaf_ms_ovl * 1e-3) / 1e9,
             "frac_all_int_ops_of_128_lanes":

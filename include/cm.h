@@ -422,7 +422,7 @@ cm_status cm_context_kernel_times(cm_context *ctx, cm_kernel_times *out, int32_t
  * counterpart): chains of three-input xors (one integer-ALU instruction each), and the
  * BLAKE2s compression function of the content address applied to register data, counted
  * as the 648 xors and rotations of a 64-byte block (10 rounds x 8 G x (4 xors + 4
- * rotations) + 8 xors; G's additions and 50 of the rotations run on the FMA pipe). Both are
+ * rotations) + 8 xors; G's additions and 30 of the rotations run on the FMA pipe). Both are
  * reported in 10^12 operations per second, best of three timed launches of four full
  * waves each. Synchronous; allocates and frees a small device buffer; takes a few ms.
  * The calling thread's current device is restored on return. */

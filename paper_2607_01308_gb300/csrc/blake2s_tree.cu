@@ -44,11 +44,13 @@ __device__ __forceinline__ uint32_t rotr7(uint32_t x) { return __funnelshift_r(x
 //
 // The rotation by 16 can move as well: x * 2^16 is its upper half, and a two-way 16-bit dot
 // product with (0, 1) adds its lower half: two multiply-type instructions for one byte
-// permutation. Moving it in t of the 8 G's of a round leaves (8 - t/8) x 2 ALU cycles,
-// (6 + t/4) x 2 FMA cycles and 14 + t/8 issue cycles per G, balanced at t = 5. Measured over
-// 52 choices of the G's on 2.4 GB of leaves: 1.06 times the best with t = 0, 1.02 with 3, 1.00 to
-// 1.02 with 5 or 6, 1.04 with 8; the choice below 1.259 ms (1.310 with the earlier order of
-// additions and no rotation moved). ALU 92 %, FMA 89 % and issue 91 % busy.
+// permutation. Moved in three of a round's eight G's it leaves a block 630 ALU, 542 FMA and 1186
+// instructions in all (656, 485 and 1155 with none; counted on 604 MB of leaves): ALU 95 %, the
+// multiplying half of the FMA pipe 81 % and issue 90 % busy. Moved further (five or all eight)
+// the ALU count stays, since the compiler gives other additions back to that pipe, and only the
+// instructions grow (1207, 1237): 2.4 GB of leaves and their norm keys 1.317 ms with none, 1.261
+// with three, 1.265 with five, 1.262 with eight; beside a render, which takes issue slots too, the
+// Qwen3-4B-shaped merge of 4 x 4096 tokens 1.631, 1.598 and (five) 1.633.
 __constant__ uint32_t g_one = 1, g_64k = 65536, g_upper_half = 0x0100;
 __device__ __forceinline__ uint32_t mad1(uint32_t x, uint32_t y) {
     uint32_t r;
@@ -63,22 +65,19 @@ __device__ __forceinline__ uint32_t rotr16_fma(uint32_t x) {
     return r;
 }
 
-// Which G's rotate by 16 on the FMA pipe (bit g of kMask: the round's G number g): five of
-// the eight in the leaf kernel and for level 1 of many nodes. Beside a render (kBesideRender),
-// whose own instructions take issue slots and the FMA pipe, three: the Qwen3-4B-shaped merge of
-// 4 x 4096 tokens 1.598 ms, 1.631 with none, 1.633 with five; a merge of five ragged fragments
-// 0.722, 0.743 and 0.732. One to four and which ones they are make 0.5 % or less.
-constexpr uint32_t kIssueBound = 0xE6u, kBesideRender = 0x94u;
-template <uint32_t kMask, int kG>
+// Which G's rotate by 16 on the FMA pipe (bit g: the round's G number g). Which three they are
+// makes half a per cent or less.
+constexpr uint32_t kFmaMask = 0x94u;
+template <int kG>
 __device__ __forceinline__ uint32_t rotate16(uint32_t x) {
-    return (kMask >> kG) & 1u ? rotr16_fma(x) : rotr16(x);
+    return (kFmaMask >> kG) & 1u ? rotr16_fma(x) : rotr16(x);
 }
 
 // The G mixing function of RFC 7693, Section 3.1 (rotation distances 16, 12, 8, 7); g is
 // G's place in its round.
 #define CM_G(g, a, b, c, d, x, y)   \
     a = add3(a, b, (x));            \
-    d = rotate16<kFmaMask, g>(d ^ a);     \
+    d = rotate16<g>(d ^ a);         \
     c = c + d;                      \
     b = rotr12(b ^ c);              \
     a = add3(a, b, (y));            \
@@ -101,7 +100,6 @@ __device__ __forceinline__ uint32_t rotate16(uint32_t x) {
 // Compression function F (RFC 7693, Section 3.2), 10 rounds. t = bytes hashed
 // so far including this block; the last-node flag is applied together with the
 // last-block flag, on the node's final compression.
-template <uint32_t kFmaMask>
 __device__ __forceinline__ void compress(uint32_t h[8], const uint32_t m[16], uint64_t t,
                                          bool last_block, bool last_node) {
     uint32_t v0 = h[0], v1 = h[1], v2 = h[2], v3 = h[3];
@@ -402,7 +400,7 @@ __device__ __forceinline__ void zero_arrivals(const LeafLaunch &a) {
 // short (a multiple of 64 bytes, as 2 L planes are): every leaf then walks its blocks in
 // halves of 32 bytes, one loop for all, so that a warp never hashes its straddling leaves
 // after the others (as it once did: the tiny merge's leaves took 42 us, now 21).
-template <uint32_t kFmaMask, bool kWhole>
+template <bool kWhole>
 __global__ void __launch_bounds__(kLeafThreads)
 leaf_hash_kernel(const __grid_constant__ LeafGroup grp) {
     // the blocks after the leaf blocks, one per fragment (done by the leaf threads this cost
@@ -432,7 +430,7 @@ leaf_hash_kernel(const __grid_constant__ LeafGroup grp) {
                         w3 = load_nc(p + at + 48);
             const uint32_t m[16] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w,
                                     w2.x, w2.y, w2.z, w2.w, w3.x, w3.y, w3.z, w3.w};
-            compress<kFmaMask>(h, m, at + 64, at + 64 == (uint32_t)kLeafBytes, last_node);
+            compress(h, m, at + 64, at + 64 == (uint32_t)kLeafBytes, last_node);
         }
     } else {
         const uint64_t rem = a.stream_bytes - begin;
@@ -444,7 +442,7 @@ leaf_hash_kernel(const __grid_constant__ LeafGroup grp) {
             const uint4 w0 = load_nc(p), w1 = load_nc(p + 16), w2 = load_nc(q), w3 = load_nc(q + 16);
             const uint32_t m[16] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w,
                                     w2.x, w2.y, w2.z, w2.w, w3.x, w3.y, w3.z, w3.w};
-            compress<kFmaMask>(h, m, (b + 1) * 64, b + 1 == nblocks, last_node);
+            compress(h, m, (b + 1) * 64, b + 1 == nblocks, last_node);
         }
     }
     if (CM_IN_BOUNDS(a.digests + leaf * kDigestBytes, kDigestBytes, a.digests,
@@ -572,7 +570,7 @@ level1_kernel(const __grid_constant__ TreeTop t) {
         const uint32_t m[16] = {w[0].x, w[0].y, w[0].z, w[0].w, w[1].x, w[1].y, w[1].z, w[1].w,
                                 w[2].x, w[2].y, w[2].z, w[2].w, w[3].x, w[3].y, w[3].z, w[3].w};
         const uint32_t end = (b + 1) * 64 < len ? (b + 1) * 64 : len;
-        compress<kIssueBound>(h, m, end, b + 1 == nblocks, last_node);
+        compress(h, m, end, b + 1 == nblocks, last_node);
     }
     if (CM_IN_BOUNDS(f.level[1] + j * kDigestBytes, kDigestBytes, f.level[1], f.size[1] * kDigestBytes))
         store_digest(f.level[1] + j * kDigestBytes, h);
@@ -694,9 +692,7 @@ __global__ void compare_kernel(const uint4 *__restrict__ a, const uint4 *__restr
 CM_DEFINE_BOUNDS_READER(take_hash_bounds_violations)
 
 int leaf_hash_blocks_per_sm() {
-    void (*const kernels[])(LeafGroup) = {
-        leaf_hash_kernel<kIssueBound, true>, leaf_hash_kernel<kIssueBound, false>,
-        leaf_hash_kernel<kBesideRender, true>, leaf_hash_kernel<kBesideRender, false>};
+    void (*const kernels[])(LeafGroup) = {leaf_hash_kernel<true>, leaf_hash_kernel<false>};
     int least = 0;
     for (void (*const kernel)(LeafGroup) : kernels) {
         int n = 0;
@@ -729,7 +725,7 @@ cudaError_t launch_after(void (*kernel)(P), uint64_t blocks, int threads, cudaSt
 
 }  // namespace
 
-cudaError_t launch_leaf_hash_group(const LeafGroup &g, LeafMode mode, int num_sms, cudaStream_t stream) {
+cudaError_t launch_leaf_hash_group(const LeafGroup &g, bool with_norms, int num_sms, cudaStream_t stream) {
     if (g.count > (uint32_t)kMaxLeafGroup) return cudaErrorInvalidValue;
     if (g.count == 0) return cudaSuccess;
     // four lanes to a leaf up to half a leaf block per SM (two such warps per scheduler; beyond,
@@ -740,17 +736,15 @@ cudaError_t launch_leaf_hash_group(const LeafGroup &g, LeafMode mode, int num_sm
     if (blocks > 0x7FFFFFFFull) return cudaErrorInvalidValue;
     bool whole = true;
     for (uint32_t i = 0; i < g.count; ++i) whole = whole && g.frag[i].plane_bytes % kLeafBytes == 0;
-    void (*const alone)(LeafGroup) = few     ? leaf_quad_kernel
-                                     : whole ? leaf_hash_kernel<kIssueBound, true>
-                                             : leaf_hash_kernel<kIssueBound, false>;
-    if (mode != LeafMode::kWithNorms) {
-        void (*const beside)(LeafGroup) =
-            whole ? leaf_hash_kernel<kBesideRender, true> : leaf_hash_kernel<kBesideRender, false>;
-        (mode == LeafMode::kBesideRender && !few ? beside : alone)<<<(unsigned)blocks, kLeafThreads, 0, stream>>>(g);
+    void (*const kernel)(LeafGroup) = few     ? leaf_quad_kernel
+                                      : whole ? leaf_hash_kernel<true>
+                                              : leaf_hash_kernel<false>;
+    if (!with_norms) {
+        kernel<<<(unsigned)blocks, kLeafThreads, 0, stream>>>(g);
         return cudaGetLastError();
     }
     const cudaError_t e = launch_norm_keys(g, (uint64_t)num_sms, stream);
-    return e != cudaSuccess ? e : launch_after(alone, blocks, kLeafThreads, stream, g);
+    return e != cudaSuccess ? e : launch_after(kernel, blocks, kLeafThreads, stream, g);
 }
 
 cudaError_t launch_norm_keys(const LeafGroup &in, uint64_t max_blocks, cudaStream_t stream) {
@@ -921,7 +915,7 @@ extern "C" cm_status cm_fragment_id_static(const cm_fragment *frag, int32_t rout
         int device = 0, num_sms = 0;
         e = cudaGetDevice(&device);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, device);
-        if (e == cudaSuccess) e = launch_leaf_hash_group(g, LeafMode::kWithNorms, num_sms, cs);
+        if (e == cudaSuccess) e = launch_leaf_hash_group(g, true, num_sms, cs);
         if (e != cudaSuccess) return report_error(CM_ERR_CUDA, cudaGetErrorString(e));
         TreeTop top;
         std::memset(&top, 0, sizeof top);
@@ -982,7 +976,7 @@ compress_probe_kernel(uint32_t *out, int blocks) {
 #pragma unroll
     for (int i = 0; i < 16; ++i) m[i] = tid ^ ((uint32_t)i * 0x9E3779B9u);
     for (int b = 0; b < blocks; ++b) {
-        compress<kIssueBound>(h, m, (uint64_t)(b + 1) * 64, false, false);
+        compress(h, m, (uint64_t)(b + 1) * 64, false, false);
         m[0] ^= h[0];
         m[7] ^= h[3];
         m[11] ^= h[6];

@@ -55,11 +55,9 @@ struct LeafGroup {
     uint64_t norm_block_begin[kMaxLeafGroup + 1];
     LeafLaunch frag[kMaxLeafGroup];
 };
-// kWithNorms: the group's norm keys too, in a launch of their own beside the leaves. Otherwise
-// they are launched elsewhere (launch_norm_keys); a render runs beside the leaves
-// (kBesideRender) or not (kAlone), a scheduling choice: the digests are the same.
-enum class LeafMode { kWithNorms, kAlone, kBesideRender };
-cudaError_t launch_leaf_hash_group(const LeafGroup &g, LeafMode mode, int num_sms, cudaStream_t stream);
+// with_norms: the group's norm keys too, in a launch of their own beside the leaves. Otherwise
+// they are launched elsewhere (launch_norm_keys).
+cudaError_t launch_leaf_hash_group(const LeafGroup &g, bool with_norms, int num_sms, cudaStream_t stream);
 // The routing-layer norm keys of the group, norm_lanes(H) threads to a token, by at most
 // max_blocks blocks. They read only K[l*], 1/(2L) of the bytes. (Norm block i of fragment f is
 // norm_block_begin[f] + i, set by the launcher.)

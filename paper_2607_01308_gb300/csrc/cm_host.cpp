@@ -370,15 +370,14 @@ cm::LeafLaunch leaf_launch(const cm_context *ctx, const cm_fragment *f, const cm
 }
 
 // Enqueues a planned pass on `stream` (the scratch already holds plan.dev_bytes and
-// plan.host_bytes): the leaf launches of up to kMaxLeafGroup fragments each, by mode beside
+// plan.host_bytes): the leaf launches of up to kMaxLeafGroup fragments each, with_norms beside
 // their norm keys, then (after the event leaves_end, if any) the tree levels above the leaves
 // (level 1, then the levels above it: one or two launches per kMaxGroup fragments). When the
 // pinned buffer is mapped, the kernels store the roots and norm keys there; otherwise they are
 // copied.
 cm_status enqueue_digest(cm_context *ctx, const DigestPlan &plan, const cm_fragment *const *frags,
-                         size_t n, cudaStream_t stream, cm::LeafMode mode,
+                         size_t n, cudaStream_t stream, bool with_norms,
                          cudaEvent_t leaves_end = nullptr) {
-    const bool with_norms = mode == cm::LeafMode::kWithNorms;
     uint8_t *base = ctx->d_scratch;
     uint8_t *results = ctx->h_pinned_dev ? static_cast<uint8_t *>(ctx->h_pinned_dev) : base;
     std::unique_ptr<cm::LeafGroup> grp(new cm::LeafGroup);
@@ -400,7 +399,7 @@ cm_status enqueue_digest(cm_context *ctx, const DigestPlan &plan, const cm_fragm
         if (grp->block_begin[gn] > 0x7FFFFFFFull)
             return fail(CM_ERR_UNSUPPORTED, "leaf-hash launch exceeds 2^31 - 1 blocks");
         CM_CUDA_TRY(timed_launch(ctx, kTimeLeaf, stream,
-                                 [&] { return cm::launch_leaf_hash_group(*grp, mode, ctx->num_sms, stream); }),
+                                 [&] { return cm::launch_leaf_hash_group(*grp, with_norms, ctx->num_sms, stream); }),
                     "leaf hash launch");
         if (ctx->timing) ctx->leaf_fragments += (int64_t)gn;
         if (ctx->timing && with_norms) ++ctx->aux_launches;
@@ -461,7 +460,7 @@ cm_status fragments_digest(cm_context *ctx, const cm_fragment *const *frags, siz
     DigestPlan plan;
     cm_status st = plan_digest(ctx, frags, n, plan);
     if (st == CM_OK) st = ensure_scratch(ctx, plan.dev_bytes, plan.host_bytes);
-    if (st == CM_OK) st = enqueue_digest(ctx, plan, frags, n, stream, cm::LeafMode::kWithNorms);
+    if (st == CM_OK) st = enqueue_digest(ctx, plan, frags, n, stream, true);
     if (st != CM_OK) return st;
     CM_CUDA_TRY(cudaStreamSynchronize(stream), "ingest synchronisation");
     collect_digest(ctx, plan, frags, n, ids, Qs);
@@ -1029,7 +1028,7 @@ cm_status compare_and_digest(cm_context *ctx, const std::vector<const cm_fragmen
     SideJoin side_join{ctx, cs};
     if (!chosen.empty()) st = enqueue_comparisons(ctx, fp, chosen, ctx->side, hash.empty() ? 6 : 2, dev_off, host_off);
     if (st == CM_OK && !hash.empty())
-        st = enqueue_digest(ctx, plan, hash.data(), hash.size(), cs, cm::LeafMode::kWithNorms);
+        st = enqueue_digest(ctx, plan, hash.data(), hash.size(), cs, true);
     const cudaError_t e = side_join.run();
     if (st == CM_OK && e != cudaSuccess) st = cuda_fail(e, "side stream ordering");
     if (st != CM_OK) return st;
@@ -1611,10 +1610,7 @@ cm_status ingest_render_impl(cm_set *const *sets, const cm_fragment *frags, int3
     const bool may_wait = !partial_wave && !large(least_tokens);   // for the leaves to end
     const bool digest_first = partial_wave || !large(most_tokens);
     auto digest = [&]() -> cm_status {
-        return enqueue_digest(ctx, plan, fp.data(), fp.size(), cs,
-                              partial_wave || large(most_tokens) ? cm::LeafMode::kBesideRender
-                                                                 : cm::LeafMode::kAlone,
-                              may_wait ? ctx->leaves_end : nullptr);
+        return enqueue_digest(ctx, plan, fp.data(), fp.size(), cs, false, may_wait ? ctx->leaves_end : nullptr);
     };
     if (digest_first) {
         st = digest();
