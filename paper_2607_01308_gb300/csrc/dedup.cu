@@ -16,7 +16,8 @@ constexpr uint32_t kPieces = 16, kPieceVecs = 16;       // of the first look: 25
 static_assert(kPieces * kPieceVecs == (uint32_t)kThreads, "a thread compares one vector of a piece");
 constexpr uint64_t kChunkVecs = kCompareChunkVecs;      // 32 KiB of each array per chunk
 constexpr int kStepVecs = 4;                            // vectors per thread at a time
-static_assert(kChunkVecs % ((uint64_t)kThreads * kStepVecs) == 0, "a chunk is a number of whole steps");
+constexpr uint64_t kStep = (uint64_t)kThreads * kStepVecs;
+static_assert(kChunkVecs % kStep == 0, "a chunk is a number of whole steps");
 static_assert(sizeof(CompareFull) <= 32764, "comparison parameters exceed the kernel parameter limit");
 
 __device__ __forceinline__ uint32_t diff4(const uint4 &x, const uint4 &y) {
@@ -49,8 +50,9 @@ __global__ void __launch_bounds__(kThreads) look_kernel(const __grid_constant__ 
 // (bound by HBM: (members + 1) reads instead of 2 per member). What other warps have found to
 // differ is learnt once per chunk, a lane to a member; such a member is read only where the next
 // of its chain is compared with it, and a group whose members all differ is left. Beside the
-// hash, which is bound by issue slots, instructions and registers count: on six copies alone 8
-// vectors a step took 152 us, 4 185, but a merge of nine deliveries hashed beside it 420 and 369.
+// hash, which is bound by issue slots, instructions and registers count: six copies alone take
+// 152 us at 8 vectors a step, 185 at 4, but a merge of nine deliveries hashed beside it 420 and
+// 367; with a test per vector (29 instead of 23 M instructions) 373.
 __global__ void __launch_bounds__(kThreads) full_kernel(const __grid_constant__ CompareFull c) {
     const uint64_t total = c.chunk_begin[c.groups];
     const uint32_t lane = threadIdx.x % 32;
@@ -75,15 +77,22 @@ __global__ void __launch_bounds__(kThreads) full_kernel(const __grid_constant__ 
         const uint32_t is_v = local >= per_array;
         const uint64_t begin = (is_v ? local - per_array : local) * kChunkVecs;
         const uint64_t end = begin + kChunkVecs < g.vecs ? begin + kChunkVecs : g.vecs;
+        const bool whole = g.vecs >= kStep;
 #pragma unroll 1
-        for (uint64_t at = begin; at < end; at += (uint64_t)kThreads * kStepVecs) {
-            const uint64_t i = at + threadIdx.x;
-            const bool whole = at + (uint64_t)kThreads * kStepVecs <= end;
+        for (uint64_t at = begin; at < end; at += kStep) {
+            // an array's last step begins early enough to be a whole one, so that none but an
+            // array shorter than a step needs a test per vector
+            const uint64_t i = (whole && at + kStep > g.vecs ? g.vecs - kStep : at) + threadIdx.x;
             auto load = [&](const uint4 *p, uint64_t vecs, uint4 (&r)[kStepVecs]) {
+                if (whole) {
 #pragma unroll
-                for (int u = 0; u < kStepVecs; ++u)
-                    r[u] = whole || i + (uint64_t)u * kThreads < end ? load_vec(p, i + (uint64_t)u * kThreads, vecs)
-                                                                     : make_uint4(0, 0, 0, 0);
+                    for (int u = 0; u < kStepVecs; ++u) r[u] = load_vec(p, i + (uint64_t)u * kThreads, vecs);
+                } else {
+#pragma unroll
+                    for (int u = 0; u < kStepVecs; ++u)
+                        r[u] = i + (uint64_t)u * kThreads < vecs ? load_vec(p, i + (uint64_t)u * kThreads, vecs)
+                                                                 : make_uint4(0, 0, 0, 0);
+                }
             };
             uint4 b[kStepVecs], a[kStepVecs];
             if (read_base) load(g.kv[is_v], g.vecs, b);
