@@ -1,6 +1,6 @@
 """Builds libcm.so in-tree (next to this file) for sm_103a with nvcc and g++.
 
-Three translation units compiled in parallel, then one shared-library link:
+Five translation units compiled in parallel, then one shared-library link:
   csrc/cm_host.cpp       host core (g++, C++17, no floating-point contraction)
   csrc/blake2s_tree.cu   content-address kernels (nvcc, sm_103a)
   csrc/render.cu         render kernel (nvcc, sm_103a)
